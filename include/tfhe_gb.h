@@ -307,15 +307,11 @@ typedef enum {
     TFHE_OPT_PROFILE = 2,    /* 1: record CUDA events around every blind-rotation   */
                              /*    and key-switch launch of circuit schedules (also */
                              /*    inside captured graphs)                          */
-    TFHE_OPT_BR_GROUP = 3,   /* blind-rotation CTA shape: 1, 2 or 4 bootstraps per  */
-                             /*    CTA (4 warps each), 5 = one per 4-warp CTA at 5  */
-                             /*    CTAs per SM, 8 = one bootstrap on 8 warps,       */
-                             /*    16 = one bootstrap on a cluster of two CTAs (two */
-                             /*    SMs, one prime each; lowest latency), 32 = two   */
-                             /*    bootstraps per CTA with each CMux step's key     */
-                             /*    staged in shared memory by bulk copies (one CTA  */
-                             /*    per SM), 33 = the same shape and occupancy with  */
-                             /*    the key read through L1 (the staging's control), */
+    TFHE_OPT_BR_GROUP = 3,   /* blind-rotation shape: 1 = four bootstraps per CTA   */
+                             /*    (4 warps each), one CTA per SM (2, 4, 5, 32 and  */
+                             /*    33 are accepted and run it too), 8 = one         */
+                             /*    bootstrap on 8 warps, 16 = one bootstrap on a    */
+                             /*    cluster of two CTAs (two SMs, one prime each),   */
                              /*    40 = one bootstrap on 8 warps with the key       */
                              /*    staged, 48 = the two-CTA cluster with each CTA's */
                              /*    half of the key staged, or 0 (default):          */
@@ -347,10 +343,9 @@ int tfhe_ctx_set_option(tfhe_ctx *ctx, int option, int64_t value);
  * context's device: for each level-width bucket (<= 152, 304, 608, 1216,
  * 2432, 4864, 9728 gates, and more) time the blind-rotation CTA shapes
  * (TFHE_OPT_BR_GROUP values) and the key-switch kernels (TFHE_OPT_KS_KERNEL
- * values) on synthetic ciphertexts, and keep the fastest; then time one
- * full wave of 4 bootstraps per SM and one of 5 per SM, from which each
- * circuit schedule picks its wave size (a few seconds; results never
- * change).  cache_path (may be NULL): a text file consulted
+ * values) on synthetic ciphertexts, and keep the fastest; each
+ * circuit schedule picks its level unit from the measured times (a few
+ * seconds; results never change).  cache_path (may be NULL): a text file consulted
  * first and appended to after tuning, keyed by device name and SM count.
  * choices (may be NULL) receives 16 ints: the 8 blind-rotation shapes, then
  * the 8 key-switch choices.  Synchronous. */

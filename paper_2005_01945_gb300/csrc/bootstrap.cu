@@ -12,32 +12,26 @@
 // GB300 design (not the paper's: it used cuFFT in floating point):
 //  * the products are exact: a negacyclic NTT modulo two primes below 2^27
 //    and a centred CRT lift back to Z/2^32;
-//  * one group of 4 warps owns one bootstrap; a CTA runs B in {1, 2, 4}
-//    bootstraps in lockstep (4B warps) and loops over gate groups
+//  * 4 warps own one bootstrap; a CTA of 16 warps per SM runs four that
+//    share constants and otherwise run independently, looping over gates
 //    (persistent grid); the accumulators never leave shared memory.  For
 //    narrow levels one bootstrap can instead take 8 warps, or a cluster of
 //    two CTAs (one prime each), and the key of the next CMux step can be
 //    staged in shared memory by bulk copies;
-//  * warp (c, h) of a bootstrap works modulo prime h for the whole CMux:
-//    it forms both digit polynomials of TLWE polynomial c (one rotation)
-//    and transforms them; then, as warp (p, h), it does the pointwise
-//    products with BK_i for output polynomial p, the inverse transform and
-//    half of the CRT + accumulate;
+//  * the first pass of the forward transforms, on digits of 10 bits, is an
+//    exact fp16 matrix product on the tensor pipe (k_blind_rotate_tc);
 //  * one 1024-point transform is one warp: 32 coefficients per lane,
 //    a 32-point transform in registers, a twiddle, one shared-memory
 //    transpose, and a second 32-point transform (four-step NTT);
-//  * code size is the binding constraint on instruction fetch: each
-//    transform exists once (the prime is a runtime value), and the warps of
-//    a CTA execute the same phase at the same time;
 //  * the bootstrapping key is pre-transformed, scaled by 2^32 N^-1 and
 //    interleaved so that lane l reads its 4 rows for one register as one
-//    16-byte load; the 33 MB key stays L2-resident across gates, and the B
-//    bootstraps of a CTA read each key row once through L1.
+//    16-byte load; the 33 MB key stays L2-resident across gates.
 #include <cstdio>
 #include <cstring>
 #include <vector>
 
 #include <cooperative_groups.h>
+#include <cuda_fp16.h>
 
 #include "common.cuh"
 
@@ -545,42 +539,6 @@ __device__ __forceinline__ void bk_issue(BkStage &G, const uint4 *bk_ntt, int i,
     G.issued[buf]++;
 }
 
-// Phase 1: warp (c, h) forms both digit polynomials of TLWE polynomial c of
-// X^a acc - acc (one rotation, two digit extractions) and transforms them
-// modulo prime h; results go to S.fwd[2c + j][h].  One transform copy: the
-// two digits are a rolled loop.
-__device__ __forceinline__ void br_digits_fwd(uint32_t (&x)[32], BrSmem &S, int c, int a,
-                                              int lane, const uint2 *__restrict__ twb,
-                                              const Prime &pr)
-{
-    const uint32_t *ac = S.acc[c];
-    uint32_t *s0 = S.fwd[2 * c][pr.P], *s1 = S.fwd[2 * c + 1][pr.P];
-#pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        const int k = lane + 32 * r;
-        const int idx = (k - a) & (2 * kN - 1);
-        uint32_t v = ac[idx & (kN - 1)];
-        v = idx >= kN ? 0u - v : v;
-        const uint32_t u = v - ac[k] + kDecompOffset;
-        x[r] = ((u >> 22) & 1023u) + (pr.q - 512u);            // level-0 digit + q
-        s1[r * 32 + lane] = ((u >> 12) & 1023u) + (pr.q - 512u);  // level-1 digit, parked
-    }
-#pragma unroll 1
-    for (int j = 0; j < 2; ++j) {
-        uint32_t *sj = j ? s1 : s0;
-        if (j) {
-#pragma unroll
-            for (int r = 0; r < 32; ++r)
-                x[r] = s1[r * 32 + lane];
-            __syncwarp();
-        }
-        fwd_ntt(x, sj, lane, twb, pr);
-#pragma unroll
-        for (int r = 0; r < 32; ++r)
-            sj[r * 32 + lane] = x[r];
-    }
-}
-
 // Phase 1 with eight warps per bootstrap: warp (c, j, h) forms digit
 // polynomial j of TLWE polynomial c of X^a acc - acc and transforms it
 // modulo prime h into S.fwd[2c + j][h] (its own slot, also the transpose
@@ -615,6 +573,25 @@ __device__ __forceinline__ void br_digit_fwd(uint32_t (&x)[32], BrSmem &S, int c
 // Phase 2: pointwise products for output polynomial p modulo prime h,
 // summed over the 4 digit rows; result in [0, 2q).  Registers R0 .. R0 +
 // NR - 1 (all 32 unless two warps share the polynomial).
+template <int R0 = 0, int NR = 32>
+__device__ __forceinline__ void br_pointwise(uint32_t (&x)[32], const uint32_t (*f)[kSlot],
+                                             const uint4 *__restrict__ bkp, int lane,
+                                             const Prime &pr)
+{
+    const uint32_t qn = c_ntt.q_inv[pr.P];
+    const uint32_t *f0 = f[0], *f1 = f[1], *f2 = f[2], *f3 = f[3];
+#pragma unroll
+    for (int r = R0; r < R0 + NR; ++r) {
+        const uint4 b = __ldg(bkp + r * 32 + lane);
+        const int e = r * 32 + lane;
+        uint64_t s = (uint64_t)f0[e] * b.x;
+        s += (uint64_t)f1[e] * b.y;
+        s += (uint64_t)f2[e] * b.z;
+        s += (uint64_t)f3[e] * b.w;
+        x[r] = mont_reduce(s, pr.q, qn);
+    }
+}
+
 template <int R0 = 0, int NR = 32>
 __device__ __forceinline__ void br_pointwise(uint32_t (&x)[32], const BrSmem &S,
                                              const uint4 *__restrict__ bkp, int lane,
@@ -658,19 +635,6 @@ __device__ __forceinline__ void br_pointwise_staged(uint32_t (&x)[32], const BrS
         s += (uint64_t)f3[e] * b.w;
         x[r] = mont_reduce(s, pr.q, qn);
     }
-}
-
-// Phase 3: inverse transform, reduce to [0, q), publish all residues for
-// the CRT (this warp's exchange slot).
-__device__ __forceinline__ void br_inverse(uint32_t (&x)[32], BrSmem &S, int w4, int lane,
-                                           int lane_brv, const uint2 *__restrict__ twb,
-                                           const Prime &pr)
-{
-    inv_ntt(x, S.fwd[w4][0], lane, lane_brv, twb, pr);
-    uint32_t *xch = S.fwd[w4][1];
-#pragma unroll
-    for (int r = 0; r < 32; ++r)
-        xch[r * 32 + lane] = csub(x[r], pr.q);
 }
 
 // Phases 2 and 3 of the 8-warp shapes: warp K of the pair (w4, w4 + 4)
@@ -717,12 +681,6 @@ __device__ __forceinline__ void crt_rows(uint32_t *acc, const uint32_t *x0, cons
         const uint32_t u = csub(mul_shoup(v1 - v0 + 2 * kQ1, c, cp, kQ1), kQ1);
         acc[e] += v0 + kQ0 * u - (u > uh ? plo : 0u);
     }
-}
-
-template <int NR>
-__device__ __forceinline__ void br_crt(BrSmem &S, int p, int r0, int lane)
-{
-    crt_rows<NR>(S.acc[p], S.fwd[p * 2 + 0][1], S.fwd[p * 2 + 1][1], r0, lane);
 }
 
 // Linear part of gate `op`: c = mu + aa ca + ab cb + ac cc.  Returns false
@@ -834,17 +792,13 @@ __device__ __forceinline__ void br_extract(const BrArgs &A, long g, const uint32
         bg[kN] = (int32_t)acc[1][0];
 }
 
-// B bootstraps per CTA, W warps each (W = 4: B in {1, 2, 4} in lockstep;
-// W = 8: B = 1, the phases spread over twice the warps for lower latency on
-// narrow levels); 128 registers per thread, 16 warps/SM.
-//   W = 4: warp (p, h) runs phase 1 as (c = p, both digits), phases 2-3 as
-//          output polynomial p modulo prime h, phase 4 on half of p.
-//   W = 8: warp (c, j, h) runs phase 1 for digit j of polynomial c; warps
-//          0..3 run phases 2-3 as (p, h); every warp runs phase 4 on a
-//          quarter of polynomial w >> 2.
-template <int B, int W, int STAGE = 0, int MINB = 0>
+// One bootstrap per CTA on W = 8 warps (one CTA per SM), for levels narrower
+// than the GPU: warp (c, j, h) runs phase 1 for digit j of polynomial c;
+// warps w and w + 4 share phases 2-3 of (p, h); every warp runs phase 4 on a
+// quarter of polynomial w >> 2.
+template <int B, int W, int STAGE>
 __global__ void __launch_bounds__(32 * W * B,
-                                  MINB ? MINB : ((W * B >= 16 || W == 8) ? 1 : 16 / (W * B)))
+                                  1)
     k_blind_rotate(const BrArgs A)
 {
     constexpr int T = 32 * W;      // threads per bootstrap
@@ -911,53 +865,31 @@ __global__ void __launch_bounds__(32 * W * B,
             const int a = S.abar[i];  // a = 0 here gives zero digits: acc unchanged
             uint32_t x[32];
             const uint4 *bki = A.keys.bk_ntt + (((long)i * 2 + p) * 2 + h) * 1024;
-            if (W == 4) {
-                br_digits_fwd(x, S, p, a, lane, A.keys.twb, pr);
-                __syncthreads();
-                bool staged = false;
-                if (STAGE) {
-                    staged = !G.abort && bk_wait(&G.full[u & 1], (u >> 1) & 1);
-                    if (!staged && !G.abort) {
-                        G.abort = 1;   // read this and later steps from global memory
-                        atomicOr(A.status, kErrTimeout);
-                    }
+            br_digit_fwd(x, S, wr >> 2, (wr >> 1) & 1, a, lane, A.keys.twb, pr);
+            __syncthreads();
+            bool staged = false;
+            if (STAGE) {
+                staged = !G.abort && bk_wait(&G.full[u & 1], (u >> 1) & 1);
+                if (!staged && !G.abort) {
+                    G.abort = 1;   // read this and later steps from global memory
+                    atomicOr(A.status, kErrTimeout);
                 }
-                if (staged)
-                    br_pointwise_staged(x, S, &G.bk[u & 1][p * 2 + h][0], lane, pr);
-                else
-                    br_pointwise(x, S, bki, lane, pr);
-                __syncthreads();
-                br_inverse(x, S, w4, lane, lane_brv, A.keys.twb, pr);
-                __syncthreads();
-                br_crt<16>(S, p, 16 * h, lane);
-                __syncthreads();
-            } else {
-                br_digit_fwd(x, S, wr >> 2, (wr >> 1) & 1, a, lane, A.keys.twb, pr);
-                __syncthreads();
-                bool staged = false;
-                if (STAGE) {
-                    staged = !G.abort && bk_wait(&G.full[u & 1], (u >> 1) & 1);
-                    if (!staged && !G.abort) {
-                        G.abort = 1;   // read this and later steps from global memory
-                        atomicOr(A.status, kErrTimeout);
-                    }
-                }
-                // warps w and w + 4 each take half the registers of (p, h);
-                // straight on: the inverse writes only the pair's own
-                // scratch, exchange and residue rows
-                if (wr < 4)
-                    split_pointwise_inverse<0>(x, S, X, w4, staged,
-                                               STAGE ? &G.bk[u & 1][p * 2 + h][0] : nullptr, bki,
-                                               lane, lane_brv, A.keys.twb, pr);
-                else
-                    split_pointwise_inverse<1>(x, S, X, w4, staged,
-                                               STAGE ? &G.bk[u & 1][p * 2 + h][0] : nullptr, bki,
-                                               lane, lane_brv, A.keys.twb, pr);
-                __syncthreads();
-                crt_rows<8>(S.acc[wr >> 2], X.xch[(wr >> 2) * 2 + 0], X.xch[(wr >> 2) * 2 + 1],
-                            8 * (wr & 3), lane);
-                __syncthreads();
             }
+            // warps w and w + 4 each take half the registers of (p, h);
+            // straight on: the inverse writes only the pair's own
+            // scratch, exchange and residue rows
+            if (wr < 4)
+                split_pointwise_inverse<0>(x, S, X, w4, staged,
+                                           STAGE ? &G.bk[u & 1][p * 2 + h][0] : nullptr, bki,
+                                           lane, lane_brv, A.keys.twb, pr);
+            else
+                split_pointwise_inverse<1>(x, S, X, w4, staged,
+                                           STAGE ? &G.bk[u & 1][p * 2 + h][0] : nullptr, bki,
+                                           lane, lane_brv, A.keys.twb, pr);
+            __syncthreads();
+            crt_rows<8>(S.acc[wr >> 2], X.xch[(wr >> 2) * 2 + 0], X.xch[(wr >> 2) * 2 + 1],
+                        8 * (wr & 3), lane);
+            __syncthreads();
         }
 
         if (active)
@@ -970,6 +902,464 @@ __global__ void __launch_bounds__(32 * W * B,
         for (int b = 0; b < 2; ++b)
             if (G.issued[b])
                 (void)bk_wait(&G.full[b], (G.issued[b] - 1) & 1);
+}
+
+// ---------------------------------------------------------------------
+// Blind rotation with the forward transforms' first pass on the tensor pipe
+// ---------------------------------------------------------------------
+//
+// The first pass of every forward transform is 32 negacyclic 32-point
+// transforms of digits, and digits are small (10 bits), so the pass is an
+// exact matrix product on the tensor pipe: for digit row s (of 4) and
+// column i1,
+//     V_h[s, i1][k1] = sum_i2 d_s[i1 + 32 i2] * psi_h^(32 (2 k1 + 1) i2),
+// i.e. a [128 x 32] fp16 matrix of digits (row 32 s + i1, exact: |d| <= 512)
+// times a constant [32 x 96] fp16 matrix per prime: the centred powers in
+// three balanced base-512 limbs (|limb| <= 256, exact in fp16).  Each fp32
+// sum s_l is at most 512 sum |limb| < 2^22 (checked when the operand is
+// built): an exact integer.  The accumulators start at 1.5 2^23 (one more
+// K step, 2048 x 6144), so a sum's bits are 0x4B400000 + s_l.
+//
+// A lane then forms x = sum_l 512^l s_l - Q q + 2q, Q = round(sum / q) from
+// two fp32 multiply-adds (off by less than 1.6, so x lies in (0, 4q)), and
+// the twiddle as a Shoup product: 17 issue cycles per point (2 ffma, 3 imad
+// or shift-adds at 2, 1 add, Shoup 8) against 35 of an 80-butterfly pass and
+// its twiddle product.  The twiddles of both primes stay in TMEM beside the
+// accumulators (64 words per lane and sub-partition, read like them), so the
+// pass takes nothing from the load/store pipe but its result's transpose.
+constexpr int kTbCols = 96;                        // 32 outputs x 3 limbs of one prime
+constexpr uint32_t kTbOpBytes = kTbCols * 32 * 2;  // constant operand of one prime, 6 KB
+constexpr int kTbTw = 4 * kTbCols;                 // TMEM column of the twiddles
+constexpr uint32_t kMagicBits = 0x4B400000u;
+
+// Transposes in 36-word rows: 16-byte rows for vector accesses along the row
+// (eight lanes cover all banks), consecutive words across.
+constexpr int kRowV = 36;
+constexpr int kSlotV = 32 * kRowV;
+
+// Word of (register r, lane) in a vector-ordered row of kN words: four
+// consecutive registers of a lane are one 16-byte access.
+__host__ __device__ constexpr int vec_word(int r, int lane)
+{
+    return ((r >> 2) * 32 + lane) * 4 + (r & 3);
+}
+
+struct TbSmem {                 // one bootstrap
+    uint32_t acc[2][kN];        // TLWE accumulator (a(X), b(X))
+    uint32_t fwd[2][4][kSlotV]; // forward outputs [prime][digit row] (vec_word); scratch
+    uint16_t abar[kLweStride];  // mod-switched mask and body
+};
+
+struct TbOps {                  // one CTA
+    // constant operands, 8 x 8 fp16 core matrices [K group][column group]
+    uint8_t b[2][kTbOpBytes];
+    uint8_t b1[kTbCols * 16 * 2];   // the K step of the accumulators' start value
+    uint8_t a1[128 * 16 * 2];
+    unsigned long long bar[4];  // MMA completion of each bootstrap
+    uint32_t tmem;
+    volatile int abort[4];      // a wait of the bootstrap ran out
+};
+
+// Inverse transform with vector-ordered input rows (see inv_ntt): the
+// transpose is written by words and read as 16-byte vectors.
+__device__ __forceinline__ void inv_ntt_v(uint32_t (&x)[32], uint32_t *sbuf, int lane, int lane_brv,
+                                          const uint2 *__restrict__ twb, const Prime &pr)
+{
+    gs32<true>(x, pr);
+    const uint2 *tw = twb + (pr.P * 2 + 1) * 1024 + lane;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+        const uint2 t = __ldg(tw + r * 32);
+        x[r] = mul_shoup(x[r], t.x, t.y, pr.q);
+    }
+    uint32_t *wr = sbuf + lane_brv, *rd = sbuf + lane * kRowV;
+#pragma unroll
+    for (int r = 0; r < 32; ++r)
+        wr[r * kRowV] = x[r];          // lane k1, i1 = r -> slot[i1][brv5(k1)]
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 32; r += 4) {  // lane i1 reads slot[i1][r ..]
+        const uint4 v = *reinterpret_cast<const uint4 *>(rd + r);
+        x[r] = v.x;
+        x[r + 1] = v.y;
+        x[r + 2] = v.z;
+        x[r + 3] = v.w;
+    }
+    __syncwarp();
+    gs32<false>(x, pr);
+}
+
+__device__ __forceinline__ void store_vec(uint32_t *row, const uint32_t (&x)[32], int lane)
+{
+#pragma unroll
+    for (int r = 0; r < 32; r += 4)
+        *reinterpret_cast<uint4 *>(row + vec_word(r, lane)) =
+            make_uint4(x[r], x[r + 1], x[r + 2], x[r + 3]);
+}
+
+// Key vectors of registers 4 g .. 4 g + 3.
+__device__ __forceinline__ void key_ld4(uint4 (&k)[4], const uint4 *__restrict__ bkp, int g, int lane)
+{
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        k[e] = __ldg(bkp + (4 * g + e) * 32 + lane);
+}
+
+// Phase 2 on vector-ordered rows; `k` holds the key vectors of group 0,
+// loaded before the barrier that made the rows complete.  The key vectors
+// of the next group are in flight while a group is multiplied.
+__device__ __forceinline__ void pointwise_v(uint32_t (&x)[32], const uint32_t (*f)[kSlotV],
+                                            uint4 (&k)[4], const uint4 *__restrict__ bkp, int lane,
+                                            const Prime &pr)
+{
+    const uint32_t qn = c_ntt.q_inv[pr.P];
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+        uint4 nk[4];
+        if (g < 7)
+            key_ld4(nk, bkp, g + 1, lane);
+        const int o = vec_word(4 * g, lane);
+        const uint4 f0 = *reinterpret_cast<const uint4 *>(f[0] + o);
+        const uint4 f1 = *reinterpret_cast<const uint4 *>(f[1] + o);
+        const uint4 f2 = *reinterpret_cast<const uint4 *>(f[2] + o);
+        const uint4 f3 = *reinterpret_cast<const uint4 *>(f[3] + o);
+        const uint32_t a0[4] = {f0.x, f0.y, f0.z, f0.w}, a1[4] = {f1.x, f1.y, f1.z, f1.w};
+        const uint32_t a2[4] = {f2.x, f2.y, f2.z, f2.w}, a3[4] = {f3.x, f3.y, f3.z, f3.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            uint64_t s = (uint64_t)a0[e] * k[e].x;
+            s += (uint64_t)a1[e] * k[e].y;
+            s += (uint64_t)a2[e] * k[e].z;
+            s += (uint64_t)a3[e] * k[e].w;
+            x[4 * g + e] = mont_reduce(s, pr.q, qn);
+        }
+        if (g < 7)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                k[e] = nk[e];
+    }
+}
+
+// Phase 4 (see crt_rows) of registers r0 .. r0 + NR - 1 on vector-ordered
+// residue rows.
+template <int NR>
+__device__ __forceinline__ void crt_rows_v(uint32_t *acc, const uint32_t *x0, const uint32_t *x1,
+                                           int r0, int lane)
+{
+    const uint32_t c = c_ntt.crt_c, cp = c_ntt.crt_cp, plo = c_ntt.p_lo;
+    constexpr uint32_t uh = (kQ1 - 1) / 2;
+#pragma unroll
+    for (int rr = 0; rr < NR; rr += 4) {
+        const int o = vec_word(r0 + rr, lane);
+        const uint4 v0 = *reinterpret_cast<const uint4 *>(x0 + o);
+        const uint4 v1 = *reinterpret_cast<const uint4 *>(x1 + o);
+        const uint32_t a0[4] = {v0.x, v0.y, v0.z, v0.w}, a1[4] = {v1.x, v1.y, v1.z, v1.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t u = csub(mul_shoup(a1[e] - a0[e] + 2 * kQ1, c, cp, kQ1), kQ1);
+            acc[(r0 + rr + e) * 32 + lane] += a0[e] + kQ0 * u - (u > uh ? plo : 0u);
+        }
+    }
+}
+
+
+// Shared-memory matrix descriptor: K-major, no swizzle; lbo = byte distance
+// of core matrices adjacent in K, sbo = of 8-row groups.
+__device__ __forceinline__ uint64_t tb_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
+{
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
+           ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
+}
+
+// kind::f16, fp16 A and B (K-major), fp32 accumulator, M = 128, N = 96.
+constexpr uint32_t kTbIdesc = (1u << 4) | ((uint32_t)(kTbCols >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+
+__device__ __forceinline__ void tb_mma1(uint32_t d, uint64_t a, uint64_t b, uint32_t acc)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+                 "l"(a), "l"(b), "r"(kTbIdesc), "r"(acc)
+                 : "memory");
+}
+
+// One thread: V_h of one bootstrap into TMEM columns d .. d + 95, completion
+// on `bar`.  The digit operand `a` holds 8 x 8 core matrices [K group 4][row
+// group 16].
+__device__ __forceinline__ void tb_mma(uint32_t d, uint32_t a, const TbOps &O, int prime,
+                                       unsigned long long *bar)
+{
+    tb_mma1(d, tb_desc(br_saddr(O.a1), 2048, 128), tb_desc(br_saddr(O.b1), kTbCols * 16, 128), 0);
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk)
+        tb_mma1(d, tb_desc(a + kk * 2 * 2048, 2048, 128),
+                tb_desc(br_saddr(&O.b[prime][0]) + kk * 2 * (kTbCols * 16), kTbCols * 16, 128), 1);
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                     br_saddr(bar))
+                 : "memory");
+}
+
+// 8 or 16 consecutive columns of this warp's 32 TMEM lanes.
+__device__ __forceinline__ void tb_ld8(uint32_t t, uint32_t (&v)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
+                   "=r"(v[6]), "=r"(v[7])
+                 : "r"(t));
+}
+
+__device__ __forceinline__ void tb_ld16(uint32_t t, uint32_t (&v)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, "
+                 "%10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
+                   "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]),
+                   "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                 : "r"(t));
+}
+
+// Barrier of the 128 threads of bootstrap slot `bi`.
+__device__ __forceinline__ void boot_sync(int bi)
+{
+    asm volatile("bar.sync %0, 128;" ::"r"(1 + bi) : "memory");
+}
+
+// Both digits of the coefficients lane + 32 r, r = 16 half .. + 15, of
+// polynomial c of X^a acc - acc, as fp16 into rows (2c + j) 32 + lane of the
+// digit operand.  1024 + field is exact in fp16 (bits 0x6400 | field).
+__device__ __forceinline__ void tb_digits(const uint32_t *ac, uint8_t *op, int c, int half, int a,
+                                          int lane)
+{
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {   // K group: 8 consecutive r
+        uint32_t d0[4], d1[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            uint32_t u[2];
+#pragma unroll
+            for (int o = 0; o < 2; ++o) {
+                const int k = lane + 32 * (16 * half + 8 * g + 2 * e + o);
+                const int idx = (k - a) & (2 * kN - 1);
+                uint32_t v = ac[idx & (kN - 1)];
+                v = idx >= kN ? 0u - v : v;
+                u[o] = v - ac[k] + kDecompOffset;
+            }
+            const uint32_t hi = (__byte_perm(u[0], u[1], 0x7632) >> 6) & 0x03FF03FFu;   // bits 22..31
+            const uint32_t lo = (__byte_perm(u[0], u[1], 0x6521) >> 4) & 0x03FF03FFu;   // bits 12..21
+            const __half2 off = __half2half2(__ushort_as_half(0x6600));   // 1536 = 1024 + 512
+            const uint32_t h1 = hi | 0x64006400u, l1 = lo | 0x64006400u;
+            const __half2 x0 = __hsub2(*reinterpret_cast<const __half2 *>(&h1), off);
+            const __half2 x1 = __hsub2(*reinterpret_cast<const __half2 *>(&l1), off);
+            d0[e] = *reinterpret_cast<const uint32_t *>(&x0);
+            d1[e] = *reinterpret_cast<const uint32_t *>(&x1);
+        }
+        uint8_t *p = op + (2 * half + g) * 2048 + (64 * c + lane) * 16;
+        *reinterpret_cast<uint4 *>(p) = make_uint4(d0[0], d0[1], d0[2], d0[3]);
+        *reinterpret_cast<uint4 *>(p + 32 * 16) = make_uint4(d1[0], d1[1], d1[2], d1[3]);
+    }
+}
+
+// Second half of the first pass for one digit row: the warp's 32 TMEM lanes
+// (lane i1) hold the sums of column k1 at t + 24 (k1 / 8) + 8 l + k1 % 8 and
+// its twiddle (w, w') at tw + 2 k1; twiddled residues in [0, 2q) go to
+// slot[i1][k1].
+__device__ __forceinline__ void tb_combine(uint32_t t, uint32_t tw, uint32_t *slot, const Prime &pr)
+{
+    const float c1 = pr.P ? (float)(512.0 / kQ1) : (float)(512.0 / kQ0);
+    const float c2 = pr.P ? (float)(262144.0 / kQ1) : (float)(262144.0 / kQ0);
+    const float c0 = pr.P ? (float)(12582912.0 * (1.0 - 262656.0 / kQ1))
+                          : (float)(12582912.0 * (1.0 - 262656.0 / kQ0));
+    const uint32_t off = 2u * pr.q + kMagicBits * pr.q - kMagicBits * (1u + 512u + 262144u);
+    const uint32_t nq = 0u - pr.q;
+#pragma unroll 1
+    for (int k0 = 0; k0 < 32; k0 += 8) {
+        uint32_t s0[8], s1[8], s2[8], w[16];
+        tb_ld8(t + 3 * k0, s0);
+        tb_ld8(t + 3 * k0 + 8, s1);
+        tb_ld8(t + 3 * k0 + 16, s2);
+        tb_ld16(tw + 2 * k0, w);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int v = 0; v < 8; v += 4) {
+            uint32_t o[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int e = v + k;
+                const float f = fmaf(__uint_as_float(s2[e]), c2, fmaf(__uint_as_float(s1[e]), c1, c0));
+                const uint32_t x = s1[e] * 512u + off + __float_as_uint(f) * nq + ((s2[e] << 18) + s0[e]);
+                o[k] = mul_shoup(x, w[2 * e], w[2 * e + 1], pr.q);
+            }
+            *reinterpret_cast<uint4 *>(slot + k0 + v) = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+    }
+}
+
+// Four bootstraps per CTA (one CTA per SM, 16 warps), 4 warps each, that
+// share the constant operands and twiddles and otherwise run independently
+// (barriers of 128 threads): one bootstrap's waits and memory phases are
+// covered by the other three.  Gate slots run through all CTAs first, so a
+// level of fewer than four bootstraps per SM spreads over the SMs.  Per CMux
+// step of a bootstrap:
+//   digits     warp wr: half of polynomial wr >> 1, both digits
+//   products   one thread: V_0 (TMEM, 96 columns)
+//   pass 1, 2  warp s (the TMEM lanes it can read): digit row s modulo q_0,
+//              while V_1 runs once every warp has read V_0; then modulo q_1
+//   pointwise, inverse, CRT as warp (p, h)
+// Bound: issue of the integer multiplies (IMAD 2, IMAD.HI and IMAD.WIDE 4
+// cycles of the one pipe that has them, with little overlap).  608 gates:
+// 5.94 ms (102K bootstraps/s) against 7.85 ms (77.4K/s) with both passes as
+// butterflies.  The same first pass in CTAs whose bootstraps run in lockstep
+// took 7.4-8.1 ms: every wait and table load stood alone.
+__global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
+{
+    constexpr int T = 128;
+    extern __shared__ uint4 smem_raw[];
+    TbSmem *all = reinterpret_cast<TbSmem *>(smem_raw);
+    TbOps &O = *reinterpret_cast<TbOps *>(all + 4);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int bi = warp / 4, wr = warp % 4, tb = tid % T;
+    TbSmem &S = all[bi];
+    const int lane_brv = brv5(lane);
+    const int n = A.keys.n;
+    const int p = wr >> 1, h = wr & 1;
+    const Prime pr((uint32_t)h);
+
+    for (int e = tid; e < (int)(2 * kTbOpBytes / 16); e += 512)
+        reinterpret_cast<uint4 *>(&O.b[0][0])[e] = __ldg(A.keys.tb_op + e);
+    // start value 2048 x 6144 = 1.5 2^23: K value 0 of every row and column
+    for (int e = tid; e < (int)(sizeof(O.a1) / 16); e += 512)
+        reinterpret_cast<uint4 *>(O.a1)[e] = make_uint4(e < 128 ? 0x6800u : 0u, 0u, 0u, 0u);
+    for (int e = tid; e < (int)(sizeof(O.b1) / 16); e += 512)
+        reinterpret_cast<uint4 *>(O.b1)[e] = make_uint4(e < kTbCols ? 0x6E00u : 0u, 0u, 0u, 0u);
+    if (tid < 4) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(br_saddr(&O.bar[tid]))
+                     : "memory");
+        O.abort[tid] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         br_saddr(&O.tmem)),
+                     "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = O.tmem;
+    const uint32_t tl = tmem + ((uint32_t)(32 * wr) << 16);   // this warp's TMEM lanes
+    if (bi == 0) {
+        // forward twiddles of column i1 = lane: (w, w') of prime P, output k1
+        // at column kTbTw + 2 (32 P + k1)
+        for (int c = 0; c < 64; c += 4) {
+            uint32_t v[8];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int P = (c + e) >> 5, k1 = (c + e) & 31;
+                const uint2 f = __ldg(A.keys.twb + ((P * 2) * 32 + brv5(k1)) * 32 + lane);
+                v[2 * e] = f.x;
+                v[2 * e + 1] = f.y;
+            }
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, "
+                         "%8};" ::"r"(tl + kTbTw + 2 * c),
+                         "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]),
+                         "r"(v[6]), "r"(v[7])
+                         : "memory");
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t acc_cols = tmem + (uint32_t)(bi * kTbCols);
+    const uint32_t dig_op = br_saddr(&S.fwd[1][0][0]);
+    uint32_t phase = 0;   // products waited for (the same in the bootstrap's threads)
+
+    for (long g = blockIdx.x + (long)bi * gridDim.x; g < A.count && !O.abort[bi];
+         g += 4L * gridDim.x) {
+        const bool active = br_prologue<T>(A, g, tb, S.abar, true);
+        boot_sync(bi);
+        br_acc_init<T>(A, S.acc, S.abar[n], tb);
+        boot_sync(bi);
+
+        for (int i = 0; i < n; ++i) {
+            const int a = S.abar[i];
+            if (a == 0)
+                continue;   // X^0 acc - acc = 0: nothing changes
+            tb_digits(S.acc[p], reinterpret_cast<uint8_t *>(&S.fwd[1][0][0]), p, h, a, lane);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            boot_sync(bi);
+            if (tb == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                tb_mma(acc_cols, dig_op, O, 0, &O.bar[bi]);
+            }
+            uint32_t x[32];
+            const uint4 *bki = A.keys.bk_ntt + (((long)i * 2 + p) * 2 + h) * 1024;
+#pragma unroll 1
+            for (int ph = 0; ph < 2; ++ph) {
+                const Prime pq((uint32_t)ph);
+                uint32_t *sl = S.fwd[ph][wr];
+                if (!bk_wait(&O.bar[bi], phase & 1)) {
+                    O.abort[bi] = 1;
+                    atomicOr(A.status, kErrTimeout);
+                }
+                ++phase;
+                __syncwarp();
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                tb_combine(tl + bi * kTbCols, tl + kTbTw + 64 * ph, sl + lane * kRowV, pq);
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                if (ph == 0) {
+                    // V_1 overwrites V_0 once the four warps have read it
+                    if (wr == 0) {
+                        asm volatile("bar.sync %0, 128;" ::"r"(5 + bi) : "memory");
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        if (lane == 0)
+                            tb_mma(acc_cols, dig_op, O, 1, &O.bar[bi]);
+                    } else {
+                        asm volatile("bar.arrive %0, 128;" ::"r"(5 + bi) : "memory");
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < 32; ++r)
+                    x[r] = sl[r * kRowV + lane];   // lane k1 reads slot[i1][k1]
+                __syncwarp();
+                ct32<true>(x, pq);
+                store_vec(sl, x, lane);
+            }
+            uint4 kv[4];
+            key_ld4(kv, bki, 0, lane);
+            boot_sync(bi);
+            pointwise_v(x, S.fwd[h], kv, bki, lane, pr);
+            boot_sync(bi);
+            inv_ntt_v(x, S.fwd[0][wr], lane, lane_brv, A.keys.twb, pr);
+#pragma unroll
+            for (int r = 0; r < 32; ++r)
+                x[r] = csub(x[r], pr.q);
+            store_vec(S.fwd[1][wr], x, lane);
+            boot_sync(bi);
+            crt_rows_v<16>(S.acc[p], S.fwd[1][p * 2 + 0], S.fwd[1][p * 2 + 1], 16 * h, lane);
+            boot_sync(bi);
+            if (O.abort[bi])
+                break;
+        }
+
+        if (active && !O.abort[bi])
+            br_extract<T>(A, g, S.acc, tb);
+        boot_sync(bi);
+    }
+    // after a wait that ran out: a product still in flight gets a bounded
+    // time to finish before TMEM is freed
+    if (O.abort[bi] && tb == 0)
+        (void)bk_wait(&O.bar[bi], (phase + 1) & 1);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
+                     : "memory");
+    }
 }
 
 // ---------------------------------------------------------------------
@@ -1201,9 +1591,55 @@ static int bitrev(int k, int bits)
     return r;
 }
 
+// Centred representative of v mod q.
+static int64_t centred(int64_t v, int64_t q)
+{
+    v %= q;
+    if (v < 0)
+        v += q;
+    return v > q / 2 ? v - q : v;
+}
+
+// Constant operand of the tensor-pipe first pass, op[prime] in its
+// shared-memory order.  Returns false if a bound the kernel relies on does
+// not hold.
+static bool build_tb_operand(uint16_t *op)
+{
+    const uint32_t qs[2] = {kQ0, kQ1};
+    for (int P = 0; P < 2; ++P) {
+        const int64_t q = qs[P];
+        const uint64_t psi = find_psi(qs[P]);
+        double smax[32][3] = {};   // largest |sum| of column (k1, limb)
+        for (int k1 = 0; k1 < 32; ++k1)
+            for (int i2 = 0; i2 < 32; ++i2) {
+                int64_t v = centred((int64_t)powmod(psi, 32ull * (2 * k1 + 1) * i2, q), q);
+                for (int l = 0; l < 3; ++l) {
+                    const int64_t d = l < 2 ? ((v + (256 + (1 << 30))) & 511) - 256 : v;
+                    v = (v - d) / 512;
+                    if (d < -256 || d > 256)
+                        return false;
+                    smax[k1][l] += 512.0 * (double)(d < 0 ? -d : d);
+                    // column 24 (k1 / 8) + 8 l + k1 % 8, core matrices [i2 / 8][column / 8]
+                    const int col = (k1 / 8) * 24 + 8 * l + k1 % 8;
+                    const __half hv = __float2half((float)d);
+                    uint16_t bits;
+                    std::memcpy(&bits, &hv, 2);
+                    op[P * (kTbOpBytes / 2) +
+                       (((i2 / 8) * (kTbCols / 8) + col / 8) * 8 + col % 8) * 8 + i2 % 8] = bits;
+                }
+            }
+        for (int k1 = 0; k1 < 32; ++k1)
+            for (int l = 0; l < 3; ++l)
+                if (smax[k1][l] >= 0x1p22)
+                    return false;
+    }
+    return true;
+}
+
 // Builds the NTT constants into c_ntt (current device) and the stage-B
-// twiddle table into twb_dev ([2][2][32][32] uint2).
-cudaError_t upload_ntt_constants(uint2 *twb_dev, cudaStream_t stream)
+// twiddle table into twb_dev ([2][2][32][32] uint2), and the constant operand
+// of the tensor-pipe first pass into tb_op_dev (kTbOpBytes per prime).
+cudaError_t upload_ntt_constants(uint2 *twb_dev, uint4 *tb_op_dev, cudaStream_t stream)
 {
     NttConst C;
     std::memset(&C, 0, sizeof(C));
@@ -1265,6 +1701,12 @@ cudaError_t upload_ntt_constants(uint2 *twb_dev, cudaStream_t stream)
                         stream);
     if (e != cudaSuccess)
         return e;
+    std::vector<uint16_t> op(kTbOpBytes);
+    if (!build_tb_operand(op.data()))
+        return cudaErrorInvalidValue;
+    e = cudaMemcpyAsync(tb_op_dev, op.data(), 2 * kTbOpBytes, cudaMemcpyHostToDevice, stream);
+    if (e != cudaSuccess)
+        return e;
     return cudaStreamSynchronize(stream);
 }
 
@@ -1276,63 +1718,12 @@ cudaError_t launch_bk_to_ntt(const int32_t *bk_dev, uint32_t *bk_ntt, int n, con
     return cudaGetLastError();
 }
 
-// Dynamic shared memory of a shape: B bootstraps, plus the key stages for
-// the staged shape and its control (which reserves them unused, so both run
-// one CTA per SM).
-template <int B, int STAGE, int W = 4>
-constexpr size_t br_smem(bool stage_room)
+constexpr size_t br_smem(bool staged)
 {
-    return B * sizeof(BrSmem) + (STAGE || stage_room ? sizeof(BkStage) : 0) +
-           (W == 8 ? sizeof(SplitExtra) : 0);
+    return sizeof(BrSmem) + (staged ? sizeof(BkStage) : 0) + sizeof(SplitExtra);
 }
 
-template <int B, int W, int STAGE = 0, int MINB = 0>
-static void br_prepare(size_t smem)
-{
-    cudaFuncSetAttribute(k_blind_rotate<B, W, STAGE, MINB>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_blind_rotate<B, W, STAGE, MINB>,
-                         cudaFuncAttributePreferredSharedMemoryCarveout,
-                         (int)cudaSharedmemCarveoutMaxShared);
-    (void)cudaGetLastError();
-}
-
-template <int B, int W, int STAGE = 0, int MINB = 0>
-static int br_blocks(int dev, bool stage_room = false)
-{
-    static int cached[2][64] = {{0}};
-    if (dev < 0 || dev >= 64)
-        return 1;
-    const size_t smem = br_smem<B, STAGE, W>(stage_room);
-    if (!cached[stage_room][dev]) {
-        // the attribute covers the larger of the two requests of the shape
-        br_prepare<B, W, STAGE, MINB>(br_smem<B, STAGE, W>(B == 2 && W == 4));
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_blind_rotate<B, W, STAGE, MINB>,
-                                                          32 * W * B, smem) != cudaSuccess) {
-            (void)cudaGetLastError();
-            nb = 0;
-        }
-        cached[stage_room][dev] = nb > 0 ? nb : 1;
-    }
-    return cached[stage_room][dev];
-}
-
-// Bootstraps in flight per SM for the variant (all variants: 16 warps).
-int br_blocks_per_sm()
-{
-    int dev = 0;
-    cudaGetDevice(&dev);
-    br_blocks<2, 4>(dev);
-    br_blocks<4, 4>(dev);
-    br_blocks<1, 8>(dev);
-    return br_blocks<1, 4>(dev);
-}
-
-// CTA shape: 1, 2 or 4 bootstraps per CTA in lockstep (4 warps each; groups
-// share instruction fetch and key reads but leave SMs idle when a level is
-// narrow), or kBrSplit: one bootstrap on 8 warps (shorter critical path
-// per CMux, for levels narrower than the GPU).
+// Shape of a launch: the forced or tuned code, else by batch size.
 static bool br_shape_ok(int v)
 {
     return v == 1 || v == 2 || v == 4 || v == kBrSplit || v == kBrPair || v == kBrStaged ||
@@ -1346,8 +1737,24 @@ static int br_group(long count, int num_sms, int forced, const int8_t *tuned)
     const int t = tuned[tune_bucket(count)];
     if (br_shape_ok(t))
         return t;
-    const long per_sm = (count + num_sms - 1) / num_sms;
-    return per_sm >= 8 ? 4 : (per_sm >= 3 ? 2 : kBrSplit);
+    // at most one bootstrap per SM: 2.58 ms on 8 warps (152 gates) against
+    // 3.29 ms for the throughput shape; 301 gates: 5.04 against 4.02 ms
+    return count > num_sms ? 1 : kBrSplit;
+}
+
+static cudaError_t launch_tc(const BrArgs &A, unsigned blocks, int dev, cudaStream_t stream)
+{
+    constexpr int smem = 4 * (int)sizeof(TbSmem) + (int)sizeof(TbOps);
+    static int prepared[64] = {0};
+    if (dev >= 0 && dev < 64 && !prepared[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(k_blind_rotate_tc,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess)
+            return e;
+        prepared[dev] = 1;
+    }
+    k_blind_rotate_tc<<<blocks, 512, smem, stream>>>(A);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_blind_rotate(const DevKeys &keys, const uint8_t *ops, const int32_t *in_a,
@@ -1406,39 +1813,31 @@ cudaError_t launch_blind_rotate(const DevKeys &keys, const uint8_t *ops, const i
         return staged ? cudaLaunchKernelEx(&cfg, k_blind_rotate_pair<1>, A)
                       : cudaLaunchKernelEx(&cfg, k_blind_rotate_pair<0>, A);
     }
-    const int B = (shape == kBrSplit || shape == kBrSplitStaged || shape == kBrFive) ? 1
-                : (shape == kBrStaged || shape == kBrStagedCtl) ? 2 : shape;
-    const long groups = (count + B - 1) / B;
-    long blocks_per_sm = shape == 4 ? br_blocks<4, 4>(dev)
-                       : shape == 2 ? br_blocks<2, 4>(dev)
-                       : shape == kBrStaged ? br_blocks<2, 4, 1>(dev)
-                       : shape == kBrStagedCtl ? br_blocks<2, 4>(dev, true)
-                       : shape == kBrSplitStaged ? br_blocks<1, 8, 1>(dev)
-                       : shape == kBrFive ? br_blocks<1, 4, 0, 5>(dev)
-                       : shape == kBrSplit ? br_blocks<1, 8>(dev) : br_blocks<1, 4>(dev);
-    const long cap = blocks_per_sm * (sms > 0 ? sms : 1);
-    const unsigned blocks = (unsigned)(groups < cap ? groups : cap);
     (void)grid;
-    switch (shape) {
-    case 4: k_blind_rotate<4, 4><<<blocks, 512, 4 * sizeof(BrSmem), stream>>>(A); break;
-    case 2: k_blind_rotate<2, 4><<<blocks, 256, 2 * sizeof(BrSmem), stream>>>(A); break;
-    case kBrStaged:
-        k_blind_rotate<2, 4, 1><<<blocks, 256, br_smem<2, 1>(false), stream>>>(A);
-        break;
-    case kBrStagedCtl:
-        k_blind_rotate<2, 4><<<blocks, 256, br_smem<2, 0>(true), stream>>>(A);
-        break;
-    case kBrSplitStaged:
-        k_blind_rotate<1, 8, 1><<<blocks, 256, br_smem<1, 1, 8>(false), stream>>>(A);
-        break;
-    case kBrFive: k_blind_rotate<1, 4, 0, 5><<<blocks, 128, sizeof(BrSmem), stream>>>(A); break;
-    case kBrSplit:
-        k_blind_rotate<1, 8><<<blocks, 256, br_smem<1, 0, 8>(false), stream>>>(A);
-        break;
-    default: k_blind_rotate<1, 4><<<blocks, 128, sizeof(BrSmem), stream>>>(A); break;
+    const long nsm = sms > 0 ? sms : 1;
+    if (shape == kBrSplit || shape == kBrSplitStaged) {
+        const bool staged = shape == kBrSplitStaged;
+        static int prepared[2][64] = {{0}};
+        if (dev >= 0 && dev < 64 && !prepared[staged][dev]) {
+            cudaFuncSetAttribute(staged ? k_blind_rotate<1, 8, 1> : k_blind_rotate<1, 8, 0>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)br_smem(staged));
+            cudaFuncSetAttribute(staged ? k_blind_rotate<1, 8, 1> : k_blind_rotate<1, 8, 0>,
+                                 cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared);
+            (void)cudaGetLastError();
+            prepared[staged][dev] = 1;
+        }
+        const unsigned blocks = (unsigned)(count < nsm ? count : nsm);
+        if (staged)
+            k_blind_rotate<1, 8, 1><<<blocks, 256, br_smem(true), stream>>>(A);
+        else
+            k_blind_rotate<1, 8, 0><<<blocks, 256, br_smem(false), stream>>>(A);
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
+    // the throughput shape (the other codes are accepted for saved tuning
+    // files and options)
+    return launch_tc(A, (unsigned)(count < nsm ? count : nsm), dev, stream);
 }
 
 }  // namespace tgb
-

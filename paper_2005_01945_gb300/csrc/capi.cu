@@ -11,7 +11,7 @@
 
 namespace tgb {
 
-cudaError_t upload_ntt_constants(uint2 *twb_dev, cudaStream_t stream);
+cudaError_t upload_ntt_constants(uint2 *twb_dev, uint4 *tb_op_dev, cudaStream_t stream);
 cudaError_t launch_bk_to_ntt(const int32_t *bk_dev, uint32_t *bk_ntt, int n, const uint2 *twb,
                              cudaStream_t stream);
 cudaError_t launch_keygen(int n, const int32_t *s, const int32_t *S, const uint32_t *bk_mask,
@@ -22,7 +22,6 @@ cudaError_t launch_encrypt(int n, const int32_t *s, const uint32_t *mask, const 
                            const uint8_t *bits, int32_t *cts, long count, cudaStream_t stream);
 cudaError_t launch_phase(int n, const int32_t *s, const int32_t *cts, uint32_t *phase, long count,
                          cudaStream_t stream);
-int br_blocks_per_sm();
 
 int fail(tfhe_ctx *ctx, int code, const char *fmt, ...)
 {
@@ -134,18 +133,21 @@ int tfhe_ctx_create(const tfhe_params *params, int device, tfhe_ctx **out)
     if (e == cudaSuccess)
         e = cudaMalloc(&ctx->twb, 2 * 2 * 32 * 32 * sizeof(uint2));
     if (e == cudaSuccess)
+        e = cudaMalloc(&ctx->tb_op, 2 * 96 * 32 * 2);
+    if (e == cudaSuccess)
         e = cudaMalloc(&ctx->status, sizeof(uint32_t));
     if (e == cudaSuccess)
         e = cudaMemset(ctx->status, 0, sizeof(uint32_t));
     if (e == cudaSuccess)
-        e = upload_ntt_constants(ctx->twb, 0);
+        e = upload_ntt_constants(ctx->twb, ctx->tb_op, 0);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         tfhe_ctx_destroy(ctx);
         return e == cudaErrorMemoryAllocation ? TFHE_ENOMEM : TFHE_ECUDA;
     }
-    ctx->br_grid = br_blocks_per_sm() * ctx->num_sms;
+    ctx->br_grid = 4 * ctx->num_sms;
     ctx->keys.twb = ctx->twb;
+    ctx->keys.tb_op = ctx->tb_op;
     ctx->keys.n = params->n;
     *out = ctx;
     return TFHE_OK;
@@ -206,6 +208,7 @@ void tfhe_ctx_destroy(tfhe_ctx *ctx)
         release_circuits(ctx);
         release_serving(ctx);
         cudaFree(ctx->twb);
+        cudaFree(ctx->tb_op);
         cudaFree(ctx->status);
         cudaFree(ctx->bk_ntt);
         cudaFree(ctx->ksk);

@@ -24,8 +24,8 @@
 // device-resident ciphertext pool.  Levels are ASAP (1 + the deeper
 // input) or, by default, deadline-driven: every gate keeps its ASAP depth
 // bound and levels are filled to whole waves of the GPU (a level unit of
-// 152, 608 or 760 gates, chosen per job mix from the autotuner's measured
-// level and wave times).  The compiled schedule is cached per job
+// 152 or 608 gates, chosen per job mix from the autotuner's measured level
+// times).  The compiled schedule is cached per job
 // signature and its level sequence is captured once as a CUDA graph and
 // replayed.
 #include <algorithm>
@@ -609,7 +609,6 @@ struct Plan {
     bool graph_profiled = false;     // graph carries event-record nodes
     long kernels_per_run = 0;        // kernel launches of one level sequence
     long wave = 0;                   // gates per level unit the schedule rounds to
-    int wide_shape = 0;              // blind-rotation shape of levels of >= wave gates
     std::vector<cudaEvent_t> ev;     // 3 per level: BR start, BR end / KS start, KS end
 
     ~Plan()
@@ -973,11 +972,8 @@ static cudaError_t enqueue_levels(tfhe_ctx *ctx, Plan &P, cudaStream_t st, bool 
         if (cnt == 0)
             continue;
         cudaError_t e = mark(3 * (l - 1));
-        DevKeys K = ctx->keys;
-        if (P.wide_shape && K.br_group == 0 && cnt >= P.wave)
-            K.br_group = P.wide_shape;
         if (e == cudaSuccess)
-            e = launch_blind_rotate(K, P.d_ops + off, P.pool, P.d_ia + off, P.pool_rows,
+            e = launch_blind_rotate(ctx->keys, P.d_ops + off, P.pool, P.d_ia + off, P.pool_rows,
                                     P.pool, P.d_ib + off, P.pool_rows, P.big, cnt, kMu,
                                     ctx->status, ctx->br_grid, st, P.d_ic ? P.pool : nullptr,
                                     P.d_ic ? P.d_ic + off : nullptr, P.pool_rows);
@@ -1099,29 +1095,25 @@ static int run_plan(tfhe_ctx *ctx, Plan &P, const tfhe_job *jobs, cudaStream_t s
 
 // Level unit of a job mix's schedule (the width the deadline scheduler
 // rounds levels up to): one bootstrap per SM (levels run at the tuned
-// narrow shape: lowest latency for a lone request), one wave of 4 per SM
-// (the tuned shapes), or one wave of 5 per SM (levels of a wave or more at
-// kBrFive).  Each candidate's schedule is costed with the autotuner's
-// measurements: a level of w gates costs the measured time of its width
-// bucket while w fits one 4-per-SM wave, ceil(w / wave) wave times above
-// (at 5 per SM for the 5-per-SM candidate), and the cheapest schedule is
-// used once it is at least 1 % cheaper than the 4-per-SM one.  Decided
+// narrow shape: lowest latency for a lone request) or one wave of 4 per SM.
+// Both schedules are costed with the autotuner's measurements: a level of w
+// gates costs the measured time of its width bucket while w fits one wave,
+// ceil(w / wave) wave times above, and the narrow unit is used once it is at
+// least 1 % cheaper.  Decided
 // once per job mix; without autotuner measurements the unit is one wave of
 // 4 per SM.
 static long choose_wave(tfhe_ctx *ctx, CircuitCache &C, const std::string &sig,
                         const tfhe_job *jobs, size_t njobs)
 {
-    const long w1 = ctx->num_sms, w4 = 4L * ctx->num_sms, w5 = 5L * ctx->num_sms;
+    const long w1 = ctx->num_sms, w4 = 4L * ctx->num_sms;
     const DevKeys &K = ctx->keys;
-    const float t4 = K.wave_ms[0], t5 = K.wave_ms[1];
+    const float t4 = K.wave_ms[0];
     if (!(t4 > 0.f))
         return w4;
     auto it = C.wave_choice.find(sig);
     if (it != C.wave_choice.end())
         return it->second;
-    auto level_cost = [&](long n, long unit) -> double {
-        if (unit == w5 && n >= w5)
-            return (double)((n + w5 - 1) / w5) * t5;
+    auto level_cost = [&](long n) -> double {
         if (n > w4)
             return (double)((n + w4 - 1) / w4) * t4;
         const int b = tune_bucket(n);
@@ -1133,23 +1125,15 @@ static long choose_wave(tfhe_ctx *ctx, CircuitCache &C, const std::string &sig,
             return -1.0;
         double c = 0;
         for (int l = 1; l <= S.depth; ++l)
-            c += level_cost(S.level_off[l] - S.level_off[l - 1], unit);
+            c += level_cost(S.level_off[l] - S.level_off[l - 1]);
         return c;
     };
     const double c4 = cost(w4);
     long pick = w4;
-    double best = c4;
-    if (c4 >= 0) {
-        if (K.tune_ms[0] > 0.f && w1 <= kTuneEdge[0]) {
-            const double c1 = cost(w1);
-            if (c1 >= 0 && c1 < 0.99 * best)
-                pick = w1, best = c1;
-        }
-        if (t5 > 0.f && t5 / w5 < 0.99f * t4 / w4) {
-            const double c5 = cost(w5);
-            if (c5 >= 0 && c5 < 0.99 * best)
-                pick = w5, best = c5;
-        }
+    if (c4 >= 0 && K.tune_ms[0] > 0.f && w1 <= kTuneEdge[0]) {
+        const double c1 = cost(w1);
+        if (c1 >= 0 && c1 < 0.99 * c4)
+            pick = w1;
     }
     C.wave_choice[sig] = pick;
     return pick;
@@ -1166,7 +1150,6 @@ int run_jobs(tfhe_ctx *ctx, const tfhe_job *jobs, size_t njobs, cudaStream_t st)
     long target = C.level_width > 0 ? C.level_width : 4L * ctx->num_sms;
     if (C.level_width == 0 && C.policy == TFHE_SCHED_BALANCED)
         target = choose_wave(ctx, C, sig, jobs, njobs);
-    const int wide = target == 5L * ctx->num_sms && C.level_width == 0 ? kBrFive : 0;
     const std::string key = sig + "|" + std::to_string(C.policy) + ":" + std::to_string(target);
     auto it = C.plans.find(key);
     if (it == C.plans.end()) {
@@ -1182,7 +1165,6 @@ int run_jobs(tfhe_ctx *ctx, const tfhe_job *jobs, size_t njobs, cudaStream_t st)
             C.order.erase(C.order.begin());
         }
         P->wave = target;
-        P->wide_shape = wide;
         C.order.push_back(key);
         it = C.plans.emplace(key, std::move(P)).first;
     }

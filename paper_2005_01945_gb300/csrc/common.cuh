@@ -70,25 +70,20 @@ __device__ __forceinline__ uint32_t mont_reduce(uint64_t x, uint32_t q, uint32_t
 #endif  // __CUDACC__
 
 // Per-context device pointers and sizes shared by the kernels.
-// Blind-rotation CTA shape codes: one bootstrap spread over 8 warps, and
-// one bootstrap on a cluster of two CTAs (one prime each).  The other
-// codes, 1, 2 and 4, count 4-warp bootstraps per CTA.
+// Blind-rotation shape codes: one bootstrap spread over 8 warps, and one
+// bootstrap on a cluster of two CTAs (one prime each).  1 is the throughput
+// shape (4 bootstraps per CTA); 2, 4, kBrStaged, kBrStagedCtl and kBrFive are
+// accepted for options and tuning files that name them and run it too.
 constexpr int kBrSplit = 8;
 constexpr int kBrPair = 16;
-// Two 4-warp bootstraps per CTA with the CMux step's key staged in shared
-// memory by bulk copies (one CTA per SM), and, for measuring that choice,
-// the same shape reading the key through L1 at the same occupancy.
 constexpr int kBrStaged = 32;
 constexpr int kBrStagedCtl = 33;
+constexpr int kBrFive = 5;
 // One bootstrap on 8 warps with the key staged (the latency shape, whose
 // single pointwise warp per sub-partition otherwise waits on L2 each step).
 constexpr int kBrSplitStaged = 40;
 // One bootstrap on a two-CTA cluster with each CTA's half of the key staged.
 constexpr int kBrPairStaged = 48;
-// One bootstrap per 4-warp CTA compiled for five CTAs per SM (96 registers,
-// 20 warps): one wave is 5 bootstraps per SM, for schedules whose levels
-// fill such waves.
-constexpr int kBrFive = 5;
 // Key-switch launch code for the tiled kernel (shared-memory key stages);
 // the codes 1 .. 32 are j-chunks of the direct kernel.
 constexpr int kKsTiled = 64;
@@ -97,20 +92,19 @@ struct DevKeys {
     const uint4 *bk_ntt;   // [n][2 poly][2 prime][32 reg][32 lane] x uint4(4 rows)
     const uint4 *ksk;      // [N][t][base-1][kLweStride/4] words
     const uint2 *twb;      // stage-B twiddles [2 prime][2 dir][32 reg][32 lane] (w, w')
+    const uint4 *tb_op;    // tensor-pipe first pass: constant operands of the two primes
     int n;
-    int br_group;          // blind-rotation CTA shape: 1, 2, 4 bootstraps per CTA,
-                           // kBrSplit = one bootstrap on 8 warps, kBrPair = one
-                           // bootstrap on two CTAs, 0 = tuned or by batch size
+    int br_group;          // blind-rotation shape code, 0 = tuned or by batch size
     int ks_kernel;         // key-switch kernel: kKsTiled, j-chunks 1 .. 32 of the
                            // direct kernel, 0 = tuned or by batch size
     int ks_stall;          // test hook (TFHE_OPT_TEST_KS_STALL): the tiled key
                            // switch's copy waits run out
     // Autotuned launch shapes per level-width bucket (0 = not tuned): bucket b
     // covers widths up to kTuneEdge[b] (the last bucket is unbounded).
-    int8_t tune_br[8];     // bootstraps per blind-rotation CTA
+    int8_t tune_br[8];     // blind-rotation shape
     int8_t tune_ks[8];     // key-switch kernel: kKsTiled, or j-chunks 1 .. 32
-    // Autotuned time (ms) of one full blind-rotation wave: [0] 4 bootstraps
-    // per SM (the tuned shape), [1] 5 per SM (kBrFive); 0 = not measured.
+    // Autotuned time (ms) of one full blind-rotation wave, 4 bootstraps per
+    // SM, in [0]; 0 = not measured ([1] keeps the tuning file's line format).
     float wave_ms[2];
     // Autotuned time (ms) of a level at each bucket's widest width with the
     // bucket's chosen shape; 0 = not measured.

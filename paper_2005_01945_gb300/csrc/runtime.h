@@ -18,6 +18,7 @@ struct tfhe_ctx {
     int num_sms = 0;
     int br_grid = 0;                 // persistent blind-rotation grid
     uint2 *twb = nullptr;            // stage-B twiddles
+    uint4 *tb_op = nullptr;          // tensor-pipe first pass: constant operands
     uint32_t *bk_ntt = nullptr;      // bootstrapping key, NTT domain
     uint4 *ksk = nullptr;            // key-switching key, padded rows
     uint32_t *status = nullptr;      // device status word

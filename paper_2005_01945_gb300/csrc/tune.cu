@@ -1,14 +1,13 @@
 // tune.cu -- autotuner for the launch shapes of the two bootstrapping
-// kernels: the blind-rotation CTA shape (1, 2 or 4 bootstraps per CTA in
-// lockstep, two per CTA with the key staged in shared memory, one
-// bootstrap spread over 8 warps with or without the staged key, or one
-// bootstrap on a cluster of two CTAs with or without it) and the
+// kernels: the blind-rotation shape (4 independent bootstraps per CTA, one
+// bootstrap spread over 8 warps with or without the key staged in shared
+// memory, or one bootstrap on a cluster of two CTAs with or without it) and the
 // key-switch kernel (the tiled kernel with shared-memory key stages, or
 // the direct kernel with its j-split of 1 .. 32 chunks), chosen per
 // level-width bucket by timing the candidates on synthetic ciphertexts
 // with the context's keys.  It also records the time of a level at each
-// bucket's widest width and of one full wave at 4 and at 5 bootstraps per
-// SM, from which the circuit schedules choose their level unit.
+// bucket's widest width, from which the circuit schedules choose their
+// level unit.
 // Results can be cached in a small text file keyed by device name and SM
 // count.  Launch shapes never change results (the arithmetic is exact and
 // order-independent), only time.
@@ -44,7 +43,10 @@ static std::string cache_key(int device)
     for (char &c : name)
         if (c == ' ')
             c = '_';
-    return name + ":" + std::to_string(prop.multiProcessorCount);
+    // the tag separates these kernels' times from those of files written for
+    // other blind-rotation kernels: an older line is not used, and tuning
+    // appends a new one
+    return name + ":" + std::to_string(prop.multiProcessorCount) + ":tc1";
 }
 
 static bool load_cache(const char *path, const std::string &key, DevKeys &k)
@@ -137,19 +139,13 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
         float level_ms[8] = {0.f};
         for (int b = 0; b < 8 && e == cudaSuccess; ++b) {
             const long W = widths[b];
-            // candidates from the finest launch granularity up: a later one
-            // is kept only if it is at least 2 % faster, because the timing
-            // is taken at the bucket's widest level (whole waves), where
-            // 1, 2 and 4 bootstraps per CTA tie, while the bucket's narrower
-            // levels end in part-filled waves that the finer shapes spread
-            // over more SMs
+            // the latency shapes first: a later candidate is kept only if it
+            // is at least 2 % faster at the bucket's widest level
             float best = 1e30f;
-            for (int B : {kBrSplit, kBrSplitStaged, kBrPair, kBrPairStaged, 1, 2, 4, kBrStaged}) {
+            for (int B : {kBrSplit, kBrSplitStaged, kBrPair, kBrPairStaged, 1}) {
                 // the latency shapes hold one bootstrap per SM (or SM pair):
                 // only candidates while a level fits in about one wave of them
-                if ((B == kBrSplit || B == kBrSplitStaged || B == kBrPair ||
-                     B == kBrPairStaged) &&
-                    W > 2L * ctx->num_sms)
+                if (B != 1 && W > 2L * ctx->num_sms)
                     continue;
                 K.br_group = B;
                 // best of three timed runs after a warm-up: one slow run
@@ -207,38 +203,10 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
                 }
             }
         }
-        // one full wave at 4 bootstraps per SM (the tuned shape of that
-        // width) and at 5 per SM: the level schedules pick their wave size
-        // from these times
-        float wave[2] = {0.f, 0.f};
-        std::memcpy(K.tune_br, br, sizeof(br));
-        for (int v = 0; v < 2 && e == cudaSuccess; ++v) {
-            const long W = (v == 0 ? 4L : 5L) * ctx->num_sms;
-            if (W > maxw)
-                break;
-            K.br_group = v == 0 ? 0 : kBrFive;
-            float tot = 0;
-            for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {
-                // after a key switch, as above (not timed)
-                e = launch_keyswitch(K.ksk, big, out, nullptr, W, W, ctx->prm.n, ctx->num_sms,
-                                     ctx->status, st, &K);
-                if (e == cudaSuccess)
-                    e = cudaEventRecord(e0, st);
-                if (e == cudaSuccess)
-                    e = launch_blind_rotate(K, nullptr, cts, nullptr, W, nullptr, nullptr, 0, big,
-                                            W, kMu, ctx->status, ctx->br_grid, st);
-                if (e == cudaSuccess)
-                    e = cudaEventRecord(e1, st);
-                if (e == cudaSuccess)
-                    e = cudaEventSynchronize(e1);
-                float ms = 0;
-                if (e == cudaSuccess && rep > 0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
-                    tot += ms;
-            }
-            wave[v] = tot / 3.f;
-        }
-        K.wave_ms[0] = wave[0];
-        K.wave_ms[1] = wave[1];
+        // one full wave (4 bootstraps per SM) is bucket 2's widest level: the
+        // level schedules cost wider levels in waves
+        K.wave_ms[0] = level_ms[tune_bucket(4L * ctx->num_sms)];
+        K.wave_ms[1] = 0.f;
         std::memcpy(K.tune_ms, level_ms, sizeof(level_ms));
         K.br_group = saved_group;
         keyswitch_force_chunks(0);
