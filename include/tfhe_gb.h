@@ -310,11 +310,9 @@ typedef enum {
     TFHE_OPT_BR_GROUP = 3,   /* blind-rotation shape: 1 = four bootstraps per CTA   */
                              /*    (4 warps each), one CTA per SM (2, 4, 5, 32 and  */
                              /*    33 are accepted and run it too), 8 = one         */
-                             /*    bootstrap on 8 warps, 16 = one bootstrap on a    */
-                             /*    cluster of two CTAs (two SMs, one prime each),   */
-                             /*    40 = one bootstrap on 8 warps with the key       */
-                             /*    staged, 48 = the two-CTA cluster with each CTA's */
-                             /*    half of the key staged, or 0 (default):          */
+                             /*    bootstrap on a CTA's 16 warps (40 too), 16 = one */
+                             /*    bootstrap on a cluster of two CTAs (two SMs, one */
+                             /*    prime each; 48 too), or 0 (default):             */
                              /*    autotuned, else by batch size                    */
     TFHE_OPT_SCHEDULE = 4,   /* tfhe_schedule policy of circuit schedules           */
     TFHE_OPT_LEVEL_WIDTH = 5,/* target gates per level for BALANCED (0: one wave    */

@@ -15,9 +15,8 @@
 //  * 4 warps own one bootstrap; a CTA of 16 warps per SM runs four that
 //    share constants and otherwise run independently, looping over gates
 //    (persistent grid); the accumulators never leave shared memory.  For
-//    narrow levels one bootstrap can instead take 8 warps, or a cluster of
-//    two CTAs (one prime each), and the key of the next CMux step can be
-//    staged in shared memory by bulk copies;
+//    levels of at most one bootstrap per SM one bootstrap takes the 16 warps
+//    (k_blind_rotate_wide), or a cluster of two CTAs (one prime each);
 //  * the first pass of the forward transforms, on digits of 10 bits, is an
 //    exact fp16 matrix product on the tensor pipe (k_blind_rotate_tc);
 //  * one 1024-point transform is one warp: 32 coefficients per lane,
@@ -294,123 +293,6 @@ __device__ __forceinline__ void fwd_ntt(uint32_t (&x)[32], uint32_t *sbuf, int l
     ct32<true>(x, pr);
 }
 
-// Inverse of fwd_ntt up to the factor N: input layout of fwd_ntt's output
-// with values in [0, 2q); output lane l, register r = N * coefficient
-// l + 32 r, in [0, 8q).
-__device__ __forceinline__ void inv_ntt(uint32_t (&x)[32], uint32_t *sbuf, int lane, int lane_brv,
-                                        const uint2 *__restrict__ twb, const Prime &pr)
-{
-    gs32<true>(x, pr);
-    const uint2 *tw = twb + (pr.P * 2 + 1) * 1024 + lane;
-#pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        const uint2 t = __ldg(tw + r * 32);
-        x[r] = mul_shoup(x[r], t.x, t.y, pr.q);
-    }
-    uint32_t *wr = sbuf + lane_brv, *rd = sbuf + lane * 33;
-#pragma unroll
-    for (int r = 0; r < 32; ++r)
-        wr[r * 33] = x[r];             // lane k1, i1 = r -> slot[i1][brv5(k1)]
-    __syncwarp();
-#pragma unroll
-    for (int r = 0; r < 32; ++r)
-        x[r] = rd[r];                  // lane i1 reads slot[i1][r]
-    __syncwarp();
-    gs32<false>(x, pr);
-}
-
-// The inverse transform shared by two warps of one sub-partition (the
-// 8-warp shapes): warp K holds registers 16K .. 16K + 15 of every lane.  In
-// each 32-point Gentleman-Sande pass the butterflies of distance 1 .. 8 stay
-// inside a warp's registers; the last stage (distance 16) pairs register j
-// with j + 16, so each warp publishes its reduced inputs of that stage in
-// `ex` ([32 registers][32 lanes]) and reads its partner's after a barrier
-// of the two warps (named barrier `bar`).  Every butterfly, twiddle and
-// reduction is the one gs32 / inv_ntt performs, so the result is identical.
-__device__ __forceinline__ void pair_sync(int bar)
-{
-    asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory");
-}
-
-template <bool CYC, int K>
-__device__ __forceinline__ void gs32_half(uint32_t (&x)[32], const Prime &pr, uint32_t *ex,
-                                          int lane, int bar)
-{
-    constexpr LazyPlan PL = CYC ? kPlanInvD : kPlanInvA;
-    const uint32_t(*tb)[32][2] = CYC ? c_ntt.izd : c_ntt.iza;
-#pragma unroll
-    for (int s = 4; s >= 1; --s) {
-        const int m = 1 << s, ln = 16 >> s;
-#pragma unroll
-        for (int g = 0; g < m; ++g) {
-            const uint32_t w = tb[pr.P][m + g][0];
-            const uint32_t wp = tb[pr.P][m + g][1];
-#pragma unroll
-            for (int jj = 0; jj < ln; ++jj) {
-                const int j = 2 * g * ln + jj;
-                if ((j >> 4) != K)
-                    continue;
-                const LazyStep &L = PL.st[s][g * ln + jj];
-                const uint32_t u = lazy_reduce_n(x[j], L.ru, L.nru, pr);
-                const uint32_t v = lazy_reduce_n(x[j + ln], L.rv, L.nrv, pr);
-                x[j] = u + v;
-                const uint32_t d = u - v + pr.kq(L.off);
-                x[j + ln] = (CYC && g == 0) ? d : mul_shoup(d, w, wp, pr.q);
-            }
-        }
-    }
-    // distance 16: warp 0 holds the u, warp 1 the v of every butterfly
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-        const LazyStep &L = PL.st[0][jj];
-        const int r = 16 * K + jj;
-        x[r] = K == 0 ? lazy_reduce_n(x[r], L.ru, L.nru, pr) : lazy_reduce_n(x[r], L.rv, L.nrv, pr);
-        ex[r * 32 + lane] = x[r];
-    }
-    pair_sync(bar);
-    const uint32_t w = tb[pr.P][1][0], wp = tb[pr.P][1][1];
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-        const LazyStep &L = PL.st[0][jj];
-        const int r = 16 * K + jj;
-        const uint32_t other = ex[(16 * (1 - K) + jj) * 32 + lane];
-        if (K == 0) {
-            x[r] = x[r] + other;
-        } else {
-            const uint32_t d = other - x[r] + pr.kq(L.off);
-            x[r] = CYC ? d : mul_shoup(d, w, wp, pr.q);
-        }
-        x[r] = lazy_reduce_n(x[r], PL.fin[r], PL.nfin[r], pr);
-    }
-}
-
-// inv_ntt on two warps (see gs32_half): same input layout restricted to
-// registers 16K .. 16K + 15, same output layout and values.  sbuf: the
-// pair's transpose scratch (kSlot words).
-template <int K>
-__device__ __forceinline__ void inv_ntt_half(uint32_t (&x)[32], uint32_t *sbuf, uint32_t *ex,
-                                             int lane, int lane_brv,
-                                             const uint2 *__restrict__ twb, const Prime &pr,
-                                             int bar)
-{
-    gs32_half<true, K>(x, pr, ex, lane, bar);
-    const uint2 *tw = twb + (pr.P * 2 + 1) * 1024 + lane;
-#pragma unroll
-    for (int r = 16 * K; r < 16 * K + 16; ++r) {
-        const uint2 t = __ldg(tw + r * 32);
-        x[r] = mul_shoup(x[r], t.x, t.y, pr.q);
-    }
-    uint32_t *wr = sbuf + lane_brv, *rd = sbuf + lane * 33;
-#pragma unroll
-    for (int r = 16 * K; r < 16 * K + 16; ++r)
-        wr[r * 33] = x[r];             // lane k1, i1 = r -> slot[i1][brv5(k1)]
-    pair_sync(bar);
-#pragma unroll
-    for (int r = 16 * K; r < 16 * K + 16; ++r)
-        x[r] = rd[r];                  // lane i1 reads slot[i1][r]
-    gs32_half<false, K>(x, pr, ex, lane, bar);
-}
-
 // ---------------------------------------------------------------------
 // Bootstrapping key -> NTT domain
 // ---------------------------------------------------------------------
@@ -464,36 +346,6 @@ struct BrArgs {
     uint32_t *status;
 };
 
-struct BrSmem {                 // one bootstrap
-    uint32_t acc[2][kN];        // TLWE accumulator (a(X), b(X))
-    uint32_t fwd[4][2][kSlot];  // forward outputs [digit][prime][reg*32+lane]; transpose scratch
-    uint16_t abar[kLweStride];  // mod-switched mask and body
-};
-
-// Bootstrapping key staged in shared memory (shape kBrStaged): the key of
-// CMux step i + 1, 64 KB, is bulk-copied (the TMA engine's cp.async.bulk,
-// completion counted on an mbarrier) into one buffer while step i reads the
-// other; the pointwise phase then reads the key from shared memory instead
-// of through L1.
-struct BkStage {
-    uint4 bk[2][4][kN];         // [buffer][poly p * 2 + prime h][reg*32+lane]
-    unsigned long long full[2]; // buffer landed
-    uint32_t issued[2];         // uses issued into each buffer
-    volatile int abort;         // a wait ran out: read the key from global memory
-};
-constexpr uint32_t kBkStepBytes = 4 * kN * sizeof(uint4);   // 64 KB
-
-// The 8-warp shape's own transpose scratch, exchange rows and residue rows
-// for its inverse transforms (one bootstrap per CTA leaves the room), so
-// that the warps go from their pointwise products straight into their
-// inverse transform without waiting for the others to finish reading the
-// digit transforms.  Warps w and w + 4 (one sub-partition) share the
-// pointwise products and inverse transform of (p, h) = (w >> 1, w & 1).
-struct SplitExtra {
-    uint32_t scratch[4][kSlot];  // transpose scratch of the warps of (p, h)
-    uint32_t xch[4][kN];         // residues [p * 2 + h][reg*32+lane]
-    uint32_t ex[4][kN];          // last-stage exchange of the two warps of (p, h)
-};
 constexpr long kBkSpin = 1L << 20;                           // x ~1 us per try
 
 __device__ __forceinline__ uint32_t br_saddr(const void *p)
@@ -504,8 +356,17 @@ __device__ __forceinline__ uint32_t br_saddr(const void *p)
 // Bounded wait for phase `parity` of a stage barrier; false if it ran out.
 __device__ __forceinline__ bool bk_wait(unsigned long long *bar, uint32_t parity)
 {
+    uint32_t ok;
+    // the first try suspends for the hardware's own time, not a timer's
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok)
+                 : "r"(br_saddr(bar)), "r"(parity)
+                 : "memory");
+    if (ok)
+        return true;
     for (long i = 0; i < kBkSpin; ++i) {
-        uint32_t ok;
         asm volatile("{\n\t.reg .pred p;\n\t"
                      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}"
@@ -516,147 +377,6 @@ __device__ __forceinline__ bool bk_wait(unsigned long long *bar, uint32_t parity
             return true;
     }
     return false;
-}
-
-// One thread: queue the key of CMux step i into buffer `buf` (four 16 KB
-// bulk copies of the step's contiguous 64 KB).
-__device__ __forceinline__ void bk_issue(BkStage &G, const uint4 *bk_ntt, int i, int buf)
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
-                     br_saddr(&G.full[buf])),
-                 "r"(kBkStepBytes)
-                 : "memory");
-    const uint4 *src = bk_ntt + (long)i * 4 * kN;
-#pragma unroll
-    for (int part = 0; part < 4; ++part)
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes "
-                     "[%0], [%1], %2, [%3];" ::"r"(br_saddr(&G.bk[buf][part][0])),
-                     "l"(src + part * kN), "r"((uint32_t)(kN * sizeof(uint4))),
-                     "r"(br_saddr(&G.full[buf]))
-                     : "memory");
-    G.issued[buf]++;
-}
-
-// Phase 1 with eight warps per bootstrap: warp (c, j, h) forms digit
-// polynomial j of TLWE polynomial c of X^a acc - acc and transforms it
-// modulo prime h into S.fwd[2c + j][h] (its own slot, also the transpose
-// scratch).
-__device__ __forceinline__ void digit_fwd(uint32_t (&x)[32], const uint32_t *ac, uint32_t *sj,
-                                          int j, int a, int lane, const uint2 *__restrict__ twb,
-                                          const Prime &pr)
-{
-    const int shift = j ? 12 : 22;
-#pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        const int k = lane + 32 * r;
-        const int idx = (k - a) & (2 * kN - 1);
-        uint32_t v = ac[idx & (kN - 1)];
-        v = idx >= kN ? 0u - v : v;
-        const uint32_t u = v - ac[k] + kDecompOffset;
-        x[r] = ((u >> shift) & 1023u) + (pr.q - 512u);
-    }
-    fwd_ntt(x, sj, lane, twb, pr);
-#pragma unroll
-    for (int r = 0; r < 32; ++r)
-        sj[r * 32 + lane] = x[r];
-}
-
-__device__ __forceinline__ void br_digit_fwd(uint32_t (&x)[32], BrSmem &S, int c, int j, int a,
-                                             int lane, const uint2 *__restrict__ twb,
-                                             const Prime &pr)
-{
-    digit_fwd(x, S.acc[c], S.fwd[2 * c + j][pr.P], j, a, lane, twb, pr);
-}
-
-// Phase 2: pointwise products for output polynomial p modulo prime h,
-// summed over the 4 digit rows; result in [0, 2q).  Registers R0 .. R0 +
-// NR - 1 (all 32 unless two warps share the polynomial).
-template <int R0 = 0, int NR = 32>
-__device__ __forceinline__ void br_pointwise(uint32_t (&x)[32], const uint32_t (*f)[kSlot],
-                                             const uint4 *__restrict__ bkp, int lane,
-                                             const Prime &pr)
-{
-    const uint32_t qn = c_ntt.q_inv[pr.P];
-    const uint32_t *f0 = f[0], *f1 = f[1], *f2 = f[2], *f3 = f[3];
-#pragma unroll
-    for (int r = R0; r < R0 + NR; ++r) {
-        const uint4 b = __ldg(bkp + r * 32 + lane);
-        const int e = r * 32 + lane;
-        uint64_t s = (uint64_t)f0[e] * b.x;
-        s += (uint64_t)f1[e] * b.y;
-        s += (uint64_t)f2[e] * b.z;
-        s += (uint64_t)f3[e] * b.w;
-        x[r] = mont_reduce(s, pr.q, qn);
-    }
-}
-
-template <int R0 = 0, int NR = 32>
-__device__ __forceinline__ void br_pointwise(uint32_t (&x)[32], const BrSmem &S,
-                                             const uint4 *__restrict__ bkp, int lane,
-                                             const Prime &pr)
-{
-    const uint32_t qn = c_ntt.q_inv[pr.P];
-    const uint32_t *f0 = S.fwd[0][pr.P], *f1 = S.fwd[1][pr.P], *f2 = S.fwd[2][pr.P],
-                   *f3 = S.fwd[3][pr.P];
-#pragma unroll
-    for (int r = R0; r < R0 + NR; ++r) {
-        const uint4 b = __ldg(bkp + r * 32 + lane);
-        const int e = r * 32 + lane;
-        uint64_t s = (uint64_t)f0[e] * b.x;
-        s += (uint64_t)f1[e] * b.y;
-        s += (uint64_t)f2[e] * b.z;
-        s += (uint64_t)f3[e] * b.w;
-        x[r] = mont_reduce(s, pr.q, qn);
-    }
-}
-
-// Phase 2 with the key staged in shared memory (shapes kBrStaged,
-// kBrSplitStaged).
-template <int R0 = 0, int NR = 32>
-__device__ __forceinline__ void br_pointwise_staged(uint32_t (&x)[32], const BrSmem &S,
-                                                    const uint4 *bks, int lane, const Prime &pr)
-{
-    const uint32_t qn = c_ntt.q_inv[pr.P];
-    const uint32_t *f0 = S.fwd[0][pr.P], *f1 = S.fwd[1][pr.P], *f2 = S.fwd[2][pr.P],
-                   *f3 = S.fwd[3][pr.P];
-    const uint32_t base = br_saddr(bks);
-#pragma unroll
-    for (int r = R0; r < R0 + NR; ++r) {
-        const int e = r * 32 + lane;
-        uint4 b;
-        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-                     : "r"(base + (uint32_t)e * 16u));
-        uint64_t s = (uint64_t)f0[e] * b.x;
-        s += (uint64_t)f1[e] * b.y;
-        s += (uint64_t)f2[e] * b.z;
-        s += (uint64_t)f3[e] * b.w;
-        x[r] = mont_reduce(s, pr.q, qn);
-    }
-}
-
-// Phases 2 and 3 of the 8-warp shapes: warp K of the pair (w4, w4 + 4)
-// takes registers 16K .. 16K + 15 of the pointwise products of (p, h) and
-// of its inverse transform (named barrier 1 + w4), and publishes them in the
-// pair's residue row.
-template <int K>
-__device__ __forceinline__ void split_pointwise_inverse(uint32_t (&x)[32], const BrSmem &S,
-                                                        SplitExtra &X, int w4, bool staged,
-                                                        const uint4 *bks,
-                                                        const uint4 *__restrict__ bki, int lane,
-                                                        int lane_brv,
-                                                        const uint2 *__restrict__ twb,
-                                                        const Prime &pr)
-{
-    if (staged)
-        br_pointwise_staged<16 * K, 16>(x, S, bks, lane, pr);
-    else
-        br_pointwise<16 * K, 16>(x, S, bki, lane, pr);
-    inv_ntt_half<K>(x, X.scratch[w4], X.ex[w4], lane, lane_brv, twb, pr, 1 + w4);
-#pragma unroll
-    for (int r = 16 * K; r < 16 * K + 16; ++r)
-        X.xch[w4][r * 32 + lane] = x[r];
 }
 
 // Phase 4: CRT of (v0 mod q0, v1 mod q1), any representatives in [0, 8q), to
@@ -673,19 +393,6 @@ __device__ __forceinline__ uint32_t crt_lift(uint32_t v0, uint32_t v1, int32_t c
     const int32_t k = (int32_t)(((int64_t)x * cp + 0x80000000ll) >> 32);
     const uint32_t u = (uint32_t)x * (uint32_t)c - (uint32_t)k * kQ1;
     return v0 + kQ0 * u;
-}
-
-// The calling warp lifts registers r0 .. r0 + NR - 1 of polynomial p.
-template <int NR>
-__device__ __forceinline__ void crt_rows(uint32_t *acc, const uint32_t *x0, const uint32_t *x1,
-                                         int r0, int lane)
-{
-    const int32_t c = c_ntt.crt_c, cp = c_ntt.crt_cp;
-#pragma unroll
-    for (int rr = 0; rr < NR; ++rr) {
-        const int e = (r0 + rr) * 32 + lane;
-        acc[e] += crt_lift(x0[e], x1[e], c, cp);
-    }
 }
 
 // Linear part of gate `op`: c = mu + aa ca + ab cb + ac cc.  Returns false
@@ -797,118 +504,6 @@ __device__ __forceinline__ void br_extract(const BrArgs &A, long g, const uint32
         bg[kN] = (int32_t)acc[1][0];
 }
 
-// One bootstrap per CTA on W = 8 warps (one CTA per SM), for levels narrower
-// than the GPU: warp (c, j, h) runs phase 1 for digit j of polynomial c;
-// warps w and w + 4 share phases 2-3 of (p, h); every warp runs phase 4 on a
-// quarter of polynomial w >> 2.
-template <int B, int W, int STAGE>
-__global__ void __launch_bounds__(32 * W * B,
-                                  1)
-    k_blind_rotate(const BrArgs A)
-{
-    constexpr int T = 32 * W;      // threads per bootstrap
-    extern __shared__ uint4 smem_raw[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int bi = warp / W, wr = warp % W, tb = tid % T;   // bootstrap slot, role
-    BrSmem &S = reinterpret_cast<BrSmem *>(smem_raw)[bi];
-    BkStage &G = *reinterpret_cast<BkStage *>(reinterpret_cast<BrSmem *>(smem_raw) + B);
-    SplitExtra &X = *reinterpret_cast<SplitExtra *>(
-        reinterpret_cast<uint8_t *>(reinterpret_cast<BrSmem *>(smem_raw) + B) +
-        (STAGE ? sizeof(BkStage) : 0));
-    const int lane_brv = brv5(lane);
-    const int n = A.keys.n;
-    const int w4 = wr & 3, p = w4 >> 1, h = wr & 1;
-    const Prime pr((uint32_t)h);
-    uint32_t uses = 0;   // staged steps so far (the same in every thread)
-
-    if (STAGE) {
-        if (tid == 0) {
-            for (int b = 0; b < 2; ++b) {
-                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(br_saddr(&G.full[b]))
-                             : "memory");
-                G.issued[b] = 0;
-            }
-            G.abort = 0;
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-        __syncthreads();
-    }
-
-    for (long grp = blockIdx.x; grp * B < A.count; grp += gridDim.x) {
-        const long g = grp * B + bi;
-        const bool active = br_prologue<T>(A, g, tb, S.abar, true);
-        if (STAGE && tid == 0 && n > 0 && !G.abort)
-            bk_issue(G, A.keys.bk_ntt, 0, uses & 1);
-        __syncthreads();
-        br_acc_init<T>(A, S.acc, S.abar[n], tb);
-        __syncthreads();
-
-        // ---- n CMux steps, all B bootstraps in lockstep
-        const BrSmem *all = reinterpret_cast<const BrSmem *>(smem_raw);
-        for (int i = 0; i < n; ++i) {
-            const uint32_t u = uses;   // this step's use of buffer u & 1
-            if (STAGE) {
-                ++uses;
-                // the other buffer was last read in step i - 1, before the
-                // barrier that ended that step's pointwise phase
-                if (tid == 0 && i + 1 < n && !G.abort)
-                    bk_issue(G, A.keys.bk_ntt, i + 1, (u + 1) & 1);
-            }
-            int any = 0;
-#pragma unroll
-            for (int b = 0; b < B; ++b)
-                any |= all[b].abar[i];
-            if (any == 0) {
-                // X^0 acc - acc = 0 for every slot: nothing changes; the
-                // step's copy still has to land before its buffer is reused
-                if (STAGE && tid == 0 && !G.abort && !bk_wait(&G.full[u & 1], (u >> 1) & 1)) {
-                    G.abort = 1;
-                    atomicOr(A.status, kErrTimeout);
-                }
-                continue;
-            }
-            const int a = S.abar[i];  // a = 0 here gives zero digits: acc unchanged
-            uint32_t x[32];
-            const uint4 *bki = A.keys.bk_ntt + (((long)i * 2 + p) * 2 + h) * 1024;
-            br_digit_fwd(x, S, wr >> 2, (wr >> 1) & 1, a, lane, A.keys.twb, pr);
-            __syncthreads();
-            bool staged = false;
-            if (STAGE) {
-                staged = !G.abort && bk_wait(&G.full[u & 1], (u >> 1) & 1);
-                if (!staged && !G.abort) {
-                    G.abort = 1;   // read this and later steps from global memory
-                    atomicOr(A.status, kErrTimeout);
-                }
-            }
-            // warps w and w + 4 each take half the registers of (p, h);
-            // straight on: the inverse writes only the pair's own
-            // scratch, exchange and residue rows
-            if (wr < 4)
-                split_pointwise_inverse<0>(x, S, X, w4, staged,
-                                           STAGE ? &G.bk[u & 1][p * 2 + h][0] : nullptr, bki,
-                                           lane, lane_brv, A.keys.twb, pr);
-            else
-                split_pointwise_inverse<1>(x, S, X, w4, staged,
-                                           STAGE ? &G.bk[u & 1][p * 2 + h][0] : nullptr, bki,
-                                           lane, lane_brv, A.keys.twb, pr);
-            __syncthreads();
-            crt_rows<8>(S.acc[wr >> 2], X.xch[(wr >> 2) * 2 + 0], X.xch[(wr >> 2) * 2 + 1],
-                        8 * (wr & 3), lane);
-            __syncthreads();
-        }
-
-        if (active)
-            br_extract<T>(A, g, S.acc, tb);
-        __syncthreads();
-    }
-    // after a wait that ran out: copies still in flight land before the
-    // CTA's shared memory is released (the last use of each buffer)
-    if (STAGE && tid == 0 && G.abort)
-        for (int b = 0; b < 2; ++b)
-            if (G.issued[b])
-                (void)bk_wait(&G.full[b], (G.issued[b] - 1) & 1);
-}
-
 // ---------------------------------------------------------------------
 // Blind rotation with the forward transforms' first pass on the tensor pipe
 // ---------------------------------------------------------------------
@@ -1010,6 +605,31 @@ __device__ __forceinline__ void key_ld4(uint4 (&k)[4], const uint4 *__restrict__
         k[e] = __ldg(bkp + (4 * g + e) * 32 + lane);
 }
 
+// Phase 2 of registers 4 g .. 4 g + 3 on vector-ordered rows into x[at ..];
+// their key vectors are k[at ..] (k[0 ..] of an array of four).
+template <int M, int KN, int W>
+__device__ __forceinline__ void pointwise_4(uint32_t (&x)[M], int at, const uint32_t (*f)[W],
+                                            int g, const uint4 (&k)[KN], int lane, const Prime &pr)
+{
+    const uint32_t qn = c_ntt.q_inv[pr.P];
+    const int o = vec_word(4 * g, lane);
+    const uint4 f0 = *reinterpret_cast<const uint4 *>(f[0] + o);
+    const uint4 f1 = *reinterpret_cast<const uint4 *>(f[1] + o);
+    const uint4 f2 = *reinterpret_cast<const uint4 *>(f[2] + o);
+    const uint4 f3 = *reinterpret_cast<const uint4 *>(f[3] + o);
+    const uint32_t a0[4] = {f0.x, f0.y, f0.z, f0.w}, a1[4] = {f1.x, f1.y, f1.z, f1.w};
+    const uint32_t a2[4] = {f2.x, f2.y, f2.z, f2.w}, a3[4] = {f3.x, f3.y, f3.z, f3.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const uint4 b = k[KN == 4 ? e : at + e];
+        uint64_t s = (uint64_t)a0[e] * b.x;
+        s += (uint64_t)a1[e] * b.y;
+        s += (uint64_t)a2[e] * b.z;
+        s += (uint64_t)a3[e] * b.w;
+        x[at + e] = mont_reduce(s, pr.q, qn);
+    }
+}
+
 // Phase 2 on vector-ordered rows; `k` holds the key vectors of group 0,
 // loaded before the barrier that made the rows complete.  The key vectors
 // of the next group are in flight while a group is multiplied.
@@ -1017,27 +637,12 @@ __device__ __forceinline__ void pointwise_v(uint32_t (&x)[32], const uint32_t (*
                                             uint4 (&k)[4], const uint4 *__restrict__ bkp, int lane,
                                             const Prime &pr)
 {
-    const uint32_t qn = c_ntt.q_inv[pr.P];
 #pragma unroll
     for (int g = 0; g < 8; ++g) {
         uint4 nk[4];
         if (g < 7)
             key_ld4(nk, bkp, g + 1, lane);
-        const int o = vec_word(4 * g, lane);
-        const uint4 f0 = *reinterpret_cast<const uint4 *>(f[0] + o);
-        const uint4 f1 = *reinterpret_cast<const uint4 *>(f[1] + o);
-        const uint4 f2 = *reinterpret_cast<const uint4 *>(f[2] + o);
-        const uint4 f3 = *reinterpret_cast<const uint4 *>(f[3] + o);
-        const uint32_t a0[4] = {f0.x, f0.y, f0.z, f0.w}, a1[4] = {f1.x, f1.y, f1.z, f1.w};
-        const uint32_t a2[4] = {f2.x, f2.y, f2.z, f2.w}, a3[4] = {f3.x, f3.y, f3.z, f3.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            uint64_t s = (uint64_t)a0[e] * k[e].x;
-            s += (uint64_t)a1[e] * k[e].y;
-            s += (uint64_t)a2[e] * k[e].z;
-            s += (uint64_t)a3[e] * k[e].w;
-            x[4 * g + e] = mont_reduce(s, pr.q, qn);
-        }
+        pointwise_4(x, 4 * g, f, g, k, lane, pr);
         if (g < 7)
 #pragma unroll
             for (int e = 0; e < 4; ++e)
@@ -1125,9 +730,23 @@ __device__ __forceinline__ void boot_sync(int bi)
     asm volatile("bar.sync %0, 128;" ::"r"(1 + bi) : "memory");
 }
 
+// Both digits of the words u0 and u1 (offset added) as fp16 pairs.
+// 1024 + field is exact in fp16 (bits 0x6400 | field).
+__device__ __forceinline__ void tb_digit2(uint32_t u0, uint32_t u1, uint32_t &d0, uint32_t &d1)
+{
+    const uint32_t hi = (__byte_perm(u0, u1, 0x7632) >> 6) & 0x03FF03FFu;   // bits 22..31
+    const uint32_t lo = (__byte_perm(u0, u1, 0x6521) >> 4) & 0x03FF03FFu;   // bits 12..21
+    const __half2 off = __half2half2(__ushort_as_half(0x6600));   // 1536 = 1024 + 512
+    const uint32_t h1 = hi | 0x64006400u, l1 = lo | 0x64006400u;
+    const __half2 x0 = __hsub2(*reinterpret_cast<const __half2 *>(&h1), off);
+    const __half2 x1 = __hsub2(*reinterpret_cast<const __half2 *>(&l1), off);
+    d0 = *reinterpret_cast<const uint32_t *>(&x0);
+    d1 = *reinterpret_cast<const uint32_t *>(&x1);
+}
+
 // Both digits of the coefficients lane + 32 r, r = 16 half .. + 15, of
 // polynomial c of X^a acc - acc, as fp16 into rows (2c + j) 32 + lane of the
-// digit operand.  1024 + field is exact in fp16 (bits 0x6400 | field).
+// digit operand.
 __device__ __forceinline__ void tb_digits(const uint32_t *ac, uint8_t *op, int c, int half, int a,
                                           int lane)
 {
@@ -1145,14 +764,7 @@ __device__ __forceinline__ void tb_digits(const uint32_t *ac, uint8_t *op, int c
                 v = idx >= kN ? 0u - v : v;
                 u[o] = v - ac[k] + kDecompOffset;
             }
-            const uint32_t hi = (__byte_perm(u[0], u[1], 0x7632) >> 6) & 0x03FF03FFu;   // bits 22..31
-            const uint32_t lo = (__byte_perm(u[0], u[1], 0x6521) >> 4) & 0x03FF03FFu;   // bits 12..21
-            const __half2 off = __half2half2(__ushort_as_half(0x6600));   // 1536 = 1024 + 512
-            const uint32_t h1 = hi | 0x64006400u, l1 = lo | 0x64006400u;
-            const __half2 x0 = __hsub2(*reinterpret_cast<const __half2 *>(&h1), off);
-            const __half2 x1 = __hsub2(*reinterpret_cast<const __half2 *>(&l1), off);
-            d0[e] = *reinterpret_cast<const uint32_t *>(&x0);
-            d1[e] = *reinterpret_cast<const uint32_t *>(&x1);
+            tb_digit2(u[0], u[1], d0[e], d1[e]);
         }
         uint8_t *p = op + (2 * half + g) * 2048 + (64 * c + lane) * 16;
         *reinterpret_cast<uint4 *>(p) = make_uint4(d0[0], d0[1], d0[2], d0[3]);
@@ -1164,7 +776,8 @@ __device__ __forceinline__ void tb_digits(const uint32_t *ac, uint8_t *op, int c
 // (lane i1) hold the sums of column k1 at t + 24 (k1 / 8) + 8 l + k1 % 8 and
 // its twiddle (w, w') at tw + 2 k1; twiddled residues in [0, 2q) go to
 // slot[i1][k1].
-__device__ __forceinline__ void tb_combine(uint32_t t, uint32_t tw, uint32_t *slot, const Prime &pr)
+__device__ __forceinline__ void tb_combine(uint32_t t, uint32_t tw, uint32_t *slot, const Prime &pr,
+                                           int k_lo = 0, int k_hi = 32)
 {
     const float c1 = pr.P ? (float)(512.0 / kQ1) : (float)(512.0 / kQ0);
     const float c2 = pr.P ? (float)(262144.0 / kQ1) : (float)(262144.0 / kQ0);
@@ -1173,7 +786,7 @@ __device__ __forceinline__ void tb_combine(uint32_t t, uint32_t tw, uint32_t *sl
     const uint32_t off = 2u * pr.q + kMagicBits * pr.q - kMagicBits * (1u + 512u + 262144u);
     const uint32_t nq = 0u - pr.q;
 #pragma unroll 1
-    for (int k0 = 0; k0 < 32; k0 += 8) {
+    for (int k0 = k_lo; k0 < k_hi; k0 += 8) {
         uint32_t s0[8], s1[8], s2[8], w[16];
         tb_ld8(t + 3 * k0, s0);
         tb_ld8(t + 3 * k0 + 8, s1);
@@ -1187,11 +800,79 @@ __device__ __forceinline__ void tb_combine(uint32_t t, uint32_t tw, uint32_t *sl
             for (int k = 0; k < 4; ++k) {
                 const int e = v + k;
                 const float f = fmaf(__uint_as_float(s2[e]), c2, fmaf(__uint_as_float(s1[e]), c1, c0));
-                const uint32_t x = s1[e] * 512u + off + __float_as_uint(f) * nq + ((s2[e] << 18) + s0[e]);
+                const uint32_t y = (s1[e] << 9) + ((s2[e] << 18) + s0[e]);
+                const uint32_t x = __float_as_uint(f) * nq + (y + off);
                 o[k] = mul_shoup(x, w[2 * e], w[2 * e + 1], pr.q);
             }
             *reinterpret_cast<uint4 *>(slot + k0 + v) = make_uint4(o[0], o[1], o[2], o[3]);
         }
+    }
+}
+
+// Prologue of a 512-thread CTA: constant operands, barriers, all of TMEM, and
+// the forward twiddles at TMEM column tw_col.
+__device__ __forceinline__ void tb_setup(const BrArgs &A, TbOps &O, int tid, int tw_col)
+{
+    const int warp = tid >> 5, lane = tid & 31;
+    for (int e = tid; e < (int)(2 * kTbOpBytes / 16); e += 512)
+        reinterpret_cast<uint4 *>(&O.b[0][0])[e] = __ldg(A.keys.tb_op + e);
+    // start value 2048 x 6144 = 1.5 2^23: K value 0 of every row and column
+    for (int e = tid; e < (int)(sizeof(O.a1) / 16); e += 512)
+        reinterpret_cast<uint4 *>(O.a1)[e] = make_uint4(e < 128 ? 0x6800u : 0u, 0u, 0u, 0u);
+    for (int e = tid; e < (int)(sizeof(O.b1) / 16); e += 512)
+        reinterpret_cast<uint4 *>(O.b1)[e] = make_uint4(e < kTbCols ? 0x6E00u : 0u, 0u, 0u, 0u);
+    if (tid < 4) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(br_saddr(&O.bar[tid]))
+                     : "memory");
+        O.abort[tid] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         br_saddr(&O.tmem)),
+                     "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp < 4) {
+        const uint32_t tl = O.tmem + ((uint32_t)(32 * warp) << 16);
+        // forward twiddles of column i1 = lane: (w, w') of prime P, output k1
+        // at column tw_col + 2 (32 P + k1)
+        for (int c = 0; c < 64; c += 4) {
+            uint32_t v[8];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int P = (c + e) >> 5, k1 = (c + e) & 31;
+                const uint2 f = __ldg(A.keys.twb + ((P * 2) * 32 + brv5(k1)) * 32 + lane);
+                v[2 * e] = f.x;
+                v[2 * e + 1] = f.y;
+            }
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, "
+                         "%8};" ::"r"(tl + tw_col + 2 * c),
+                         "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]),
+                         "r"(v[6]), "r"(v[7])
+                         : "memory");
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+
+// Frees TMEM; the last thing a CTA does.
+__device__ __forceinline__ void tb_release(uint32_t tmem, int warp)
+{
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
+                     : "memory");
     }
 }
 
@@ -1225,55 +906,9 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
     const int p = wr >> 1, h = wr & 1;
     const Prime pr((uint32_t)h);
 
-    for (int e = tid; e < (int)(2 * kTbOpBytes / 16); e += 512)
-        reinterpret_cast<uint4 *>(&O.b[0][0])[e] = __ldg(A.keys.tb_op + e);
-    // start value 2048 x 6144 = 1.5 2^23: K value 0 of every row and column
-    for (int e = tid; e < (int)(sizeof(O.a1) / 16); e += 512)
-        reinterpret_cast<uint4 *>(O.a1)[e] = make_uint4(e < 128 ? 0x6800u : 0u, 0u, 0u, 0u);
-    for (int e = tid; e < (int)(sizeof(O.b1) / 16); e += 512)
-        reinterpret_cast<uint4 *>(O.b1)[e] = make_uint4(e < kTbCols ? 0x6E00u : 0u, 0u, 0u, 0u);
-    if (tid < 4) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(br_saddr(&O.bar[tid]))
-                     : "memory");
-        O.abort[tid] = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         br_saddr(&O.tmem)),
-                     "r"(512u)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tb_setup(A, O, tid, kTbTw);
     const uint32_t tmem = O.tmem;
     const uint32_t tl = tmem + ((uint32_t)(32 * wr) << 16);   // this warp's TMEM lanes
-    if (bi == 0) {
-        // forward twiddles of column i1 = lane: (w, w') of prime P, output k1
-        // at column kTbTw + 2 (32 P + k1)
-        for (int c = 0; c < 64; c += 4) {
-            uint32_t v[8];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int P = (c + e) >> 5, k1 = (c + e) & 31;
-                const uint2 f = __ldg(A.keys.twb + ((P * 2) * 32 + brv5(k1)) * 32 + lane);
-                v[2 * e] = f.x;
-                v[2 * e + 1] = f.y;
-            }
-            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, "
-                         "%8};" ::"r"(tl + kTbTw + 2 * c),
-                         "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]),
-                         "r"(v[6]), "r"(v[7])
-                         : "memory");
-        }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t acc_cols = tmem + (uint32_t)(bi * kTbCols);
     const uint32_t dig_op = br_saddr(&S.fwd[1][0][0]);
     uint32_t phase = 0;   // products waited for (the same in the bootstrap's threads)
@@ -1352,201 +987,542 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
     // time to finish before TMEM is freed
     if (O.abort[bi] && tb == 0)
         (void)bk_wait(&O.bar[bi], (phase + 1) & 1);
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
-                     : "memory");
+    tb_release(tmem, warp);
+}
+
+// ---------------------------------------------------------------------
+// One bootstrap on the 16 warps of a CTA, for levels of at most one
+// bootstrap per SM, whose time is the length of a CMux step.
+// ---------------------------------------------------------------------
+//
+// The arithmetic of k_blind_rotate_tc with every phase spread over all 16
+// warps (q, z) = (warp % 4, warp / 4); a 32-point pass is cut into register
+// blocks that exchange through shared memory:
+//   digits      polynomial q >> 1, 4 coefficients per lane
+//   first pass  digit row q (the TMEM lanes it can read), prime z >> 1,
+//               outputs 16 (z & 1) ..; both primes' products run at once
+//   second pass the same row and prime, output half z & 1
+//   pointwise, inverse passes   (p, h) = (q >> 1, q & 1), 8 registers; after
+//               three stages the four warps of a (p, h) exchange and run the
+//               last two on two quadruples
+//   CRT         polynomial p, 4 coefficients per lane (kept in registers: the
+//               same as the digits')
+// The key of a step is loaded behind the fence of its digits (which would wait
+// for it), the inverse's twiddles once.
+// Bound: the integer multiplies (their pipe is busy 60 % of a step's 7.9K cycles)
+// and the waits between nine barriers.  One gate 2.43 -> 2.05 ms, 152 gates
+// 2.65 -> 2.09 ms against a shape of 8 warps whose first pass was butterflies.
+struct WideSmem {
+    uint32_t acc[2][kN];            // TLWE accumulator (a(X), b(X))
+    uint8_t dig[128 * 32 * 2];      // digit operand
+    uint32_t slot[2][4][kSlotV];    // transposes of the forward transforms
+    uint32_t fwd[2][4][kN];         // forward outputs [prime][digit row] (vec_word)
+    uint32_t ex[4][kN];             // exchange of the inverse passes [p * 2 + h]
+    uint32_t tr[4][kSlotV];         // transposes of the inverse transforms
+    uint32_t res[4][kN];            // residues [p * 2 + h][reg*32+lane]
+    uint16_t abar[kLweStride];
+};
+
+template <int T>
+__device__ __forceinline__ void warps_sync(int bar)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(T) : "memory");
+}
+
+// Half K (registers 16 K .. 16 K + 15) of ct32<true>: the first stage reads
+// all 32 inputs, the others stay inside the half.
+template <int K>
+__device__ __forceinline__ void ct32_cyc_half(uint32_t (&y)[32], const uint32_t *row, int stride,
+                                              const Prime &pr)
+{
+    constexpr LazyPlan PL = kPlanFwdD;
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) {
+        const LazyStep &L = PL.st[0][jj];
+        const uint32_t u = lazy_reduce_n(row[jj * stride], L.ru, L.nru, pr);
+        const uint32_t v = lazy_reduce_n(row[(jj + 16) * stride], L.rv, L.nrv, pr);
+        y[16 * K + jj] = K == 0 ? u + v : u - v + pr.kq(L.off);
     }
+#pragma unroll
+    for (int s = 1; s < 5; ++s) {
+        const int m = 1 << s, ln = 16 >> s;
+#pragma unroll
+        for (int g = K * m / 2; g < (K + 1) * m / 2; ++g) {
+            const uint32_t w = c_ntt.zd[pr.P][m + g][0];
+            const uint32_t wp = c_ntt.zd[pr.P][m + g][1];
+#pragma unroll
+            for (int jj = 0; jj < ln; ++jj) {
+                const int j = 2 * g * ln + jj;
+                const LazyStep &L = PL.st[s][g * ln + jj];
+                const uint32_t u = lazy_reduce_n(y[j], L.ru, L.nru, pr);
+                const uint32_t t = g == 0 ? lazy_reduce_n(y[j + ln], L.rv, L.nrv, pr)
+                                          : mul_shoup(y[j + ln], w, wp, pr.q);
+                y[j] = u + t;
+                y[j + ln] = u - t + pr.kq(L.off);
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 16 * K; r < 16 * K + 16; ++r)
+        y[r] = lazy_reduce_n(y[r], PL.fin[r], PL.nfin[r], pr);
+}
+
+// The first three stages of gs32 on the register block 8 z .. 8 z + 7;
+// inputs [0, 2q).  The bounds by position are 16, 8, 4, 4, 2, 2, 2, 2 (times
+// q), the first two reduced to `fin` (a group whose twiddle is 1 takes its
+// product too, so that the four warps run the same code).
+template <bool CYC>
+__device__ __forceinline__ void gs32_block(uint32_t (&x)[8], int z, const Prime &pr)
+{
+    const uint32_t(*tb)[2] = CYC ? c_ntt.izd[pr.P] : c_ntt.iza[pr.P];
+#pragma unroll
+    for (int s = 4; s >= 2; --s) {
+        const int m = 1 << s, ln = 16 >> s;
+#pragma unroll
+        for (int gl = 0; gl < m / 4; ++gl) {
+            const uint32_t w = tb[m + z * (m / 4) + gl][0], wp = tb[m + z * (m / 4) + gl][1];
+#pragma unroll
+            for (int jj = 0; jj < ln; ++jj) {
+                const int j = 2 * gl * ln + jj;
+                const uint32_t u = x[j], v = x[j + ln];
+                x[j] = u + v;
+                x[j + ln] = mul_shoup(u - v + pr.kq(2 * ln), w, wp, pr.q);
+            }
+        }
+    }
+    x[0] = csub(x[0], pr.kq(8));
+    if (!CYC) {
+        x[0] = csub(x[0], pr.kq(4));
+        x[1] = csub(x[1], pr.kq(4));
+    }
+}
+
+// The last two stages of gs32 on registers jj, jj + 8, jj + 16, jj + 24.
+// CYC: inputs below 8q, results below 32q (into a Shoup product); else inputs
+// below 4q, results below 8q.
+template <bool CYC>
+__device__ __forceinline__ void gs32_last(uint32_t &a0, uint32_t &a1, uint32_t &a2, uint32_t &a3,
+                                          const Prime &pr)
+{
+    const uint32_t(*tb)[2] = CYC ? c_ntt.izd[pr.P] : c_ntt.iza[pr.P];
+    constexpr int B = CYC ? 8 : 4;
+    const uint32_t t0 = a0 + a1, t2 = a2 + a3;
+    uint32_t t1 = a0 - a1 + pr.kq(B);
+    if (!CYC)
+        t1 = mul_shoup(t1, tb[2][0], tb[2][1], pr.q);
+    const uint32_t t3 = mul_shoup(a2 - a3 + pr.kq(B), tb[3][0], tb[3][1], pr.q);
+    a0 = t0 + t2;
+    a1 = t1 + t3;
+    a2 = t0 - t2 + pr.kq(2 * B);
+    a3 = t1 - t3 + pr.kq(2);
+    if (!CYC) {
+        a0 = csub(a0, pr.kq(8));
+        a2 = mul_shoup(a2, tb[1][0], tb[1][1], pr.q);
+        a3 = mul_shoup(a3, tb[1][0], tb[1][1], pr.q);
+    }
+}
+
+// One 32-point inverse pass of a (p, h): x holds registers 8 z + e, on
+// return registers 2 z + (e & 1) + 8 (e >> 1).
+template <bool CYC>
+__device__ __forceinline__ void gs32_four(uint32_t (&x)[8], uint32_t *ex, int z, int lane, int bar,
+                                          const Prime &pr)
+{
+    gs32_block<CYC>(x, z, pr);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        ex[(8 * z + e) * 32 + lane] = x[e];
+    warps_sync<128>(bar);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        x[e] = ex[(2 * z + (e & 1) + 8 * (e >> 1)) * 32 + lane];
+    gs32_last<CYC>(x[0], x[2], x[4], x[6], pr);
+    gs32_last<CYC>(x[1], x[3], x[5], x[7], pr);
+}
+
+// Both digits of the thread's four coefficients lane + 32 (c_lo + e) of one
+// polynomial, 8 bytes each at o (level 1) and 32 rows on (level 2).
+__device__ __forceinline__ void wide_digits(const uint32_t *ac, const uint32_t (&own)[4], uint8_t *o,
+                                            int c_lo, int a, int lane)
+{
+    uint32_t u[4], d0[2], d1[2];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int idx = (lane + 32 * (c_lo + e) - a) & (2 * kN - 1);
+        uint32_t v = ac[idx & (kN - 1)];
+        v = idx >= kN ? 0u - v : v;
+        u[e] = v - own[e] + kDecompOffset;
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+        tb_digit2(u[2 * e], u[2 * e + 1], d0[e], d1[e]);
+    *reinterpret_cast<uint2 *>(o) = make_uint2(d0[0], d0[1]);
+    *reinterpret_cast<uint2 *>(o + 32 * 16) = make_uint2(d1[0], d1[1]);
+}
+
+// Inverse transform by four warps (block z of each), see gs32_four.
+__device__ __forceinline__ void wide_inverse(uint32_t (&x)[8], uint32_t *ex, uint32_t *tr,
+                                             const uint2 (&tw)[8], int z, int lane, int lane_brv,
+                                             int bar, const Prime &pr)
+{
+    gs32_four<true>(x, ex, z, lane, bar, pr);
+    uint32_t *wr = tr + lane_brv;
+#pragma unroll
+    for (int e = 0; e < 8; ++e)   // lane k1, i1 -> row i1
+        wr[(2 * z + (e & 1) + 8 * (e >> 1)) * kRowV] = mul_shoup(x[e], tw[e].x, tw[e].y, pr.q);
+    warps_sync<128>(bar);
+    const uint32_t *rd = tr + lane * kRowV + 8 * z;
+    const uint4 v0 = *reinterpret_cast<const uint4 *>(rd);
+    const uint4 v1 = *reinterpret_cast<const uint4 *>(rd + 4);
+    x[0] = v0.x, x[1] = v0.y, x[2] = v0.z, x[3] = v0.w;
+    x[4] = v1.x, x[5] = v1.y, x[6] = v1.z, x[7] = v1.w;
+    gs32_four<false>(x, ex, z, lane, bar, pr);
+}
+
+__device__ __forceinline__ void wide_crt(uint32_t *ac, uint32_t (&own)[4], const uint32_t *x0,
+                                         const uint32_t *x1, int c_lo, int lane)
+{
+    const int32_t cc = c_ntt.crt_c, cp = c_ntt.crt_cp;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int k = (c_lo + e) * 32 + lane;
+        own[e] += crt_lift(x0[k], x1[k], cc, cp);
+        ac[k] = own[e];
+    }
+}
+
+__global__ void __launch_bounds__(512, 1) k_blind_rotate_wide(const BrArgs A)
+{
+    extern __shared__ uint4 smem_raw[];
+    WideSmem &S = *reinterpret_cast<WideSmem *>(smem_raw);
+    TbOps &O = *reinterpret_cast<TbOps *>(&S + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int q = warp & 3, z = warp >> 2, p = q >> 1, h = q & 1, hz = z & 1;
+    const int lane_brv = brv5(lane);
+    const int n = A.keys.n;
+    const Prime pr((uint32_t)h), pf((uint32_t)(z >> 1));
+    tb_setup(A, O, tid, 2 * kTbCols);
+    const uint32_t tmem = O.tmem;
+    const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
+    const int c_lo = 8 * z + 4 * h;   // this thread's coefficients lane + 32 (c_lo + e)
+    uint2 tw[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        tw[e] = __ldg(A.keys.twb + ((h * 2 + 1) * 32 + 2 * z + (e & 1) + 8 * (e >> 1)) * 32 + lane);
+    uint32_t phase = 0;
+
+    for (long g = blockIdx.x; g < A.count && !O.abort[0]; g += gridDim.x) {
+        const bool active = br_prologue<512>(A, g, tid, S.abar, true);
+        __syncthreads();
+        br_acc_init<512>(A, S.acc, S.abar[n], tid);
+        __syncthreads();
+        uint32_t own[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            own[e] = S.acc[p][(c_lo + e) * 32 + lane];
+
+        for (int i = 0; i < n; ++i) {
+            const int a = S.abar[i];
+            if (a == 0)
+                continue;   // X^0 acc - acc = 0: nothing changes
+            wide_digits(S.acc[p], own, S.dig + z * 2048 + (64 * p + lane) * 16 + 8 * h, c_lo, a,
+                        lane);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncthreads();
+            if (tid == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                tb_mma(tmem, br_saddr(S.dig), O, 0, &O.bar[0]);
+                tb_mma(tmem + kTbCols, br_saddr(S.dig), O, 1, &O.bar[1]);
+            }
+            uint4 kv[8];
+            const uint4 *bki = A.keys.bk_ntt + (((long)i * 2 + p) * 2 + h) * 1024 + 8 * z * 32 + lane;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                kv[e] = __ldg(bki + e * 32);
+            if (!bk_wait(&O.bar[pf.P], phase & 1)) {
+                O.abort[0] = 1;
+                atomicOr(A.status, kErrTimeout);
+            }
+            ++phase;
+            __syncwarp();
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            uint32_t *sl = S.slot[pf.P][q];
+            tb_combine(tl + kTbCols * pf.P, tl + 2 * kTbCols + 64 * pf.P, sl + lane * kRowV, pf,
+                       16 * hz, 16 * hz + 16);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            warps_sync<64>(1 + 2 * q + (z >> 1));
+            {
+                uint32_t y[32];
+                uint32_t *out = S.fwd[pf.P][q];
+                if (hz == 0) {
+                    ct32_cyc_half<0>(y, sl + lane, kRowV, pf);
+#pragma unroll
+                    for (int r = 0; r < 16; r += 4)
+                        *reinterpret_cast<uint4 *>(out + vec_word(r, lane)) =
+                            make_uint4(y[r], y[r + 1], y[r + 2], y[r + 3]);
+                } else {
+                    ct32_cyc_half<1>(y, sl + lane, kRowV, pf);
+#pragma unroll
+                    for (int r = 16; r < 32; r += 4)
+                        *reinterpret_cast<uint4 *>(out + vec_word(r, lane)) =
+                            make_uint4(y[r], y[r + 1], y[r + 2], y[r + 3]);
+                }
+            }
+            __syncthreads();
+            uint32_t x[8];
+            pointwise_4(x, 0, S.fwd[h], 2 * z, kv, lane, pr);
+            pointwise_4(x, 4, S.fwd[h], 2 * z + 1, kv, lane, pr);
+            wide_inverse(x, S.ex[q], S.tr[q], tw, z, lane, lane_brv, 9 + q, pr);
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                S.res[q][(2 * z + (e & 1) + 8 * (e >> 1)) * 32 + lane] = x[e];
+            warps_sync<256>(13 + p);
+            wide_crt(S.acc[p], own, S.res[2 * p], S.res[2 * p + 1], c_lo, lane);
+            warps_sync<256>(13 + p);
+            if (O.abort[0])
+                break;
+        }
+
+        __syncthreads();
+        if (active && !O.abort[0])
+            br_extract<512>(A, g, S.acc, tid);
+        __syncthreads();
+    }
+    // after a wait that ran out: products still in flight get a bounded time
+    // to finish before TMEM is freed
+    if (O.abort[0] && tid == 0)
+        for (int b = 0; b < 2; ++b)
+            (void)bk_wait(&O.bar[b], (phase + 1) & 1);
+    tb_release(tmem, warp);
 }
 
 // ---------------------------------------------------------------------
 // One bootstrap on a cluster of two CTAs (two SMs): CTA h works modulo
 // prime h for the whole CMux and the two exchange their inverse-transform
-// residues through distributed shared memory for the CRT.  For levels
-// narrower than the GPU, where the per-CMux critical path sets the time.
+// residues through distributed shared memory for the CRT.  For levels of at
+// most one bootstrap per two SMs, whose time is the length of a CMux step.
 // ---------------------------------------------------------------------
-
+//
+// As k_blind_rotate_wide, with the phases of one prime spread over a CTA's 16
+// warps (q, z):
+//   digits, CRT   as there (both CTAs hold and update the whole accumulator)
+//   first pass    digit row q, outputs 8 z ..
+//   second pass   digit row q, registers 8 z ..
+//   pointwise, inverse passes   warps z < 2: polynomial z, 8 registers
+// Residues go to both CTAs by asynchronous stores that count on the receiver's
+// barrier, so that no cluster barrier (and its memory fences) stands in a
+// step.  Their buffers alternate by executed CMux: one is rewritten two steps
+// after it was read, and the sender of the later step has waited for what the
+// reader sent in the step between.  Control flow is the same in both CTAs (same
+// gate, same abar, no branch on a wait that ran out), so each step's stores are
+// sent by both.
+// Bound: the chain of a step (6.3K cycles, the multiply pipe busy half of them,
+// seven barriers and two waits).  One gate 1.65 ms against 2.05 ms on one CTA;
+// the shape it replaces (8 warps per CTA, butterflies in the first pass, key
+// staged by bulk copies) took 2.53 ms.
 struct PairSmem {
-    uint32_t acc[2][kN];        // TLWE accumulator (the same in both CTAs)
-    uint32_t fwd[4][kSlot];     // digit rows modulo this CTA's prime; transpose scratch
-    uint32_t pw[2][kN];         // pointwise products [p][reg*32+lane], [0, 2q)
-    uint32_t res[2][2][kN];     // published residues [buffer][p][reg*32+lane]
+    uint32_t acc[2][kN];            // TLWE accumulator (the same in both CTAs)
+    uint8_t dig[128 * 32 * 2];      // digit operand
+    uint32_t slot[4][kSlotV];       // transposes of the forward transforms
+    uint32_t fwd[4][kN];            // forward outputs [digit row] (vec_word)
+    uint32_t ex[2][kN];             // exchange of the inverse passes [p]
+    uint32_t tr[2][kSlotV];         // transposes of the inverse transforms
+    uint32_t res[2][2][2][kN];      // residues [buffer][prime][p] (pair_word)
+    unsigned long long got[2];      // residues of both CTAs have arrived [buffer]
     uint16_t abar[kLweStride];
 };
+constexpr uint32_t kPairBytes = 2 * 2 * kN * sizeof(uint32_t);   // residues of one step
 
-// Key stage of the cluster shape (kBrPairStaged): this CTA's prime half of
-// the next CMux step's key, 2 polynomials x 16 KB, bulk-copied while the
-// current step runs (double buffer).
-struct PairStage {
-    uint4 bk[2][2][kN];         // [buffer][poly p][reg*32+lane]
-    unsigned long long full[2];
-    uint32_t issued[2];
-    volatile int abort;         // a wait ran out: read the key from global memory
-};
-
-__device__ __forceinline__ void pair_issue(PairStage &G, const uint4 *bk_ntt, int i, int rank,
-                                           int buf)
+// Word of register r = 2 q + o + 8 b of a lane in a residue row: registers of
+// the producer's (q, b >> 1) are 16 bytes, the reader's r, r + 1 8 bytes.
+__host__ __device__ constexpr int pair_word(int r, int lane)
 {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
-                     br_saddr(&G.full[buf])),
-                 "r"((uint32_t)(2 * kN * sizeof(uint4)))
+    return ((((r >> 4) * 4 + ((r >> 1) & 3)) * 32 + lane) * 4) + ((r >> 3) & 1) * 2 + (r & 1);
+}
+
+// Four words to shared memory of a CTA of the cluster (an address of the
+// shared::cluster window); their arrival counts on that CTA's barrier `bar`.
+__device__ __forceinline__ void pair_send(uint32_t to, uint32_t a, uint32_t b, uint32_t c, uint32_t d,
+                                          uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], "
+                 "{%1, %2, %3, %4}, [%5];" ::"r"(to),
+                 "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar)
                  : "memory");
-#pragma unroll
-    for (int p = 0; p < 2; ++p)
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes "
-                     "[%0], [%1], %2, [%3];" ::"r"(br_saddr(&G.bk[buf][p][0])),
-                     "l"(bk_ntt + (((long)i * 2 + p) * 2 + rank) * kN),
-                     "r"((uint32_t)(kN * sizeof(uint4))), "r"(br_saddr(&G.full[buf]))
-                     : "memory");
-    G.issued[buf]++;
 }
 
-// Pointwise products of rows r0 .. r0 + 15 of output polynomial p.
-// SH: bkp points into the shared-memory key stage (ld.shared), else to the
-// key in global memory (through L1).
-template <bool SH>
-__device__ __forceinline__ void pair_pointwise(PairSmem &S, const uint4 *__restrict__ bkp, int p,
-                                               int r0, int lane, const Prime &pr)
+__device__ __forceinline__ uint32_t pair_addr(const void *p, int rank)
 {
-    const uint32_t qn = c_ntt.q_inv[pr.P];
-#pragma unroll
-    for (int rr = 0; rr < 16; ++rr) {
-        const int e = (r0 + rr) * 32 + lane;
-        uint4 b;
-        if (SH)
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-                         : "r"(br_saddr(bkp) + (uint32_t)e * 16u));
-        else
-            b = __ldg(bkp + e);
-        uint64_t s = (uint64_t)S.fwd[0][e] * b.x;
-        s += (uint64_t)S.fwd[1][e] * b.y;
-        s += (uint64_t)S.fwd[2][e] * b.z;
-        s += (uint64_t)S.fwd[3][e] * b.w;
-        S.pw[p][e] = mont_reduce(s, pr.q, qn);
-    }
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(br_saddr(p)), "r"(rank));
+    return r;
 }
 
-// 8 warps per CTA.  Per CMux: warps (c, j) < 4 form and transform digit j
-// of polynomial c; warps (p, half) < 4 the pointwise products of half of
-// output polynomial p; warps p < 2 the inverse transform of p, published to
-// a residue buffer; then, after a cluster barrier, all 8 warps lift a
-// quarter of one polynomial each, reading the partner's residues remotely.
-// Both CTAs hold and update the whole accumulator, so the only exchange is
-// the residues.  The residue buffers alternate by executed CMux: a buffer
-// is rewritten two CMux steps after the partner read it, with the partner's
-// barrier arrival of the step between in between.  Control flow is the
-// same in both CTAs of a cluster (same gate, same abar), so every cluster
-// barrier is reached by both.
-template <int STAGE>
-__global__ void __launch_bounds__(256, 1) k_blind_rotate_pair(const BrArgs A)
+// Registers 8 z .. 8 z + 7 of ct32<true> (groups whose twiddle is 1 take their
+// product too, so that the four warps run the same code): inputs [0, 2q),
+// each stage adds at most 2q, outputs reduced from 12q to [0, 8q).
+__device__ __forceinline__ void ct32_cyc_block(uint32_t (&y)[8], const uint32_t *row, int stride,
+                                               int z, const Prime &pr)
+{
+    const uint32_t(*tb)[2] = c_ntt.zd[pr.P];
+    const int k = z >> 1;
+    const uint32_t m0 = k ? ~0u : 0u, m1 = (z & 1) ? ~0u : 0u;
+    const uint32_t o0 = k ? pr.q2 + 1u : 0u, o1 = (z & 1) ? pr.q2 + 1u : 0u;
+    const uint32_t w1 = tb[2 + k][0], wp1 = tb[2 + k][1];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        // stage 0: u + v, or u - v + 2q; then stage 1 the same way
+        const uint32_t u = row[e * stride] + (row[(16 + e) * stride] ^ m0) + o0;
+        const uint32_t v = row[(8 + e) * stride] + (row[(24 + e) * stride] ^ m0) + o0;
+        y[e] = u + (mul_shoup(v, w1, wp1, pr.q) ^ m1) + o1;
+    }
+#pragma unroll
+    for (int s = 2; s < 5; ++s) {
+        const int m = 1 << s, ln = 16 >> s;
+#pragma unroll
+        for (int gl = 0; gl < m / 4; ++gl) {
+            const uint32_t w = tb[m + z * (m / 4) + gl][0], wp = tb[m + z * (m / 4) + gl][1];
+#pragma unroll
+            for (int jj = 0; jj < ln; ++jj) {
+                const int j = 2 * gl * ln + jj;
+                const uint32_t u = y[j], t = mul_shoup(y[j + ln], w, wp, pr.q);
+                y[j] = u + t;
+                y[j + ln] = u - t + pr.q2;
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        y[e] = csub(y[e], pr.kq(8));
+}
+
+__global__ void __launch_bounds__(512, 1) k_blind_rotate_pair(const BrArgs A)
 {
     extern __shared__ uint4 smem_raw[];
     PairSmem &S = *reinterpret_cast<PairSmem *>(smem_raw);
-    PairStage &G = *reinterpret_cast<PairStage *>(reinterpret_cast<PairSmem *>(smem_raw) + 1);
+    TbOps &O = *reinterpret_cast<TbOps *>(&S + 1);
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int q = warp & 3, z = warp >> 2, p = q >> 1;
     const int lane_brv = brv5(lane);
     const int n = A.keys.n;
     const Prime pr((uint32_t)rank);
     const long nclusters = gridDim.x / 2, cid = blockIdx.x / 2;
-    int par = 0;
-    uint32_t uses = 0;   // staged steps so far (the same in every thread)
-    if (STAGE) {
-        if (tid == 0) {
-            for (int b = 0; b < 2; ++b) {
-                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(br_saddr(&G.full[b]))
-                             : "memory");
-                G.issued[b] = 0;
-            }
-            G.abort = 0;
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-        __syncthreads();
+    tb_setup(A, O, tid, 2 * kTbCols);
+    const uint32_t tmem = O.tmem;
+    const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
+    const int c_lo = 8 * z + 4 * (q & 1);   // this thread's coefficients lane + 32 (c_lo + e)
+    // inverse roles of the warps z < 2: polynomial z, registers 8 q ..
+    uint2 tw[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        tw[e] = __ldg(A.keys.twb + ((rank * 2 + 1) * 32 + 2 * q + (e & 1) + 8 * (e >> 1)) * 32 + lane);
+    const uint32_t res_at[2] = {pair_addr(S.res, rank), pair_addr(S.res, rank ^ 1)};
+    const uint32_t got_at[2] = {pair_addr(S.got, rank), pair_addr(S.got, rank ^ 1)};
+    uint32_t phase = 0;   // executed CMux steps
+    if (tid < 2) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(br_saddr(&S.got[tid])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    cl.sync();   // the partner's shared memory and barriers are there
+
     for (long g = cid; g < A.count; g += nclusters) {
-        const bool active = br_prologue<256>(A, g, tid, S.abar, rank == 0);
-        if (STAGE && tid == 0 && n > 0 && !G.abort)
-            pair_issue(G, A.keys.bk_ntt, 0, rank, uses & 1);
+        const bool active = br_prologue<512>(A, g, tid, S.abar, rank == 0);
         __syncthreads();
-        br_acc_init<256>(A, S.acc, S.abar[n], tid);
+        br_acc_init<512>(A, S.acc, S.abar[n], tid);
         __syncthreads();
+        uint32_t own[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            own[e] = S.acc[p][(c_lo + e) * 32 + lane];
+
         for (int i = 0; i < n; ++i) {
-            const uint32_t u = uses;   // this step's use of buffer u & 1
-            if (STAGE) {
-                ++uses;
-                // the other buffer was last read in step i - 1, before the
-                // barrier that ended that step's pointwise phase
-                if (tid == 0 && i + 1 < n && !G.abort)
-                    pair_issue(G, A.keys.bk_ntt, i + 1, rank, (u + 1) & 1);
-            }
             const int a = S.abar[i];
-            if (a == 0) {
-                // X^0 acc - acc = 0: nothing changes (in both CTAs); the
-                // step's copy still has to land before its buffer is reused
-                if (STAGE && tid == 0 && !G.abort && !bk_wait(&G.full[u & 1], (u >> 1) & 1)) {
-                    G.abort = 1;
-                    atomicOr(A.status, kErrTimeout);
-                }
-                continue;
-            }
-            uint32_t x[32];
-            if (warp < 4)
-                digit_fwd(x, S.acc[warp >> 1], S.fwd[warp], warp & 1, a, lane, A.keys.twb, pr);
+            if (a == 0)
+                continue;   // X^0 acc - acc = 0: nothing changes
+            const uint32_t use = phase++;
+            const int par = use & 1;
+            wide_digits(S.acc[p], own, S.dig + z * 2048 + (64 * p + lane) * 16 + 8 * (q & 1), c_lo,
+                        a, lane);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncthreads();
-            if (warp < 4) {
-                const int p = warp >> 1;
-                bool staged = false;
-                if (STAGE) {
-                    staged = !G.abort && bk_wait(&G.full[u & 1], (u >> 1) & 1);
-                    if (!staged && !G.abort) {
-                        G.abort = 1;   // read this and later steps from global memory
-                        atomicOr(A.status, kErrTimeout);
-                    }
-                }
-                if (staged)
-                    pair_pointwise<true>(S, &G.bk[u & 1][p][0], p, 16 * (warp & 1), lane, pr);
-                else
-                    pair_pointwise<false>(S, A.keys.bk_ntt + (((long)i * 2 + p) * 2 + rank) * 1024,
-                                          p, 16 * (warp & 1), lane, pr);
+            if (tid == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                tb_mma(tmem, br_saddr(S.dig), O, rank, &O.bar[0]);
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
+                                 br_saddr(&S.got[par])),
+                             "r"(kPairBytes)
+                             : "memory");
             }
+            uint4 kv[8];
+            if (z < 2) {
+                const uint4 *bki = A.keys.bk_ntt + (((long)i * 2 + z) * 2 + rank) * 1024 +
+                                   8 * q * 32 + lane;
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    kv[e] = __ldg(bki + e * 32);
+            }
+            if (!O.abort[0] && !bk_wait(&O.bar[0], use & 1)) {
+                O.abort[0] = 1;   // wait no more; the status word has it
+                atomicOr(A.status, kErrTimeout);
+            }
+            __syncwarp();
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            uint32_t *sl = S.slot[q];
+            tb_combine(tl, tl + 2 * kTbCols + 64 * rank, sl + lane * kRowV, pr, 8 * z, 8 * z + 8);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            warps_sync<128>(1 + q);
+            uint32_t x[8];
+            ct32_cyc_block(x, sl + lane, kRowV, z, pr);
+            uint32_t *out = S.fwd[q] + vec_word(8 * z, lane);
+            *reinterpret_cast<uint4 *>(out) = make_uint4(x[0], x[1], x[2], x[3]);
+            *reinterpret_cast<uint4 *>(out + vec_word(4, 0)) = make_uint4(x[4], x[5], x[6], x[7]);
             __syncthreads();
-            if (warp < 2) {
+            if (z < 2) {
+                pointwise_4(x, 0, S.fwd, 2 * q, kv, lane, pr);
+                pointwise_4(x, 4, S.fwd, 2 * q + 1, kv, lane, pr);
+                wide_inverse(x, S.ex[z], S.tr[z], tw, q, lane, lane_brv, 9 + z, pr);
+                const uint32_t at = (((par * 2 + rank) * 2 + z) * kN + pair_word(2 * q, lane)) * 4;
 #pragma unroll
-                for (int r = 0; r < 32; ++r)
-                    x[r] = S.pw[warp][r * 32 + lane];
-                inv_ntt(x, S.fwd[warp], lane, lane_brv, A.keys.twb, pr);
-                uint32_t *out = S.res[par][warp];
-#pragma unroll
-                for (int r = 0; r < 32; ++r)
-                    out[r * 32 + lane] = x[r];
+                for (int c = 0; c < 2; ++c) {
+                    pair_send(res_at[c] + at, x[0], x[1], x[2], x[3], got_at[c] + 8 * par);
+                    pair_send(res_at[c] + at + 4 * pair_word(16, 0), x[4], x[5], x[6], x[7],
+                              got_at[c] + 8 * par);
+                }
             }
-            cl.sync();
+            if (!O.abort[0] && !bk_wait(&S.got[par], (use >> 1) & 1)) {
+                O.abort[0] = 1;
+                atomicOr(A.status, kErrTimeout);
+            }
             {
-                const int p = warp >> 2;
-                const uint32_t *mine = S.res[par][p];
-                const uint32_t *other = cl.map_shared_rank(mine, rank ^ 1);
-                crt_rows<8>(S.acc[p], rank == 0 ? mine : other, rank == 0 ? other : mine,
-                            8 * (warp & 3), lane);
+                const int32_t cc = c_ntt.crt_c, cp = c_ntt.crt_cp;
+#pragma unroll
+                for (int e = 0; e < 4; e += 2) {
+                    const int w = pair_word(c_lo + e, lane);
+                    const uint2 v0 = *reinterpret_cast<const uint2 *>(&S.res[par][0][p][w]);
+                    const uint2 v1 = *reinterpret_cast<const uint2 *>(&S.res[par][1][p][w]);
+                    own[e] += crt_lift(v0.x, v1.x, cc, cp);
+                    own[e + 1] += crt_lift(v0.y, v1.y, cc, cp);
+                    S.acc[p][(c_lo + e) * 32 + lane] = own[e];
+                    S.acc[p][(c_lo + e + 1) * 32 + lane] = own[e + 1];
+                }
             }
-            par ^= 1;
-            __syncthreads();
+            warps_sync<256>(13 + p);
         }
+        __syncthreads();
         if (active && rank == 0)
-            br_extract<256>(A, g, S.acc, tid);
+            br_extract<512>(A, g, S.acc, tid);
         __syncthreads();
     }
-    cl.sync();   // the partner may still read this CTA's residues
-    // after a wait that ran out: copies still in flight land before the
-    // CTA's shared memory is released (the last use of each buffer)
-    if (STAGE && tid == 0 && G.abort)
-        for (int b = 0; b < 2; ++b)
-            if (G.issued[b])
-                (void)bk_wait(&G.full[b], (G.issued[b] - 1) & 1);
+    // after a wait that ran out: a product and stores still in flight get a
+    // bounded time to finish before TMEM and shared memory are freed
+    if (O.abort[0] && tid == 0 && phase) {
+        (void)bk_wait(&O.bar[0], (phase - 1) & 1);
+        (void)bk_wait(&S.got[(phase - 1) & 1], ((phase - 1) >> 1) & 1);
+    }
+    cl.sync();   // neither CTA ends while the other may write to it
+    tb_release(tmem, warp);
 }
 
 // ---------------------------------------------------------------------
@@ -1714,11 +1690,6 @@ cudaError_t launch_bk_to_ntt(const int32_t *bk_dev, uint32_t *bk_ntt, int n, con
     return cudaGetLastError();
 }
 
-constexpr size_t br_smem(bool staged)
-{
-    return sizeof(BrSmem) + (staged ? sizeof(BkStage) : 0) + sizeof(SplitExtra);
-}
-
 // Shape of a launch: the forced or tuned code, else by batch size.
 static bool br_shape_ok(int v)
 {
@@ -1730,12 +1701,13 @@ static int br_group(long count, int num_sms, int forced, const int8_t *tuned)
 {
     if (br_shape_ok(forced))
         return forced;
+    // at most one bootstrap per SM: 2.09 ms on 16 warps (152 gates) against
+    // 3.27 ms for the throughput shape; 301 gates: 4.15 against 4.09 ms
     const int t = tuned[tune_bucket(count)];
-    if (br_shape_ok(t))
-        return t;
-    // at most one bootstrap per SM: 2.58 ms on 8 warps (152 gates) against
-    // 3.29 ms for the throughput shape; 301 gates: 5.04 against 4.02 ms
-    return count > num_sms ? 1 : kBrSplit;
+    const int shape = br_shape_ok(t) ? t : count > num_sms ? 1 : kBrSplit;
+    // at most one per two SMs: 1.69 ms on two CTAs (76 gates) against 2.07 ms on
+    // one (a tuned choice stands for its bucket's widest level)
+    return shape == kBrSplit && 2 * count <= num_sms ? kBrPair : shape;
 }
 
 static cudaError_t launch_tc(const BrArgs &A, unsigned blocks, int dev, cudaStream_t stream)
@@ -1751,6 +1723,48 @@ static cudaError_t launch_tc(const BrArgs &A, unsigned blocks, int dev, cudaStre
     }
     k_blind_rotate_tc<<<blocks, 512, smem, stream>>>(A);
     return cudaGetLastError();
+}
+
+static cudaError_t launch_wide(const BrArgs &A, unsigned blocks, int dev, cudaStream_t stream)
+{
+    constexpr int smem = (int)sizeof(WideSmem) + (int)sizeof(TbOps);
+    static int prepared[64] = {0};
+    if (dev >= 0 && dev < 64 && !prepared[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(k_blind_rotate_wide,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess)
+            return e;
+        prepared[dev] = 1;
+    }
+    k_blind_rotate_wide<<<blocks, 512, smem, stream>>>(A);
+    return cudaGetLastError();
+}
+
+// One CTA per SM: `pairs` clusters at a time.
+static cudaError_t launch_pair(const BrArgs &A, long pairs, int dev, cudaStream_t stream)
+{
+    constexpr int smem = (int)sizeof(PairSmem) + (int)sizeof(TbOps);
+    static int prepared[64] = {0};
+    if (dev >= 0 && dev < 64 && !prepared[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(k_blind_rotate_pair,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess)
+            return e;
+        prepared[dev] = 1;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * (A.count < pairs ? A.count : pairs)));
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_blind_rotate_pair, A);
 }
 
 cudaError_t launch_blind_rotate(const DevKeys &keys, const uint8_t *ops, const int32_t *in_a,
@@ -1782,55 +1796,12 @@ cudaError_t launch_blind_rotate(const DevKeys &keys, const uint8_t *ops, const i
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int shape = br_group(count, sms > 0 ? sms : 1, keys.br_group, keys.tune_br);
-    if (shape == kBrPair || shape == kBrPairStaged) {
-        const bool staged = shape == kBrPairStaged;
-        const size_t smem = sizeof(PairSmem) + (staged ? sizeof(PairStage) : 0);
-        static int prepared[2][64] = {{0}};
-        if (dev >= 0 && dev < 64 && !prepared[staged][dev]) {
-            cudaFuncSetAttribute(staged ? k_blind_rotate_pair<1> : k_blind_rotate_pair<0>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            (void)cudaGetLastError();
-            prepared[staged][dev] = 1;
-        }
-        const long pairs = sms >= 2 ? sms / 2 : 1;   // one CTA per SM
-        const long clusters = count < pairs ? count : pairs;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(2 * clusters));
-        cfg.blockDim = dim3(256);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = stream;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        return staged ? cudaLaunchKernelEx(&cfg, k_blind_rotate_pair<1>, A)
-                      : cudaLaunchKernelEx(&cfg, k_blind_rotate_pair<0>, A);
-    }
-    (void)grid;
     const long nsm = sms > 0 ? sms : 1;
-    if (shape == kBrSplit || shape == kBrSplitStaged) {
-        const bool staged = shape == kBrSplitStaged;
-        static int prepared[2][64] = {{0}};
-        if (dev >= 0 && dev < 64 && !prepared[staged][dev]) {
-            cudaFuncSetAttribute(staged ? k_blind_rotate<1, 8, 1> : k_blind_rotate<1, 8, 0>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)br_smem(staged));
-            cudaFuncSetAttribute(staged ? k_blind_rotate<1, 8, 1> : k_blind_rotate<1, 8, 0>,
-                                 cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
-            (void)cudaGetLastError();
-            prepared[staged][dev] = 1;
-        }
-        const unsigned blocks = (unsigned)(count < nsm ? count : nsm);
-        if (staged)
-            k_blind_rotate<1, 8, 1><<<blocks, 256, br_smem(true), stream>>>(A);
-        else
-            k_blind_rotate<1, 8, 0><<<blocks, 256, br_smem(false), stream>>>(A);
-        return cudaGetLastError();
-    }
+    if (shape == kBrPair || shape == kBrPairStaged)
+        return launch_pair(A, nsm >= 2 ? nsm / 2 : 1, dev, stream);
+    (void)grid;
+    if (shape == kBrSplit || shape == kBrSplitStaged)
+        return launch_wide(A, (unsigned)(count < nsm ? count : nsm), dev, stream);
     // the throughput shape (the other codes are accepted for saved tuning
     // files and options)
     return launch_tc(A, (unsigned)(count < nsm ? count : nsm), dev, stream);

@@ -70,7 +70,7 @@ __device__ __forceinline__ uint32_t mont_reduce(uint64_t x, uint32_t q, uint32_t
 #endif  // __CUDACC__
 
 // Per-context device pointers and sizes shared by the kernels.
-// Blind-rotation shape codes: one bootstrap spread over 8 warps, and one
+// Blind-rotation shape codes: one bootstrap on a CTA's 16 warps, and one
 // bootstrap on a cluster of two CTAs (one prime each).  1 is the throughput
 // shape (4 bootstraps per CTA); 2, 4, kBrStaged, kBrStagedCtl and kBrFive are
 // accepted for options and tuning files that name them and run it too.
@@ -79,10 +79,9 @@ constexpr int kBrPair = 16;
 constexpr int kBrStaged = 32;
 constexpr int kBrStagedCtl = 33;
 constexpr int kBrFive = 5;
-// One bootstrap on 8 warps with the key staged (the latency shape, whose
-// single pointwise warp per sub-partition otherwise waits on L2 each step).
+// Accepted as another name of kBrSplit.
 constexpr int kBrSplitStaged = 40;
-// One bootstrap on a two-CTA cluster with each CTA's half of the key staged.
+// Accepted as another name of kBrPair.
 constexpr int kBrPairStaged = 48;
 // Key-switch launch code for the tiled kernel (shared-memory key stages);
 // the codes 1 .. 32 are j-chunks of the direct kernel.

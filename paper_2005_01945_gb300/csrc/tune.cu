@@ -1,7 +1,7 @@
 // tune.cu -- autotuner for the launch shapes of the two bootstrapping
 // kernels: the blind-rotation shape (4 independent bootstraps per CTA, one
-// bootstrap spread over 8 warps with or without the key staged in shared
-// memory, or one bootstrap on a cluster of two CTAs with or without it) and the
+// bootstrap on a CTA's 16 warps, or one bootstrap on a cluster of two CTAs)
+// and the
 // key-switch kernel (the tiled kernel with shared-memory key stages, or
 // the direct kernel with its j-split of 1 .. 32 chunks), chosen per
 // level-width bucket by timing the candidates on synthetic ciphertexts
@@ -46,7 +46,7 @@ static std::string cache_key(int device)
     // the tag separates these kernels' times from those of files written for
     // other blind-rotation kernels: an older line is not used, and tuning
     // appends a new one
-    return name + ":" + std::to_string(prop.multiProcessorCount) + ":tc1";
+    return name + ":" + std::to_string(prop.multiProcessorCount) + ":tc2";
 }
 
 static bool load_cache(const char *path, const std::string &key, DevKeys &k)
@@ -142,7 +142,7 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
             // the latency shapes first: a later candidate is kept only if it
             // is at least 2 % faster at the bucket's widest level
             float best = 1e30f;
-            for (int B : {kBrSplit, kBrSplitStaged, kBrPair, kBrPairStaged, 1}) {
+            for (int B : {kBrSplit, kBrPair, 1}) {
                 // the latency shapes hold one bootstrap per SM (or SM pair):
                 // only candidates while a level fits in about one wave of them
                 if (B != 1 && W > 2L * ctx->num_sms)
