@@ -49,6 +49,10 @@ struct NttConst {
     uint32_t zd[2][32][2];   // forward stage D: cyclic size-32 twiddles
     uint32_t iza[2][32][2];  // inverse of stage A
     uint32_t izd[2][32][2];  // inverse of stage D
+    // signed transforms, centred (w, round(2^32 w / q)): stage D twiddles, the
+    // inverse's by position ln + j, and the last pass's w64^-r
+    int32_t zs[2][32][2], izs[2][32][2], post[2][32][2];
+    int32_t one[2];          // round(2^32 / q)
     uint32_t q_inv[2];       // q^-1 mod 2^32
     int32_t crt_c, crt_cp;   // q0^-1 mod q1, centred, and round(2^32 crt_c / q1)
     uint32_t bk_scale[2][2]; // 2^32 N^-1 mod q and companion
@@ -83,11 +87,8 @@ struct Prime {
 // in the same order as the code and places the fewest reductions that keep
 // every sum below thr q (<= kLazyMax q < 2^32), and the final outputs below
 // fin q:
-//  * CT butterfly (u, v) -> (u + t, u - t + K' q), t = v (trivial twiddle)
-//    or Shoup(v) in [0, 2q), K' >= bound(t) the smallest power of two;
-//  * GS butterfly (u, v) -> (u + v, d), d = u - v + K' q (K' >= bound(v)),
-//    passed on as is (trivial twiddle) or as Shoup(d) in [0, 2q).
-// The reduction is applied to the larger operand until the sum fits.
+// CT butterfly (u, v) -> (u + t, u - t + K' q), t = v (trivial twiddle) or
+// Shoup(v) in [0, 2q), K' >= bound(t) the smallest power of two.  The reduction is applied to the larger operand until the sum fits.
 // ---------------------------------------------------------------------
 struct LazyStep {
     uint8_t ru[4], nru;     // csub multiples K applied to u, in order
@@ -119,7 +120,7 @@ __host__ __device__ constexpr int lazy_step(int b, int &K)
     return K > b - K ? K : b - K;
 }
 
-__host__ __device__ constexpr LazyPlan make_lazy_plan(bool ct, bool trivial_first, int in_b, int thr, int fin)
+__host__ __device__ constexpr LazyPlan make_lazy_plan(bool trivial_first, int in_b, int thr, int fin)
 {
     LazyPlan P{};
     P.ok = true;
@@ -127,7 +128,7 @@ __host__ __device__ constexpr LazyPlan make_lazy_plan(bool ct, bool trivial_firs
     for (int i = 0; i < 32; ++i)
         b[i] = in_b;
     for (int it = 0; it < 5; ++it) {
-        const int s = ct ? it : 4 - it;
+        const int s = it;
         const int m = 1 << s, ln = 16 >> s;
         for (int g = 0; g < m; ++g) {
             const bool triv = trivial_first && g == 0;
@@ -136,11 +137,11 @@ __host__ __device__ constexpr LazyPlan make_lazy_plan(bool ct, bool trivial_firs
                 LazyStep &L = P.st[s][g * ln + jj];
                 int bu = b[j], bv = b[j + ln];
                 for (int guard = 0; guard < 8; ++guard) {
-                    const int bt = (ct && !triv) ? 2 : bv;
+                    const int bt = triv ? bv : 2;
                     if (bu + bt <= thr && bu + lazy_off(bt) <= kLazyMax)
                         break;
                     int K = 0;
-                    if ((!ct || triv) && bt >= bu) {
+                    if (triv && bt >= bu) {
                         const int nb = lazy_step(bv, K);
                         if (nb == bv || L.nrv == 4) { P.ok = false; break; }
                         L.rv[L.nrv++] = (uint8_t)K;
@@ -152,16 +153,11 @@ __host__ __device__ constexpr LazyPlan make_lazy_plan(bool ct, bool trivial_firs
                         bu = nb;
                     }
                 }
-                const int bt = (ct && !triv) ? 2 : bv;
+                const int bt = triv ? bv : 2;
                 L.off = (uint8_t)lazy_off(bt);
                 P.reductions += L.nru + L.nrv;
-                if (ct) {
-                    b[j] = bu + bt;
-                    b[j + ln] = bu + L.off;
-                } else {
-                    b[j] = bu + bv;
-                    b[j + ln] = triv ? bu + L.off : 2;
-                }
+                b[j] = bu + bt;
+                b[j + ln] = bu + L.off;
                 if (b[j] > kLazyMax || b[j + ln] > kLazyMax)
                     P.ok = false;
             }
@@ -180,20 +176,14 @@ __host__ __device__ constexpr LazyPlan make_lazy_plan(bool ct, bool trivial_firs
     return P;
 }
 
-// Forward passes: stage A (negacyclic twiddles, inputs [0, 2q), outputs
-// < 12q, no reduction needed) and stage D (cyclic, the first twiddle of
-// every level is 1; inputs [0, 2q), outputs [0, 8q) for the pointwise
-// products).  Inverse passes: stage D' (cyclic GS, inputs [0, 2q) from the
-// pointwise Montgomery step, outputs < 32q into the Shoup twiddle) and
-// stage A' (negacyclic GS, inputs [0, 2q), outputs [0, 8q) for crt_lift).  The
-// thresholds are the ones that need the fewest reductions.
-constexpr LazyPlan kPlanFwdA = make_lazy_plan(true, false, 2, 12, kLazyMax);
-constexpr LazyPlan kPlanFwdD = make_lazy_plan(true, true, 2, 8, 8);
-constexpr LazyPlan kPlanInvD = make_lazy_plan(false, true, 2, kLazyMax, kLazyMax);
-constexpr LazyPlan kPlanInvA = make_lazy_plan(false, false, 2, kLazyMax, 8);
-static_assert(kPlanFwdA.ok && kPlanFwdD.ok && kPlanInvD.ok && kPlanInvA.ok, "lazy plan");
-static_assert(kPlanFwdA.reductions == 0 && kPlanFwdD.reductions == 33 &&
-              kPlanInvD.reductions == 4 && kPlanInvA.reductions == 8, "lazy plan size");
+// Stage A (negacyclic twiddles, inputs [0, 2q), outputs < 12q, no reduction
+// needed) and stage D (cyclic, the first twiddle of every level is 1; inputs
+// [0, 2q), outputs [0, 8q) for the pointwise products).  The thresholds are the
+// ones that need the fewest reductions.
+constexpr LazyPlan kPlanFwdA = make_lazy_plan(false, 2, 12, kLazyMax);
+constexpr LazyPlan kPlanFwdD = make_lazy_plan(true, 2, 8, 8);
+static_assert(kPlanFwdA.ok && kPlanFwdD.ok, "lazy plan");
+static_assert(kPlanFwdA.reductions == 0 && kPlanFwdD.reductions == 33, "lazy plan size");
 
 __device__ __forceinline__ uint32_t lazy_reduce_n(uint32_t x, const uint8_t (&ks)[4], int n,
                                                   const Prime &pr)
@@ -236,35 +226,118 @@ __device__ __forceinline__ void ct32(uint32_t (&x)[32], const Prime &pr)
         x[r] = lazy_reduce_n(x[r], PL.fin[r], PL.nfin[r], pr);
 }
 
-// Inverse (Gentleman-Sande) of ct32, reductions by plan; the result is 32
-// times the inverse transform.
-template <bool CYC>
-__device__ __forceinline__ void gs32(uint32_t (&x)[32], const Prime &pr)
+// ---------------------------------------------------------------------
+// Signed passes (k_blind_rotate_tc).  With centred twiddles (|w| <= q / 2, w' =
+// round(2^32 w / q)) a Shoup product of a signed x, |x| <= a q <= 16 q, lies in
+// [-a / 64, 1 + a / 64] q.  A decimation-in-time butterfly then takes four
+// instructions,
+//     hi = mulhi(x, w');  s = (x w + u) - hi q;  d = 2 u - s,
+// where an unsigned one takes five (a sum, and a difference with an offset),
+// and bounds grow by one q a stage except along the twiddles 1, so that a
+// forward pass needs 7 reductions instead of 33.  (The sum and difference of a
+// product formed first: 608 gates 5.93 ms, so 5.56.)
+// ---------------------------------------------------------------------
+struct SignedPlan {
+    bool ru[5][16], rv[5][16];   // reduce u / v of a butterfly first
+    bool fin[32];                // reduce the output
+    int reductions;
+    bool ok;
+};
+
+// Intervals in units of q / 64: inputs [lo, hi], no sum beyond thr, outputs
+// within +-out.  dit: distances 1 .. 16, twiddle 1 at j = 0; else distances
+// 16 .. 1, twiddle 1 in group 0.
+__host__ __device__ constexpr SignedPlan make_signed_plan(bool dit, int lo0, int hi0, int thr, int out)
 {
-    constexpr LazyPlan PL = CYC ? kPlanInvD : kPlanInvA;
+    SignedPlan P{};
+    P.ok = true;
+    int lo[32] = {}, hi[32] = {};
+    for (int i = 0; i < 32; ++i)
+        lo[i] = lo0, hi[i] = hi0;
+    for (int s = 0; s < 5; ++s) {
+        const int ln = dit ? 1 << s : 16 >> s;
+        for (int b = 0; b < 16; ++b) {
+            const int g = b / ln, j = b % ln, iu = 2 * g * ln + j, iv = iu + ln;
+            const bool triv = dit ? j == 0 : g == 0;
+            for (int guard = 0; guard < 3; ++guard) {
+                const int av = lo[iv] < -hi[iv] ? -lo[iv] : hi[iv], au = lo[iu] < -hi[iu] ? -lo[iu] : hi[iu];
+                const int t = triv ? av : 64 + (av + 63) / 64;
+                if (au + t <= thr)
+                    break;
+                const bool v = triv && av >= au;
+                const int i = v ? iv : iu, a = ((v ? av : au) + 63) / 64;
+                (v ? P.rv : P.ru)[s][b] = true;
+                lo[i] = -a, hi[i] = 64 + a;
+                ++P.reductions;
+                P.ok = P.ok && guard < 2;
+            }
+            const int a = ((lo[iv] < -hi[iv] ? -lo[iv] : hi[iv]) + 63) / 64;
+            const int tl = triv ? lo[iv] : -a, th = triv ? hi[iv] : 64 + a;
+            const int ul = lo[iu], uh = hi[iu];
+            lo[iu] = ul + tl, hi[iu] = uh + th;
+            lo[iv] = ul - th, hi[iv] = uh - tl;
+        }
+    }
+    for (int i = 0; i < 32; ++i) {
+        P.fin[i] = lo[i] < -out || hi[i] > out;
+        P.reductions += P.fin[i];
+    }
+    return P;
+}
+
+constexpr int kSignedMax = 15 * 64;   // 15 q < 2^31
+// Forward second pass: inputs below q (1 + 4 / 32), outputs within 8q for the
+// pointwise products.  Inverse passes: inputs from the pointwise step
+// (-q, q), then from the twiddle; outputs into a Shoup product.
+constexpr SignedPlan kSignedFwd = make_signed_plan(false, 0, 72, kSignedMax, 8 * 64);
+constexpr SignedPlan kSignedInvD = make_signed_plan(true, -64, 64, kSignedMax, kSignedMax);
+constexpr SignedPlan kSignedInvA = make_signed_plan(true, -16, 80, kSignedMax, kSignedMax);
+static_assert(kSignedFwd.ok && kSignedInvD.ok && kSignedInvA.ok, "signed plan");
+static_assert(kSignedFwd.reductions == 7 && kSignedInvD.reductions == 3 &&
+              kSignedInvA.reductions == 3, "signed plan size");
+
+__device__ __forceinline__ int32_t mul_signed(int32_t x, int32_t w, int32_t wp, int32_t q)
+{
+    return (int32_t)((uint32_t)x * (uint32_t)w - (uint32_t)__mulhi(x, wp) * (uint32_t)q);
+}
+
+__device__ __forceinline__ int32_t reduce_signed(int32_t x, const Prime &pr)
+{
+    return (int32_t)((uint32_t)x - (uint32_t)__mulhi(x, c_ntt.one[pr.P]) * pr.q);
+}
+
+// DIT false: ct32<true>; true: 32 times its inverse, input in ct32's output order.
+template <bool DIT, bool LAST = false>
+__device__ __forceinline__ void pass32_signed(int32_t (&x)[32], const Prime &pr)
+{
+    constexpr SignedPlan PL = !DIT ? kSignedFwd : LAST ? kSignedInvA : kSignedInvD;
+    const int32_t(*tb)[2] = DIT ? c_ntt.izs[pr.P] : c_ntt.zs[pr.P];
 #pragma unroll
-    for (int s = 4; s >= 0; --s) {
-        const int m = 1 << s, ln = 16 >> s;
+    for (int s = 0; s < 5; ++s) {
+        const int ln = DIT ? 1 << s : 16 >> s;
 #pragma unroll
-        for (int g = 0; g < m; ++g) {
-            const uint32_t(*tb)[32][2] = CYC ? c_ntt.izd : c_ntt.iza;
-            const uint32_t w = tb[pr.P][m + g][0];
-            const uint32_t wp = tb[pr.P][m + g][1];
-#pragma unroll
-            for (int jj = 0; jj < ln; ++jj) {
-                const int j = 2 * g * ln + jj;
-                const LazyStep &L = PL.st[s][g * ln + jj];
-                const uint32_t u = lazy_reduce_n(x[j], L.ru, L.nru, pr);
-                const uint32_t v = lazy_reduce_n(x[j + ln], L.rv, L.nrv, pr);
-                x[j] = u + v;
-                const uint32_t d = u - v + pr.kq(L.off);
-                x[j + ln] = (CYC && g == 0) ? d : mul_shoup(d, w, wp, pr.q);
+        for (int b = 0; b < 16; ++b) {
+            const int g = b / ln, j = b % ln, iu = 2 * g * ln + j, iv = iu + ln;
+            const bool triv = DIT ? j == 0 : g == 0;
+            const int32_t u = PL.ru[s][b] ? reduce_signed(x[iu], pr) : x[iu];
+            const int32_t v = PL.rv[s][b] ? reduce_signed(x[iv], pr) : x[iv];
+            if (triv) {
+                x[iu] = u + v;
+                x[iv] = u - v;
+            } else {
+                const int k = DIT ? ln + j : (1 << s) + g;
+                const int32_t hi = __mulhi(v, tb[k][1]);
+                const uint32_t sum = ((uint32_t)v * (uint32_t)tb[k][0] + (uint32_t)u) -
+                                     (uint32_t)hi * pr.q;
+                x[iu] = (int32_t)sum;
+                x[iv] = (int32_t)((uint32_t)u + (uint32_t)u - sum);
             }
         }
     }
 #pragma unroll
     for (int r = 0; r < 32; ++r)
-        x[r] = lazy_reduce_n(x[r], PL.fin[r], PL.nfin[r], pr);
+        if (PL.fin[r])
+            x[r] = reduce_signed(x[r], pr);
 }
 
 // Forward negacyclic NTT of one polynomial held by one warp.
@@ -326,7 +399,7 @@ __global__ void __launch_bounds__(128) k_bk_to_ntt(const int32_t *__restrict__ b
     for (int k = 0; k < 32; ++k) {
         uint32_t v = x[k] % q;                         // [0, 8q) -> [0, q)
         v = csub(mul_shoup(v, sc, scp, q), q);        // * 2^32 N^-1, in [0, q)
-        dst[k * 32 * 4] = v;
+        dst[k * 32 * 4] = v > q / 2 ? v - q : v;       // centred
     }
 }
 
@@ -379,7 +452,7 @@ __device__ __forceinline__ bool bk_wait(unsigned long long *bar, uint32_t parity
     return false;
 }
 
-// Phase 4: CRT of (v0 mod q0, v1 mod q1), any representatives in [0, 8q), to
+// Phase 4: CRT of (v0 mod q0, v1 mod q1), any representatives in [-8q, 8q), to
 // the centred integer, mod 2^32.  Garner: the exact coefficient S satisfies
 // |S| <= 4 N 2^9 2^31 = 2^52, so u = (S - v0) / q0 is an integer of magnitude
 // at most 2^25 + 8, about q1 / 4, and u = (v1 - v0) q0^-1 mod q1.  The
@@ -529,6 +602,7 @@ __device__ __forceinline__ void br_extract(const BrArgs &A, long g, const uint32
 // pass takes nothing from the load/store pipe but its result's transpose.
 constexpr int kTbCols = 96;                        // 32 outputs x 3 limbs of one prime
 constexpr uint32_t kTbOpBytes = kTbCols * 32 * 2;  // constant operand of one prime, 6 KB
+static_assert(2 * kTbOpBytes + 2 * 1024 * sizeof(int2) == kTbDevBytes, "operand buffer");
 constexpr int kTbTw = 4 * kTbCols;                 // TMEM column of the twiddles
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
@@ -560,41 +634,54 @@ struct TbOps {                  // one CTA
     volatile int abort[4];      // a wait of the bootstrap ran out
 };
 
-// Inverse transform with vector-ordered input rows (see inv_ntt): the
-// transpose is written by words and read as 16-byte vectors.
-__device__ __forceinline__ void inv_ntt_v(uint32_t (&x)[32], uint32_t *sbuf, int lane, int lane_brv,
-                                          const uint2 *__restrict__ twb, const Prime &pr)
+// Barrier of the 128 threads of bootstrap slot `bi`.
+__device__ __forceinline__ void boot_sync(int bi)
 {
-    gs32<true>(x, pr);
-    const uint2 *tw = twb + (pr.P * 2 + 1) * 1024 + lane;
-#pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        const uint2 t = __ldg(tw + r * 32);
-        x[r] = mul_shoup(x[r], t.x, t.y, pr.q);
-    }
+    asm volatile("bar.sync %0, 128;" ::"r"(1 + bi) : "memory");
+}
+
+// Inverse transform up to the factor N, signed: lane k1, register k2 (bit-
+// reversed), values in (-q, q), to lane i1, register i2, residues in
+// [-q / 4, 5 q / 4].  The transpose is written by words and read as 16-byte
+// vectors.  The last pass is the cyclic one and a product by w64^-r behind it:
+// 49 + 31 products in four-instruction butterflies and alone, where the
+// negacyclic pass has 80 in five-instruction ones.
+__device__ __forceinline__ void inv_ntt_v(int32_t (&x)[32], uint32_t *sbuf, int lane, int lane_brv,
+                                          const int2 *__restrict__ tw, const Prime &pr, int bi)
+{
+    pass32_signed<true>(x, pr);
+    boot_sync(bi);   // the other warps have read the row that is the scratch
     uint32_t *wr = sbuf + lane_brv, *rd = sbuf + lane * kRowV;
+    // products and stores alternate (all stores behind the products: 608 gates
+    // 6.07 ms, so 5.56)
 #pragma unroll
-    for (int r = 0; r < 32; ++r)
-        wr[r * kRowV] = x[r];          // lane k1, i1 = r -> slot[i1][brv5(k1)]
+    for (int r = 0; r < 32; ++r) {     // lane k1, i1 = r -> slot[i1][brv5(k1)]
+        const int2 t = __ldg(tw + r * 32);
+        wr[r * kRowV] = (uint32_t)mul_signed(x[r], t.x, t.y, pr.q);
+    }
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < 32; r += 4) {  // lane i1 reads slot[i1][r ..]
-        const uint4 v = *reinterpret_cast<const uint4 *>(rd + r);
+        const int4 v = *reinterpret_cast<const int4 *>(rd + r);
         x[r] = v.x;
         x[r + 1] = v.y;
         x[r + 2] = v.z;
         x[r + 3] = v.w;
     }
     __syncwarp();
-    gs32<false>(x, pr);
+    pass32_signed<true, true>(x, pr);
+    x[0] = reduce_signed(x[0], pr);
+#pragma unroll
+    for (int r = 1; r < 32; ++r)
+        x[r] = mul_signed(x[r], c_ntt.post[pr.P][r][0], c_ntt.post[pr.P][r][1], pr.q);
 }
 
-__device__ __forceinline__ void store_vec(uint32_t *row, const uint32_t (&x)[32], int lane)
+__device__ __forceinline__ void store_vec(uint32_t *row, const int32_t (&x)[32], int lane)
 {
 #pragma unroll
     for (int r = 0; r < 32; r += 4)
-        *reinterpret_cast<uint4 *>(row + vec_word(r, lane)) =
-            make_uint4(x[r], x[r + 1], x[r + 2], x[r + 3]);
+        *reinterpret_cast<int4 *>(row + vec_word(r, lane)) =
+            make_int4(x[r], x[r + 1], x[r + 2], x[r + 3]);
 }
 
 // Key vectors of registers 4 g .. 4 g + 3.
@@ -605,35 +692,38 @@ __device__ __forceinline__ void key_ld4(uint4 (&k)[4], const uint4 *__restrict__
         k[e] = __ldg(bkp + (4 * g + e) * 32 + lane);
 }
 
-// Phase 2 of registers 4 g .. 4 g + 3 on vector-ordered rows into x[at ..];
-// their key vectors are k[at ..] (k[0 ..] of an array of four).
+// Phase 2 of registers 4 g .. 4 g + 3 on vector-ordered rows (values within
+// 8q) into x[at ..], in (-q, q); their key vectors (centred) are k[at ..] (k[0 ..]
+// of an array of four).  Montgomery: with |s| <= 4 8q q/2 < 2^31 q and m = s
+// q^-1 mod 2^32 signed, (s - m q) 2^-32 is the difference of the high words.
 template <int M, int KN, int W>
-__device__ __forceinline__ void pointwise_4(uint32_t (&x)[M], int at, const uint32_t (*f)[W],
-                                            int g, const uint4 (&k)[KN], int lane, const Prime &pr)
+__device__ __forceinline__ void pointwise_4(int32_t (&x)[M], int at, const uint32_t (*f)[W], int g,
+                                            const uint4 (&k)[KN], int lane, const Prime &pr)
 {
     const uint32_t qn = c_ntt.q_inv[pr.P];
     const int o = vec_word(4 * g, lane);
-    const uint4 f0 = *reinterpret_cast<const uint4 *>(f[0] + o);
-    const uint4 f1 = *reinterpret_cast<const uint4 *>(f[1] + o);
-    const uint4 f2 = *reinterpret_cast<const uint4 *>(f[2] + o);
-    const uint4 f3 = *reinterpret_cast<const uint4 *>(f[3] + o);
-    const uint32_t a0[4] = {f0.x, f0.y, f0.z, f0.w}, a1[4] = {f1.x, f1.y, f1.z, f1.w};
-    const uint32_t a2[4] = {f2.x, f2.y, f2.z, f2.w}, a3[4] = {f3.x, f3.y, f3.z, f3.w};
+    const int4 f0 = *reinterpret_cast<const int4 *>(f[0] + o);
+    const int4 f1 = *reinterpret_cast<const int4 *>(f[1] + o);
+    const int4 f2 = *reinterpret_cast<const int4 *>(f[2] + o);
+    const int4 f3 = *reinterpret_cast<const int4 *>(f[3] + o);
+    const int32_t a0[4] = {f0.x, f0.y, f0.z, f0.w}, a1[4] = {f1.x, f1.y, f1.z, f1.w};
+    const int32_t a2[4] = {f2.x, f2.y, f2.z, f2.w}, a3[4] = {f3.x, f3.y, f3.z, f3.w};
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const uint4 b = k[KN == 4 ? e : at + e];
-        uint64_t s = (uint64_t)a0[e] * b.x;
-        s += (uint64_t)a1[e] * b.y;
-        s += (uint64_t)a2[e] * b.z;
-        s += (uint64_t)a3[e] * b.w;
-        x[at + e] = mont_reduce(s, pr.q, qn);
+        int64_t s = (int64_t)a0[e] * (int32_t)b.x;
+        s += (int64_t)a1[e] * (int32_t)b.y;
+        s += (int64_t)a2[e] * (int32_t)b.z;
+        s += (int64_t)a3[e] * (int32_t)b.w;
+        const int32_t m = (int32_t)((uint32_t)s * qn);
+        x[at + e] = (int32_t)(s >> 32) - __mulhi(m, (int32_t)pr.q);
     }
 }
 
 // Phase 2 on vector-ordered rows; `k` holds the key vectors of group 0,
 // loaded before the barrier that made the rows complete.  The key vectors
 // of the next group are in flight while a group is multiplied.
-__device__ __forceinline__ void pointwise_v(uint32_t (&x)[32], const uint32_t (*f)[kSlotV],
+__device__ __forceinline__ void pointwise_v(int32_t (&x)[32], const uint32_t (*f)[kSlotV],
                                             uint4 (&k)[4], const uint4 *__restrict__ bkp, int lane,
                                             const Prime &pr)
 {
@@ -724,12 +814,6 @@ __device__ __forceinline__ void tb_ld16(uint32_t t, uint32_t (&v)[16])
                  : "r"(t));
 }
 
-// Barrier of the 128 threads of bootstrap slot `bi`.
-__device__ __forceinline__ void boot_sync(int bi)
-{
-    asm volatile("bar.sync %0, 128;" ::"r"(1 + bi) : "memory");
-}
-
 // Both digits of the words u0 and u1 (offset added) as fp16 pairs.
 // 1024 + field is exact in fp16 (bits 0x6400 | field).
 __device__ __forceinline__ void tb_digit2(uint32_t u0, uint32_t u1, uint32_t &d0, uint32_t &d1)
@@ -772,6 +856,25 @@ __device__ __forceinline__ void tb_digits(const uint32_t *ac, uint8_t *op, int c
     }
 }
 
+// (a0, a1) * b + c of packed fp32 bits, and the same from two words.
+__device__ __forceinline__ uint64_t ffma2_of(uint32_t a0, uint32_t a1, float b, float c)
+{
+    uint64_t r;
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %3};\n\t"
+        "mov.b64 c, {%4, %4};\n\tfma.rn.f32x2 %0, a, b, c;\n\t}"
+        : "=l"(r)
+        : "r"(a0), "r"(a1), "f"(b), "f"(c));
+    return r;
+}
+
+__device__ __forceinline__ void ffma2(uint32_t &a0, uint32_t &a1, float b, uint64_t c)
+{
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %2};\n\t"
+        "fma.rn.f32x2 a, a, b, %3;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "+r"(a0), "+r"(a1)
+        : "f"(b), "l"(c));
+}
+
 // Second half of the first pass for one digit row: the warp's 32 TMEM lanes
 // (lane i1) hold the sums of column k1 at t + 24 (k1 / 8) + 8 l + k1 % 8 and
 // its twiddle (w, w') at tw + 2 k1; twiddled residues in [0, 2q) go to
@@ -795,13 +898,18 @@ __device__ __forceinline__ void tb_combine(uint32_t t, uint32_t tw, uint32_t *sl
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
         for (int v = 0; v < 8; v += 4) {
-            uint32_t o[4];
+            uint32_t o[4], f[4];   // f: the quotients' bits
+#pragma unroll
+            for (int k = 0; k < 4; k += 2) {
+                const int e = v + k;
+                f[k] = s2[e], f[k + 1] = s2[e + 1];
+                ffma2(f[k], f[k + 1], c2, ffma2_of(s1[e], s1[e + 1], c1, c0));
+            }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int e = v + k;
-                const float f = fmaf(__uint_as_float(s2[e]), c2, fmaf(__uint_as_float(s1[e]), c1, c0));
                 const uint32_t y = (s1[e] << 9) + ((s2[e] << 18) + s0[e]);
-                const uint32_t x = __float_as_uint(f) * nq + (y + off);
+                const uint32_t x = f[k] * nq + (y + off);
                 o[k] = mul_shoup(x, w[2 * e], w[2 * e + 1], pr.q);
             }
             *reinterpret_cast<uint4 *>(slot + k0 + v) = make_uint4(o[0], o[1], o[2], o[3]);
@@ -887,11 +995,15 @@ __device__ __forceinline__ void tb_release(uint32_t tmem, int warp)
 //   pass 1, 2  warp s (the TMEM lanes it can read): digit row s modulo q_0,
 //              while V_1 runs once every warp has read V_0; then modulo q_1
 //   pointwise, inverse, CRT as warp (p, h)
-// Bound: issue of the integer multiplies (IMAD 2, IMAD.HI and IMAD.WIDE 4
-// cycles of the one pipe that has them, with little overlap).  608 gates:
-// 5.94 ms (102K bootstraps/s) against 7.85 ms (77.4K/s) with both passes as
-// butterflies.  The same first pass in CTAs whose bootstraps run in lockstep
-// took 7.4-8.1 ms: every wait and table load stood alone.
+// Bound: the integer multiplies (IMAD 2, IMAD.HI and IMAD.WIDE 4 cycles of the
+// one pipe that has them): 4.2K cycles of that pipe per warp and step, busy 3/4
+// of the time.  608 gates with the key switch: 5.56 ms (109K bootstraps/s)
+// against 7.85 ms with both passes as unsigned butterflies.  The same first
+// pass in CTAs whose bootstraps run in lockstep took 7.4-8.1 ms: every wait and
+// table load stood alone.  The inverse's last pass on the tensor pipe too
+// (three limbs of each residue, CRT from the sums): 6.4 ms; the products take
+// 1.6K cycles of a bootstrap's step, its splitting and sums as many
+// instructions as the butterflies.
 __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
 {
     constexpr int T = 128;
@@ -911,6 +1023,8 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
     const uint32_t tl = tmem + ((uint32_t)(32 * wr) << 16);   // this warp's TMEM lanes
     const uint32_t acc_cols = tmem + (uint32_t)(bi * kTbCols);
     const uint32_t dig_op = br_saddr(&S.fwd[1][0][0]);
+    const int2 *tw_inv = reinterpret_cast<const int2 *>(A.keys.tb_op + 2 * kTbOpBytes / 16) +
+                         1024 * h + lane;
     uint32_t phase = 0;   // products waited for (the same in the bootstrap's threads)
 
     for (long g = blockIdx.x + (long)bi * gridDim.x; g < A.count && !O.abort[bi];
@@ -931,9 +1045,11 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 tb_mma(acc_cols, dig_op, O, 0, &O.bar[bi]);
             }
-            uint32_t x[32];
+            int32_t x[32];
             const uint4 *bki = A.keys.bk_ntt + (((long)i * 2 + p) * 2 + h) * 1024;
-#pragma unroll 1
+            // unrolled: with the prime known, twiddles are operands in the constant
+            // bank and not loaded (608 gates 6.10 -> 5.74 ms)
+#pragma unroll
             for (int ph = 0; ph < 2; ++ph) {
                 const Prime pq((uint32_t)ph);
                 uint32_t *sl = S.fwd[ph][wr];
@@ -960,17 +1076,16 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
                 __syncwarp();
 #pragma unroll
                 for (int r = 0; r < 32; ++r)
-                    x[r] = sl[r * kRowV + lane];   // lane k1 reads slot[i1][k1]
+                    x[r] = (int32_t)sl[r * kRowV + lane];   // lane k1 reads slot[i1][k1]
                 __syncwarp();
-                ct32<true>(x, pq);
+                pass32_signed<false>(x, pq);
                 store_vec(sl, x, lane);
             }
             uint4 kv[4];
             key_ld4(kv, bki, 0, lane);
             boot_sync(bi);
             pointwise_v(x, S.fwd[h], kv, bki, lane, pr);
-            boot_sync(bi);
-            inv_ntt_v(x, S.fwd[0][wr], lane, lane_brv, A.keys.twb, pr);
+            inv_ntt_v(x, S.fwd[0][wr], lane, lane_brv, tw_inv, pr, bi);
             store_vec(S.fwd[1][wr], x, lane);
             boot_sync(bi);
             crt_rows_v<16>(S.acc[p], S.fwd[1][p * 2 + 0], S.fwd[1][p * 2 + 1], 16 * h, lane);
@@ -1067,7 +1182,8 @@ __device__ __forceinline__ void ct32_cyc_half(uint32_t (&y)[32], const uint32_t 
         y[r] = lazy_reduce_n(y[r], PL.fin[r], PL.nfin[r], pr);
 }
 
-// The first three stages of gs32 on the register block 8 z .. 8 z + 7;
+// The first three stages of a 32-point Gentleman-Sande pass (the inverse of ct32,
+// 32 times) on the register block 8 z .. 8 z + 7;
 // inputs [0, 2q).  The bounds by position are 16, 8, 4, 4, 2, 2, 2, 2 (times
 // q), the first two reduced to `fin` (a group whose twiddle is 1 takes its
 // product too, so that the four warps run the same code).
@@ -1097,7 +1213,7 @@ __device__ __forceinline__ void gs32_block(uint32_t (&x)[8], int z, const Prime 
     }
 }
 
-// The last two stages of gs32 on registers jj, jj + 8, jj + 16, jj + 24.
+// The last two stages of that pass on registers jj, jj + 8, jj + 16, jj + 24.
 // CYC: inputs below 8q, results below 32q (into a Shoup product); else inputs
 // below 4q, results below 8q.
 template <bool CYC>
@@ -1269,9 +1385,13 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_wide(const BrArgs A)
                 }
             }
             __syncthreads();
+            int32_t y[8];
             uint32_t x[8];
-            pointwise_4(x, 0, S.fwd[h], 2 * z, kv, lane, pr);
-            pointwise_4(x, 4, S.fwd[h], 2 * z + 1, kv, lane, pr);
+            pointwise_4(y, 0, S.fwd[h], 2 * z, kv, lane, pr);
+            pointwise_4(y, 4, S.fwd[h], 2 * z + 1, kv, lane, pr);
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                x[e] = (uint32_t)y[e] + pr.q;
             wide_inverse(x, S.ex[q], S.tr[q], tw, z, lane, lane_brv, 9 + q, pr);
 #pragma unroll
             for (int e = 0; e < 8; ++e)
@@ -1480,8 +1600,12 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_pair(const BrArgs A)
             *reinterpret_cast<uint4 *>(out + vec_word(4, 0)) = make_uint4(x[4], x[5], x[6], x[7]);
             __syncthreads();
             if (z < 2) {
-                pointwise_4(x, 0, S.fwd, 2 * q, kv, lane, pr);
-                pointwise_4(x, 4, S.fwd, 2 * q + 1, kv, lane, pr);
+                int32_t y[8];
+                pointwise_4(y, 0, S.fwd, 2 * q, kv, lane, pr);
+                pointwise_4(y, 4, S.fwd, 2 * q + 1, kv, lane, pr);
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    x[e] = (uint32_t)y[e] + pr.q;
                 wide_inverse(x, S.ex[z], S.tr[z], tw, q, lane, lane_brv, 9 + z, pr);
                 const uint32_t at = (((par * 2 + rank) * 2 + z) * kN + pair_word(2 * q, lane)) * 4;
 #pragma unroll
@@ -1575,6 +1699,11 @@ static int64_t centred(int64_t v, int64_t q)
     return v > q / 2 ? v - q : v;
 }
 
+static int32_t signed_shoup_of(int32_t w, uint32_t q)
+{
+    return (int32_t)std::llround((double)w * 0x1p32 / (double)q);
+}
+
 // Constant operand of the tensor-pipe first pass, op[prime] in its
 // shared-memory order.  Returns false if a bound the kernel relies on does
 // not hold.
@@ -1613,12 +1742,15 @@ static bool build_tb_operand(uint16_t *op)
 
 // Builds the NTT constants into c_ntt (current device) and the stage-B
 // twiddle table into twb_dev ([2][2][32][32] uint2), and the constant operand
-// of the tensor-pipe first pass into tb_op_dev (kTbOpBytes per prime).
+// of the tensor-pipe first pass (kTbOpBytes per prime) and the signed inverse
+// twiddles ([2][32][32] int2) into tb_op_dev.
 cudaError_t upload_ntt_constants(uint2 *twb_dev, uint4 *tb_op_dev, cudaStream_t stream)
 {
     NttConst C;
     std::memset(&C, 0, sizeof(C));
     std::vector<uint2> twb(2 * 2 * 32 * 32);
+    std::vector<uint16_t> op(kTbDevBytes / 2);
+    int2 *tws = reinterpret_cast<int2 *>(op.data() + kTbOpBytes);   // signed inverse twiddles
     const uint32_t qs[2] = {kQ0, kQ1};
     for (int P = 0; P < 2; ++P) {
         const uint32_t q = qs[P];
@@ -1645,6 +1777,19 @@ cudaError_t upload_ntt_constants(uint2 *twb_dev, uint4 *tb_op_dev, cudaStream_t 
                 C.izd[P][m + g][1] = shoup_of(id, q);
             }
         }
+        const auto put = [q](int32_t (&d)[2], uint64_t w) {
+            d[0] = (int32_t)centred((int64_t)w, q);
+            d[1] = signed_shoup_of(d[0], q);
+        };
+        for (int k = 1; k < 32; ++k) {
+            put(C.zs[P][k], C.zd[P][k][0]);
+            int ln = 16;
+            while (ln > k)
+                ln >>= 1;
+            put(C.izs[P][k], powmod(iw32, (uint64_t)(k - ln) * (16 / ln), q));
+            put(C.post[P][k], powmod(iw64, k, q));
+        }
+        C.one[P] = signed_shoup_of(1, q);
         for (int r = 0; r < 32; ++r)
             for (int l = 0; l < 32; ++l) {
                 // forward: lane i1 = l, register r carries k1 = brv5(r)
@@ -1653,6 +1798,8 @@ cudaError_t upload_ntt_constants(uint2 *twb_dev, uint4 *tb_op_dev, cudaStream_t 
                 uint32_t iv = (uint32_t)powmod(ipsi, (uint64_t)(2 * l + 1) * r, q);
                 twb[((P * 2 + 0) * 32 + r) * 32 + l] = make_uint2(f, shoup_of(f, q));
                 twb[((P * 2 + 1) * 32 + r) * 32 + l] = make_uint2(iv, shoup_of(iv, q));
+                const int32_t ivc = (int32_t)centred(iv, q);
+                tws[(P * 32 + r) * 32 + l] = make_int2(ivc, signed_shoup_of(ivc, q));
             }
         // q^-1 mod 2^32 by Newton iteration
         uint32_t inv = q;
@@ -1673,10 +1820,9 @@ cudaError_t upload_ntt_constants(uint2 *twb_dev, uint4 *tb_op_dev, cudaStream_t 
                         stream);
     if (e != cudaSuccess)
         return e;
-    std::vector<uint16_t> op(kTbOpBytes);
     if (!build_tb_operand(op.data()))
         return cudaErrorInvalidValue;
-    e = cudaMemcpyAsync(tb_op_dev, op.data(), 2 * kTbOpBytes, cudaMemcpyHostToDevice, stream);
+    e = cudaMemcpyAsync(tb_op_dev, op.data(), kTbDevBytes, cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess)
         return e;
     return cudaStreamSynchronize(stream);

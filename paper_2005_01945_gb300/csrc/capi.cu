@@ -133,7 +133,7 @@ int tfhe_ctx_create(const tfhe_params *params, int device, tfhe_ctx **out)
     if (e == cudaSuccess)
         e = cudaMalloc(&ctx->twb, 2 * 2 * 32 * 32 * sizeof(uint2));
     if (e == cudaSuccess)
-        e = cudaMalloc(&ctx->tb_op, 2 * 96 * 32 * 2);
+        e = cudaMalloc(&ctx->tb_op, kTbDevBytes);
     if (e == cudaSuccess)
         e = cudaMalloc(&ctx->status, sizeof(uint32_t));
     if (e == cudaSuccess)

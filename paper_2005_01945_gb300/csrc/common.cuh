@@ -31,7 +31,8 @@ constexpr uint32_t kDecompOffset = (1u << 31) + (1u << 21) + (1u << 11);
 // exceeds twice the largest magnitude of an exact external-product
 // coefficient, 4 * N * 2^9 * 2^31 = 2^52, so the centred CRT lift is the
 // exact integer.  q < 2^27 keeps every lazy value below 32 q < 2^32 and the
-// 4-term pointwise sum of [0,8q) x [0,q) products below q * 2^32.
+// 4-term pointwise sum of products of values within 8q and within q / 2 below
+// 16 q^2 < q 2^31.
 constexpr uint32_t kQ0 = 134215681u;     // 0x07FFF801
 constexpr uint32_t kQ1 = 134203393u;     // 0x07FFC801
 static_assert(32ull * kQ0 < (1ull << 32) && 32ull * kQ1 < (1ull << 32), "lazy bound");
@@ -57,19 +58,8 @@ __device__ __forceinline__ uint32_t csub(uint32_t x, uint32_t m)
 {
     return min(x, x - m);
 }
-
-// Montgomery reduction of a 64-bit x = hi 2^32 + lo < q 2^32: with
-// m = lo q^-1 mod 2^32, m q has low word lo, so x - m q = (hi - mulhi(m, q))
-// 2^32 exactly; the result hi - mulhi(m, q) + q = x 2^-32 mod q lies in
-// (0, 2q).  q_inv = q^-1 mod 2^32.
-__device__ __forceinline__ uint32_t mont_reduce(uint64_t x, uint32_t q, uint32_t q_inv)
-{
-    const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
-    return hi - __umulhi(lo * q_inv, q) + q;
-}
 #endif  // __CUDACC__
 
-// Per-context device pointers and sizes shared by the kernels.
 // Blind-rotation shape codes: one bootstrap on a CTA's 16 warps, and one
 // bootstrap on a cluster of two CTAs (one prime each).  1 is the throughput
 // shape (4 bootstraps per CTA); 2, 4, kBrStaged, kBrStagedCtl and kBrFive are
@@ -86,12 +76,16 @@ constexpr int kBrPairStaged = 48;
 // Key-switch launch code for the tiled kernel (shared-memory key stages);
 // the codes 1 .. 32 are j-chunks of the direct kernel.
 constexpr int kKsTiled = 64;
+// Device bytes of the tensor-pipe first pass's constant operands and the signed
+// inverse twiddles.
+constexpr int kTbDevBytes = 28672;
 
+// Per-context device pointers and sizes shared by the kernels.
 struct DevKeys {
     const uint4 *bk_ntt;   // [n][2 poly][2 prime][32 reg][32 lane] x uint4(4 rows)
     const uint4 *ksk;      // [N][t][base-1][kLweStride/4] words
     const uint2 *twb;      // stage-B twiddles [2 prime][2 dir][32 reg][32 lane] (w, w')
-    const uint4 *tb_op;    // tensor-pipe first pass: constant operands of the two primes
+    const uint4 *tb_op;    // tensor-pipe first pass: constant operands, inverse twiddles
     int n;
     int br_group;          // blind-rotation shape code, 0 = tuned or by batch size
     int ks_kernel;         // key-switch kernel: kKsTiled, j-chunks 1 .. 32 of the

@@ -2,9 +2,9 @@
 //
 // A serving process that restarts, or a second process on the same GPU,
 // can reuse keys without the client's key material and without redoing the
-// bootstrapping key's transform: the file holds the keys exactly as the
-// context keeps them in device memory (the bootstrapping key in the NTT
-// domain of the library's two primes, the key-switching key in padded
+// bootstrapping key's transform: the file holds the keys as the context
+// keeps them in device memory (the bootstrapping key in the NTT domain of the
+// library's two primes, as residues in [0, q), the key-switching key in padded
 // rows).  The format is tied to this library: a header records the
 // parameters, the primes, the sizes and a 64-bit FNV-1a checksum of the
 // payload, and loading rejects any mismatch.
@@ -38,6 +38,21 @@ static uint64_t fnv1a(uint64_t h, const uint8_t *p, size_t len)
 static size_t bk_ntt_bytes(const tfhe_ctx *ctx)
 {
     return (size_t)ctx->prm.n * 2 * 2 * kN * kRows * sizeof(uint32_t);
+}
+
+// The file holds the transformed key's residues in [0, q); on the device they
+// are centred.  Element index bit 12 selects the prime (common.cuh, bk_ntt).
+static void bk_residues(uint8_t *payload, size_t bytes, bool centred)
+{
+    static_assert(kN * kRows == 1 << 12, "prime bit");
+    uint32_t *w = reinterpret_cast<uint32_t *>(payload);
+    for (size_t i = 0; i < bytes / sizeof(uint32_t); ++i) {
+        const uint32_t q = (i >> 12) & 1 ? kQ1 : kQ0;
+        if (centred)
+            w[i] = w[i] > q / 2 ? w[i] - q : w[i];
+        else
+            w[i] = (int32_t)w[i] < 0 ? w[i] + q : w[i];
+    }
 }
 
 static size_t ksk_bytes()
@@ -84,6 +99,7 @@ extern "C" int tfhe_ctx_save_keys(tfhe_ctx *ctx, const char *path)
         e = cudaMemcpy(payload.data() + h.bk_bytes, ctx->ksk, h.ksk_bytes, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "tfhe_ctx_save_keys");
+    bk_residues(payload.data(), h.bk_bytes, false);
     h.checksum = fnv1a(0xCBF29CE484222325ull, payload.data(), payload.size());
     FILE *f = std::fopen(path, "wb");
     if (!f)
@@ -131,6 +147,7 @@ extern "C" int tfhe_ctx_load_keys(tfhe_ctx *ctx, const char *path)
         return fail(ctx, TFHE_EINVAL, "tfhe_ctx_load_keys: %s is truncated", path);
     if (fnv1a(0xCBF29CE484222325ull, payload.data(), payload.size()) != h.checksum)
         return fail(ctx, TFHE_EINVAL, "tfhe_ctx_load_keys: checksum mismatch in %s", path);
+    bk_residues(payload.data(), h.bk_bytes, true);
     DeviceGuard dg(ctx->device);
     cudaError_t e = cudaSuccess;
     if (!ctx->bk_ntt)
