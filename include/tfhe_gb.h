@@ -322,7 +322,9 @@ typedef enum {
     TFHE_OPT_KS_KERNEL = 6,  /* key-switch kernel: 64 = tiled (64 gates per CTA, key */
                              /*    rows staged in shared memory by bulk copies),    */
                              /*    1, 2, 4, .. 32 = direct kernel with that j-split, */
-                             /*    or 0 (default): autotuned, else by batch size    */
+                             /*    or 0 (default): autotuned, else the tensor-pipe  */
+                             /*    kernel above 64 gates and the tiled kernel up to */
+                             /*    there (recorded by the autotuner as 64)          */
     TFHE_OPT_TEST_FREE_HBM = 8,/* test hook for serving admission, 0 (default) off: */
                              /*    a serving loop started afterwards takes this     */
                              /*    many bytes as the device's free memory           */

@@ -760,14 +760,6 @@ __device__ __forceinline__ void crt_rows_v(uint32_t *acc, const uint32_t *x0, co
 }
 
 
-// Shared-memory matrix descriptor: K-major, no swizzle; lbo = byte distance
-// of core matrices adjacent in K, sbo = of 8-row groups.
-__device__ __forceinline__ uint64_t tb_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
-{
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
-           ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
-}
-
 // kind::f16, fp16 A and B (K-major), fp32 accumulator, M = 128, N = 96.
 constexpr uint32_t kTbIdesc = (1u << 4) | ((uint32_t)(kTbCols >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 
@@ -795,22 +787,12 @@ __device__ __forceinline__ void tb_mma(uint32_t d, uint32_t a, const TbOps &O, i
                  : "memory");
 }
 
-// 8 or 16 consecutive columns of this warp's 32 TMEM lanes.
+// 8 consecutive columns of this warp's 32 TMEM lanes (16: tb_ld16).
 __device__ __forceinline__ void tb_ld8(uint32_t t, uint32_t (&v)[8])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
                    "=r"(v[6]), "=r"(v[7])
-                 : "r"(t));
-}
-
-__device__ __forceinline__ void tb_ld16(uint32_t t, uint32_t (&v)[16])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, "
-                 "%10, %11, %12, %13, %14, %15}, [%16];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
-                   "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]),
-                   "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                  : "r"(t));
 }
 

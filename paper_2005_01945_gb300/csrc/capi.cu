@@ -12,6 +12,7 @@
 namespace tgb {
 
 cudaError_t upload_ntt_constants(uint2 *twb_dev, uint4 *tb_op_dev, cudaStream_t stream);
+cudaError_t launch_ksk_limbs(const uint4 *ksk, uint4 *limb, cudaStream_t stream);
 cudaError_t launch_bk_to_ntt(const int32_t *bk_dev, uint32_t *bk_ntt, int n, const uint2 *twb,
                              cudaStream_t stream);
 cudaError_t launch_keygen(int n, const int32_t *s, const int32_t *S, const uint32_t *bk_mask,
@@ -168,6 +169,8 @@ int tfhe_ctx_set_keys(tfhe_ctx *ctx, const int32_t *bk, const int32_t *ksk, void
         e = cudaMalloc(&ctx->bk_ntt, (size_t)n * 2 * 2 * kN * kRows * sizeof(uint32_t));
     if (e == cudaSuccess && !ctx->ksk)
         e = cudaMalloc(&ctx->ksk, ksk_rows * kLweStride * sizeof(int32_t));
+    if (e == cudaSuccess && !ctx->ksk_limb)
+        e = cudaMalloc(&ctx->ksk_limb, kKlBytes);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "cudaMalloc(keys)");
     const int32_t *bk_dev = bk;
@@ -189,12 +192,15 @@ int tfhe_ctx_set_keys(tfhe_ctx *ctx, const int32_t *bk, const int32_t *ksk, void
                               (size_t)(n + 1) * sizeof(int32_t), (size_t)(n + 1) * sizeof(int32_t),
                               ksk_rows, cudaMemcpyDefault, st);
     if (e == cudaSuccess)
+        e = launch_ksk_limbs(ctx->ksk, ctx->ksk_limb, st);
+    if (e == cudaSuccess)
         e = cudaStreamSynchronize(st);
     cudaFree(bk_tmp);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "tfhe_ctx_set_keys");
     ctx->keys.bk_ntt = reinterpret_cast<const uint4 *>(ctx->bk_ntt);
     ctx->keys.ksk = ctx->ksk;
+    ctx->keys.ksk_limb = ctx->ksk_limb;
     ctx->keys_loaded = true;
     return TFHE_OK;
 }
@@ -212,6 +218,7 @@ void tfhe_ctx_destroy(tfhe_ctx *ctx)
         cudaFree(ctx->status);
         cudaFree(ctx->bk_ntt);
         cudaFree(ctx->ksk);
+        cudaFree(ctx->ksk_limb);
         cudaFree(ctx->big);
         (void)cudaGetLastError();
     }

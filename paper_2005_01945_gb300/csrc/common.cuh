@@ -58,6 +58,25 @@ __device__ __forceinline__ uint32_t csub(uint32_t x, uint32_t m)
 {
     return min(x, x - m);
 }
+
+// Shared-memory matrix descriptor: K-major, no swizzle; lbo = byte distance
+// of core matrices adjacent in K, sbo = of 8-row groups.
+__device__ __forceinline__ uint64_t tb_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
+{
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
+           ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
+}
+
+// 16 consecutive columns of this warp's 32 TMEM lanes.
+__device__ __forceinline__ void tb_ld16(uint32_t t, uint32_t (&v)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, "
+                 "%10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
+                   "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]),
+                   "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                 : "r"(t));
+}
 #endif  // __CUDACC__
 
 // Blind-rotation shape codes: one bootstrap on a CTA's 16 warps, and one
@@ -76,6 +95,10 @@ constexpr int kBrPairStaged = 48;
 // Key-switch launch code for the tiled kernel (shared-memory key stages);
 // the codes 1 .. 32 are j-chunks of the direct kernel.
 constexpr int kKsTiled = 64;
+// ... and for the tensor-pipe kernel (one-hot digits times key limbs).
+constexpr int kKsTensor = 65;
+// Device bytes of the key-switching key's limbs: 3 fp16 limbs of 512 words.
+constexpr size_t kKlBytes = (size_t)kN * kKsT * kKsDigits * kLweStride * 3 * 2;
 // Device bytes of the tensor-pipe first pass's constant operands and the signed
 // inverse twiddles.
 constexpr int kTbDevBytes = 28672;
@@ -84,6 +107,7 @@ constexpr int kTbDevBytes = 28672;
 struct DevKeys {
     const uint4 *bk_ntt;   // [n][2 poly][2 prime][32 reg][32 lane] x uint4(4 rows)
     const uint4 *ksk;      // [N][t][base-1][kLweStride/4] words
+    const uint4 *ksk_limb; // fp16 limbs of it for the tensor-pipe key switch (kKlBytes)
     const uint2 *twb;      // stage-B twiddles [2 prime][2 dir][32 reg][32 lane] (w, w')
     const uint4 *tb_op;    // tensor-pipe first pass: constant operands, inverse twiddles
     int n;

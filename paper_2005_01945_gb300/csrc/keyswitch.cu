@@ -8,8 +8,10 @@
 //
 // GB300 design: the key-switching key (50 MB padded) is the only large
 // operand, and the work is 3/4 x 8192 row subtractions of 512 words per
-// gate.  Two kernels, picked per level width by the autotuner:
-//  * k_keyswitch_tiled (default): a CTA owns 64 gates x one 256-word half
+// gate.  Three kernels, picked per level width by the autotuner:
+//  * k_keyswitch_tensor (default above 64 gates): the sum as an exact matrix product of
+//    one-hot digits and fp16 limbs of the key on the tensor pipe.
+//  * k_keyswitch_tiled (default up to 64 gates): a CTA owns 64 gates x one 256-word half
 //    row x a range of j.  Warp 0 streams the 24 key-row halves of each j
 //    (8 digits x 3 non-zero values, 24 KB) into a 2-stage shared-memory
 //    ring with bulk asynchronous copies (cp.async.bulk, mbarrier
@@ -23,6 +25,8 @@
 //    result is bit-identical to a sequential sum).
 //  * k_keyswitch: 16 gates per CTA, key rows read straight through L1, the
 //    j-range split up to 32 ways (the autotuner's other candidate).
+#include <cuda_fp16.h>
+
 #include "common.cuh"
 
 namespace tgb {
@@ -32,6 +36,7 @@ constexpr int kKsThreads = 128;
 
 struct KsArgs {
     const uint4 *ksk;         // [N][t][3][kLweStride/4]
+    const uint4 *limb;        // tensor-pipe kernel: the key's limbs
     const int32_t *big;       // [count][kBigStride]
     int32_t *out;             // output base, row stride kLweStride
     const int32_t *idx_out;   // optional scatter rows (nullptr: row g)
@@ -472,6 +477,342 @@ __global__ void __launch_bounds__(32 * kKtWarps, 2) k_keyswitch_tiled(const KsAr
 }
 
 // ---------------------------------------------------------------------
+// Tensor-pipe key switch: one-hot digits times key limbs
+// ---------------------------------------------------------------------
+//
+// sum_(j,q) KSK[j][q][d_(j,q)] is a matrix product: the one-hot digits of the
+// gates, [gates x 24576] zeros and ones (K value (j, d, q) is 1 where digit q
+// of a'_j is d), times the key, whose words stand as three balanced base-2^11
+// limbs: v = l0 + 2^11 l1 + 2^22 l2, |l| <= 1024, exact in fp16.  A sum has at
+// most 8192 terms, |sum| <= 2^23: an exact fp32 integer, and the words follow
+// mod 2^32.
+//
+// A CTA: 256 gates (two accumulators of 128 rows) x 64 words (192 columns) x a
+// range of j.  Warps 0 - 7: each thread writes the one-hot values of its gate,
+// 8 per 16-byte store (one j and d); warp 8: bulk copies of the key limbs and
+// the products, through a ring of 4 stages of 64 K values, operands swizzled by
+// 128 bytes.  Partial sums of a j-split
+// are added into rows that k_ks_init prepared.
+// Bound: the key limbs from L2 (75 MB per 256 gates, 24 KB of each stage in
+// flight) against products that take 0.4 us a stage.  With the initialisation:
+// 1 gate 37 us (the tiled kernel: 45), 256 gates 47 (106), 608 gates 95 (235),
+// 2500 gates 285 (1082), 9000 gates 848 (3192).  The operands without a swizzle
+// took 118 us at 608 gates: their reads take twice the shared-memory cycles.
+constexpr int kKlWords = 64;                              // words per CTA
+constexpr int kKlCols = 3 * kKlWords;                     // limb-major columns
+constexpr int kKlGates = 256;                             // gates per CTA
+constexpr int kKlWin = 8;                                 // j per load of a'_j
+constexpr int kKlWins = kN / kKlWin;
+constexpr int kKlUnits = kN * kKsDigits / 8;              // stages: 8 groups of 8 K values
+constexpr int kKlStages = 4;
+constexpr uint32_t kKlBBytes = kKlCols * 128;             // 24 KB of limbs
+constexpr uint32_t kKlABytes = 128 * 128;                 // 16 KB of one-hot rows (128 gates)
+constexpr int kKlRow = kKlWords + 1;                      // words of a transposed result row
+static_assert(kKlBytes == (size_t)(kLweStride / kKlWords) * kKlUnits * kKlBBytes, "limb bytes");
+
+struct KlSmem {
+    uint8_t a[kKlStages][2][kKlABytes];
+    uint8_t b[kKlStages][kKlBBytes];
+    unsigned long long full_a[kKlStages], full_b[kKlStages], empty[kKlStages], done;
+    uint32_t tmem;
+    volatile int abort;                                   // a wait ran out
+};
+static_assert(sizeof(KlSmem::a) + sizeof(KlSmem::b) >= kKlGates * kKlRow * 4, "result rows");
+
+// 16-byte unit of (row, group of 8 K values) in a 128-byte-swizzled operand.
+__host__ __device__ constexpr int kl_unit(int row, int group) { return row * 8 + (group ^ (row & 7)); }
+
+// Limbs [word tile][8 groups of K values (j, d)][column][group][8 q], swizzled.
+__global__ void k_ksk_limbs(const uint32_t *__restrict__ ksk, uint4 *limb)
+{
+    const int j = blockIdx.x, d = blockIdx.y, word = threadIdx.x;
+    uint32_t l[3][4];
+    for (int q = 0; q < kKsT; ++q) {
+        int32_t v = (int32_t)ksk[((long)(j * kKsT + q) * kKsDigits + d) * kLweStride + word];
+        int32_t x[3];
+        for (int k = 0; k < 2; ++k) {
+            x[k] = (int32_t)(((uint32_t)v + 1024u) & 2047u) - 1024;
+            v = (int32_t)(((int64_t)v - x[k]) >> 11);
+        }
+        x[2] = v;
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t h = __half_as_ushort(__int2half_rn(x[k]));
+            l[k][q / 2] = q & 1 ? l[k][q / 2] | h << 16 : h;
+        }
+    }
+    const int tile = word / kKlWords, c = word % kKlWords;
+    const int kg = j * kKsDigits + d;
+    uint4 *o = limb + ((long)tile * kKlUnits + kg / 8) * (kKlBBytes / 16);
+    for (int k = 0; k < 3; ++k)
+        o[kl_unit(k * kKlWords + c, kg % 8)] = make_uint4(l[k][0], l[k][1], l[k][2], l[k][3]);
+}
+
+// Bounded wait that also ends when another thread's wait ran out.
+__device__ __forceinline__ bool kl_wait(KlSmem &S, unsigned long long *bar, uint32_t parity, long spin)
+{
+    for (long i = 0; i < spin && !S.abort; ++i)
+        if (mbar_try_wait(bar, parity))
+            return true;
+    return false;
+}
+
+// 16 bytes of one-hot fp16: value q is 1 where bit 14 - 2 q of m is set.
+__device__ __forceinline__ uint4 kl_onehot(uint32_t m)
+{
+    // of two words each, the even q's bits and, eight bits above them, the odd
+    // ones': shifted to bits 4 and 12 they select byte 0 (0) or byte 1 of 0x3C00
+    const uint32_t u = (m & 0x4400u) | (m & 0x1100u) << 10, v = (m & 0x44u) | (m & 0x11u) << 10;
+    return make_uint4(__byte_perm(0x3C00u, 0u, (u >> 10) & 0x1010u),
+                      __byte_perm(0x3C00u, 0u, (u >> 6) & 0x1010u),
+                      __byte_perm(0x3C00u, 0u, (v >> 2) & 0x1010u),
+                      __byte_perm(0x3C00u, 0u, (v << 2) & 0x1010u));
+}
+
+// Eight consecutive words of a row (16-byte loads where the address allows).
+__device__ __forceinline__ void kl_window(uint32_t (&w)[kKlWin], const int32_t *src, bool live)
+{
+    if (!live)
+        return;
+    if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+#pragma unroll
+        for (int k = 0; k < 8; k += 4) {
+            const int4 v = __ldg(reinterpret_cast<const int4 *>(src + k));
+            w[k] = (uint32_t)v.x, w[k + 1] = (uint32_t)v.y;
+            w[k + 2] = (uint32_t)v.z, w[k + 3] = (uint32_t)v.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            w[k] = (uint32_t)__ldg(src + k);
+    }
+}
+
+__device__ __forceinline__ void kl_load_b(KlSmem &S, const uint4 *limb, int tile, int unit, int slot)
+{
+    mbar_expect_tx(&S.full_b[slot], kKlBBytes);
+    bulk_g2s(S.b[slot], limb + ((long)tile * kKlUnits + unit) * (kKlBBytes / 16), kKlBBytes,
+             &S.full_b[slot]);
+}
+
+// kind::f16, fp16 A and B (K-major), fp32 accumulator, M = 128, N = 192.
+constexpr uint32_t kKlIdesc = (1u << 4) | ((uint32_t)(kKlCols >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+
+// Operand descriptor: K-major, 128-byte swizzle, 8-row groups 1 KB apart.
+__device__ __forceinline__ uint64_t kl_desc(uint32_t addr)
+{
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           (1ull << 46) | (2ull << 61);
+}
+
+__device__ __forceinline__ void kl_mma(uint32_t d, uint64_t a, uint64_t b, bool acc)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+                 "l"(a), "l"(b), "r"(kKlIdesc), "r"((uint32_t)acc)
+                 : "memory");
+}
+
+__device__ __forceinline__ void kl_commit(unsigned long long *bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                     smem_addr(bar))
+                 : "memory");
+}
+
+// grid: (j-chunks, 8 word tiles, tiles of 256 gates)
+__global__ void __launch_bounds__(288, 1) k_keyswitch_tensor(const KsArgs A)
+{
+    extern __shared__ __align__(1024) uint8_t kl_raw[];
+    KlSmem &S = *reinterpret_cast<KlSmem *>(kl_raw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tile = blockIdx.y;
+    const int w0 = (int)((long)blockIdx.x * kKlWins / gridDim.x);
+    const int nw = (int)((long)(blockIdx.x + 1) * kKlWins / gridDim.x) - w0;
+    const int p0 = 3 * w0, np = 3 * nw;   // stages
+    const long g0 = (long)blockIdx.z * kKlGates;
+    const bool two = g0 + 128 < A.count;   // the second accumulator has gates
+
+    if (tid == 0) {
+        for (int s = 0; s < kKlStages; ++s) {
+            mbar_init(&S.full_a[s], 8);
+            mbar_init(&S.full_b[s], 1);
+            mbar_init(&S.empty[s], 1);
+        }
+        mbar_init(&S.done, 1);
+        S.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_addr(&S.tmem)),
+                     "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = S.tmem;
+
+    if (warp == 8) {
+        if (lane == 0) {
+            const uint4 *limb = A.limb;
+            int issued = 0;
+            bool left = false;   // a wait ran out
+            for (; issued < kKlStages && issued < np; ++issued)
+                kl_load_b(S, limb, tile, p0 + issued, issued);
+            for (int it = 0; it < np; ++it) {
+                const int s = it % kKlStages;
+                const uint32_t ph = (uint32_t)(it / kKlStages) & 1u;
+                left = !kl_wait(S, &S.full_b[s], ph, A.spin) || !kl_wait(S, &S.full_a[s], ph, A.spin);
+                if (left)
+                    break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t bs = smem_addr(S.b[s]);
+                for (int m = 0; m < (two ? 2 : 1); ++m) {
+                    const uint32_t as = smem_addr(S.a[s][m]);
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        kl_mma(tmem + m * kKlCols, kl_desc(as + kk * 32), kl_desc(bs + kk * 32),
+                               it > 0 || kk > 0);
+                }
+                kl_commit(&S.empty[s]);
+                // refill the slot of the stage before this one
+                if (it > 0 && issued < np) {
+                    const int ps = (it - 1) % kKlStages;
+                    left = !kl_wait(S, &S.empty[ps], (uint32_t)((it - 1) / kKlStages) & 1u, A.spin);
+                    if (left)
+                        break;
+                    kl_load_b(S, limb, tile, p0 + issued, ps);
+                    ++issued;
+                }
+            }
+            kl_commit(&S.done);
+            if (!mbar_wait_bounded(&S.done, 0u, A.spin) || left) {
+                S.abort = 1;
+                atomicOr(A.status, kErrTimeout);
+            }
+            // after a wait that ran out: copies in flight get a bounded time
+            if (S.abort)
+                for (int k = issued > kKlStages ? issued - kKlStages : 0; k < issued; ++k)
+                    (void)mbar_wait_bounded(&S.full_b[k % kKlStages],
+                                            (uint32_t)(k / kKlStages) & 1u, A.spin);
+        }
+        __syncwarp();
+    } else {
+        const long g = g0 + tid;
+        const bool live = g < A.count;
+        const int32_t *src = A.big + (live ? g : 0) * kBigStride + w0 * kKlWin;
+        const int row = tid & 127;
+        uint8_t *dst = &S.a[0][tid >> 7][row * 128];
+        const uint32_t swz = (uint32_t)(row & 7) << 4;
+        // the words of a window are loaded one window ahead (a stage's fence waits
+        // for loads in flight, so one in three does)
+        uint32_t nx[kKlWin] = {}, cur[kKlWin];
+        kl_window(nx, src, live);
+        int it = 0;
+        for (int win = 0; win < nw; ++win) {
+#pragma unroll
+            for (int k = 0; k < kKlWin; ++k)
+                cur[k] = live ? (nx[k] + (1u << 15)) >> 16 : 0u;   // rounded to 16 bits
+            if (win + 1 < nw)
+                kl_window(nx, src + (win + 1) * kKlWin, live);
+            bool ok = true;
+#pragma unroll
+            for (int u = 0; u < 3; ++u, ++it) {
+                const int s = it % kKlStages;
+                ok = ok && (it < kKlStages ||
+                            kl_wait(S, &S.empty[s], (uint32_t)(it / kKlStages - 1) & 1u, A.spin));
+                if (!ok)
+                    break;
+                if (two || tid < 128) {
+                    uint8_t *o = dst + s * (2 * kKlABytes);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        const uint32_t x = cur[(8 * u + c) / 3], y = x >> 1;
+                        const int d = (8 * u + c) % 3;   // digit d + 1
+                        *reinterpret_cast<uint4 *>(o + ((uint32_t)(16 * c) ^ swz)) =
+                            kl_onehot((d == 0 ? x & ~y : d == 1 ? y & ~x : x & y) & 0x5555u);
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&S.full_a[s]))
+                                 : "memory");
+            }
+            if (!ok) {
+                if (!S.abort) {
+                    S.abort = 1;
+                    atomicOr(A.status, kErrTimeout);
+                }
+                break;
+            }
+        }
+    }
+    __syncthreads();   // the issuing thread has waited for every product
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+
+    // rows of sums to words, through the (idle) ring so that a warp's stores and
+    // reductions cover 32 consecutive words
+    uint32_t *rows = reinterpret_cast<uint32_t *>(&S.a[0][0][0]);
+    if (warp < 8 && !S.abort && (two || warp < 4)) {
+        const uint32_t t = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (warp >> 2) * kKlCols;
+#pragma unroll 1
+        for (int c = 0; c < kKlWords; c += 16) {
+            uint32_t s0[16], s1[16], s2[16];
+            tb_ld16(t + c, s0);
+            tb_ld16(t + kKlWords + c, s1);
+            tb_ld16(t + 2 * kKlWords + c, s2);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const uint32_t i0 = (uint32_t)__float2int_rn(__uint_as_float(s0[e]));
+                const uint32_t i1 = (uint32_t)__float2int_rn(__uint_as_float(s1[e]));
+                const uint32_t i2 = (uint32_t)__float2int_rn(__uint_as_float(s2[e]));
+                rows[tid * kKlRow + c + e] = 0u - (i0 + (i1 << 11) + (i2 << 22));
+            }
+        }
+        __syncwarp();
+        for (int r = 0; r < 32; ++r) {
+            const long g = g0 + warp * 32 + r;
+            if (g >= A.count)
+                break;
+            const long d = ks_dest(A, g);
+            if (d < 0 || d >= A.rows_out) {
+                if (lane == 0 && tile == 0 && !A.atomic)   // else flagged by k_ks_init
+                    atomicOr(A.status, kErrScatter);
+                continue;
+            }
+            const uint32_t *row = rows + (warp * 32 + r) * kKlRow;
+            int32_t *o = A.out + d * kLweStride + tile * kKlWords;
+#pragma unroll
+            for (int c = lane; c < kKlWords; c += 32) {
+                if (A.atomic)
+                    red_add(o + c, row[c]);
+                else
+                    o[c] = (int32_t)(row[c] + (tile * kKlWords + c == A.n
+                                                   ? (uint32_t)A.big[g * kBigStride + kN] : 0u));
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 8) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
+                     : "memory");
+    }
+}
+
+cudaError_t launch_ksk_limbs(const uint4 *ksk, uint4 *limb, cudaStream_t stream)
+{
+    k_ksk_limbs<<<dim3(kN, kKsDigits), kLweStride, 0, stream>>>(
+        reinterpret_cast<const uint32_t *>(ksk), limb);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------
 // Launch
 // ---------------------------------------------------------------------
 
@@ -481,19 +822,39 @@ static thread_local int ks_forced_chunks = 0;
 
 // Launch choice: kKsTiled selects the tiled kernel, 1..32 the j-chunks of
 // k_keyswitch.  A forced choice (autotuner, TFHE_OPT_KS_KERNEL) wins, then
-// the tuned value for the width bucket; untuned, the tiled kernel (on
-// GB300 it is the faster one from 1 to 10^4 gates).
+// the tuned value for the width bucket; untuned, or where the tuner kept the
+// default (recorded as kKsTiled), the tensor-pipe kernel above one tile of the
+// tiled one.  Up to there the two take 41 and 45 us alone, but behind a blind
+// rotation the 75 MB of limbs come from further away than the 50 MB of rows: one
+// gate 1.645 ms with the limbs, 1.625 with the rows.
 static int ks_chunks(long count, int num_sms, const DevKeys *choice)
 {
     if (ks_forced_chunks)
         return ks_forced_chunks;
     if (choice && choice->ks_kernel > 0)
         return choice->ks_kernel;
-    if (choice && choice->tune_ks[tune_bucket(count)] > 0)
-        return choice->tune_ks[tune_bucket(count)];
-    (void)count;
+    const int tuned = choice ? choice->tune_ks[tune_bucket(count)] : 0;
+    if (tuned > 0 && tuned != kKsTiled)
+        return tuned;
     (void)num_sms;
-    return kKsTiled;
+    return choice && choice->ksk_limb && !choice->ks_stall && count > kKtTile ? kKsTensor : kKsTiled;
+}
+
+// j-chunks of the tensor-pipe kernel: the split with the least CTA waves times
+// windows per CTA (a CTA's start and end take as long as about 6 windows).
+static int kl_chunks(long count, int num_sms)
+{
+    const long ctas = 8 * ((count + kKlGates - 1) / kKlGates);
+    int best = 1;
+    long cost = 0;
+    for (int c = 1; c <= 32; ++c) {
+        const long t = (ctas * c + num_sms - 1) / num_sms * ((kKlWins + c - 1) / c + 6);
+        if (c == 1 || t < cost) {
+            best = c;
+            cost = t;
+        }
+    }
+    return best;
 }
 
 // j-chunks of the tiled kernel: enough CTAs for two per SM (16 warps).
@@ -514,6 +875,8 @@ int keyswitch_kernels(long count, int num_sms, const DevKeys *choice)
     const int c = ks_chunks(count, num_sms, choice);
     if (c == kKsTiled)
         return kt_chunks(count, num_sms) > 1 ? 2 : 1;
+    if (c == kKsTensor)
+        return kl_chunks(count, num_sms) > 1 ? 2 : 1;
     return c > 1 ? 2 : 1;
 }
 
@@ -526,9 +889,12 @@ cudaError_t launch_keyswitch(const uint4 *ksk, const int32_t *big, int32_t *out,
         return cudaSuccess;
     const int pick = ks_chunks(count, num_sms, choice);
     const bool tiled = pick == kKsTiled;
-    const int chunks = tiled ? kt_chunks(count, num_sms) : pick;
+    const bool tensor = pick == kKsTensor;
+    const int chunks = tiled ? kt_chunks(count, num_sms)
+                     : tensor ? kl_chunks(count, num_sms) : pick;
     KsArgs A;
     A.ksk = ksk;
+    A.limb = tensor ? choice->ksk_limb : nullptr;
     A.big = big;
     A.out = out;
     A.idx_out = idx_out;
@@ -546,6 +912,23 @@ cudaError_t launch_keyswitch(const uint4 *ksk, const int32_t *big, int32_t *out,
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess)
             return e;
+    }
+    if (tensor) {
+        static int prepared[64] = {0};
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (dev >= 0 && dev < 64 && !prepared[dev]) {
+            cudaError_t e = cudaFuncSetAttribute(k_keyswitch_tensor,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)sizeof(KlSmem));
+            if (e != cudaSuccess)
+                return e;
+            prepared[dev] = 1;
+        }
+        dim3 grid((unsigned)chunks, (unsigned)(kLweStride / kKlWords),
+                  (unsigned)((count + kKlGates - 1) / kKlGates));
+        k_keyswitch_tensor<<<grid, 288, sizeof(KlSmem), stream>>>(A);
+        return cudaGetLastError();
     }
     if (tiled) {
         static int prepared[64] = {0};

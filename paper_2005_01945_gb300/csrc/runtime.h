@@ -21,6 +21,7 @@ struct tfhe_ctx {
     uint4 *tb_op = nullptr;          // tensor-pipe first pass: constant operands
     uint32_t *bk_ntt = nullptr;      // bootstrapping key, NTT domain
     uint4 *ksk = nullptr;            // key-switching key, padded rows
+    uint4 *ksk_limb = nullptr;       // its limbs for the tensor-pipe key switch
     uint32_t *status = nullptr;      // device status word
     int32_t *big = nullptr;          // LWE_N scratch between the two stages
     size_t big_rows = 0;

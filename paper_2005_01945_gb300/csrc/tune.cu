@@ -2,7 +2,7 @@
 // kernels: the blind-rotation shape (4 independent bootstraps per CTA, one
 // bootstrap on a CTA's 16 warps, or one bootstrap on a cluster of two CTAs)
 // and the
-// key-switch kernel (the tiled kernel with shared-memory key stages, or
+// key-switch kernel (the default, on the tensor pipe, recorded as 64, or
 // the direct kernel with its j-split of 1 .. 32 chunks), chosen per
 // level-width bucket by timing the candidates on synthetic ciphertexts
 // with the context's keys.  It also records the time of a level at each
@@ -46,7 +46,7 @@ static std::string cache_key(int device)
     // the tag separates these kernels' times from those of files written for
     // other blind-rotation kernels: an older line is not used, and tuning
     // appends a new one
-    return name + ":" + std::to_string(prop.multiProcessorCount) + ":tc2";
+    return name + ":" + std::to_string(prop.multiProcessorCount) + ":tc3";
 }
 
 static bool load_cache(const char *path, const std::string &key, DevKeys &k)
@@ -178,8 +178,8 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
                 }
             }
             best = 1e30f;
-            for (int c : {kKsTiled, 1, 2, 4, 8, 16, 32}) {
-                if (c != kKsTiled && (W + 15) / 16 * c > 64L * ctx->num_sms)
+            for (int c : {kKsTensor, 1, 2, 4, 8, 16, 32}) {
+                if (c != kKsTensor && (W + 15) / 16 * c > 64L * ctx->num_sms)
                     continue;   // far more CTAs than useful
                 keyswitch_force_chunks(c);
                 float tot = 0;
@@ -187,7 +187,7 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
                     e = cudaEventRecord(e0, st);
                     if (e == cudaSuccess)
                         e = launch_keyswitch(K.ksk, big, out, nullptr, W, W, ctx->prm.n,
-                                             ctx->num_sms, ctx->status, st);
+                                             ctx->num_sms, ctx->status, st, &K);
                     if (e == cudaSuccess)
                         e = cudaEventRecord(e1, st);
                     if (e == cudaSuccess)
@@ -199,7 +199,7 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
                 keyswitch_force_chunks(0);
                 if (e == cudaSuccess && tot < best) {
                     best = tot;
-                    ks[b] = (int8_t)c;
+                    ks[b] = (int8_t)(c == kKsTensor ? kKsTiled : c);   // the default
                 }
             }
         }
