@@ -414,7 +414,7 @@ struct BrArgs {
     long rows_a, rows_b, rows_c;          // rows addressable through the bases
     const uint8_t *ops;              // gate opcodes (nullptr: bootstrap in_a as is)
     int32_t *big;                    // out: LWE_N samples [count][kBigStride]
-    long count;
+    long first, count;               // gates first .. count - 1
     uint32_t mu;                     // test-vector amplitude
     uint32_t *status;
 };
@@ -1009,7 +1009,7 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
                          1024 * h + lane;
     uint32_t phase = 0;   // products waited for (the same in the bootstrap's threads)
 
-    for (long g = blockIdx.x + (long)bi * gridDim.x; g < A.count && !O.abort[bi];
+    for (long g = A.first + blockIdx.x + (long)bi * gridDim.x; g < A.count && !O.abort[bi];
          g += 4L * gridDim.x) {
         const bool active = br_prologue<T>(A, g, tb, S.abar, true);
         boot_sync(bi);
@@ -1309,7 +1309,7 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_wide(const BrArgs A)
         tw[e] = __ldg(A.keys.twb + ((h * 2 + 1) * 32 + 2 * z + (e & 1) + 8 * (e >> 1)) * 32 + lane);
     uint32_t phase = 0;
 
-    for (long g = blockIdx.x; g < A.count && !O.abort[0]; g += gridDim.x) {
+    for (long g = A.first + blockIdx.x; g < A.count && !O.abort[0]; g += gridDim.x) {
         const bool active = br_prologue<512>(A, g, tid, S.abar, true);
         __syncthreads();
         br_acc_init<512>(A, S.acc, S.abar[n], tid);
@@ -1529,7 +1529,7 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_pair(const BrArgs A)
     }
     cl.sync();   // the partner's shared memory and barriers are there
 
-    for (long g = cid; g < A.count; g += nclusters) {
+    for (long g = A.first + cid; g < A.count; g += nclusters) {
         const bool active = br_prologue<512>(A, g, tid, S.abar, rank == 0);
         __syncthreads();
         br_acc_init<512>(A, S.acc, S.abar[n], tid);
@@ -1853,8 +1853,10 @@ static cudaError_t launch_tc(const BrArgs &A, unsigned blocks, int dev, cudaStre
     return cudaGetLastError();
 }
 
-static cudaError_t launch_wide(const BrArgs &A, unsigned blocks, int dev, cudaStream_t stream)
+static cudaError_t launch_wide(const BrArgs &A, long sms, int dev, cudaStream_t stream)
 {
+    const long count = A.count - A.first;
+    const unsigned blocks = (unsigned)(count < sms ? count : sms);
     constexpr int smem = (int)sizeof(WideSmem) + (int)sizeof(TbOps);
     static int prepared[64] = {0};
     if (dev >= 0 && dev < 64 && !prepared[dev]) {
@@ -1881,7 +1883,8 @@ static cudaError_t launch_pair(const BrArgs &A, long pairs, int dev, cudaStream_
         prepared[dev] = 1;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * (A.count < pairs ? A.count : pairs)));
+    const long count = A.count - A.first;
+    cfg.gridDim = dim3((unsigned)(2 * (count < pairs ? count : pairs)));
     cfg.blockDim = dim3(512);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -1893,6 +1896,28 @@ static cudaError_t launch_pair(const BrArgs &A, long pairs, int dev, cudaStream_
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_blind_rotate_pair, A);
+}
+
+static cudaError_t launch_shape(const BrArgs &A, int shape, long nsm, int dev, cudaStream_t stream)
+{
+    const long count = A.count - A.first;
+    if (shape == kBrPair || shape == kBrPairStaged)
+        return launch_pair(A, nsm >= 2 ? nsm / 2 : 1, dev, stream);
+    if (shape == kBrSplit || shape == kBrSplitStaged)
+        return launch_wide(A, nsm, dev, stream);
+    // the throughput shape (the other codes are accepted for saved tuning
+    // files and options)
+    return launch_tc(A, (unsigned)(count < nsm ? count : nsm), dev, stream);
+}
+
+// Gates at the end of a level that leave at most one bootstrap per SM for its
+// last wave of the throughput shape: they run on the shapes of narrow levels
+// instead, behind it (a wave of one per SM takes 3.0 - 3.3 ms there, 1.7 - 2.1
+// ms on those; two per SM, 3.6 ms, would take two rounds).
+static long br_tail(long count, long nsm, int forced, int shape)
+{
+    const long tail = count % (4 * nsm);
+    return forced == 0 && shape == 1 && count > 4 * nsm && tail <= nsm ? tail : 0;
 }
 
 cudaError_t launch_blind_rotate(const DevKeys &keys, const uint8_t *ops, const int32_t *in_a,
@@ -1916,23 +1941,34 @@ cudaError_t launch_blind_rotate(const DevKeys &keys, const uint8_t *ops, const i
     A.rows_c = rows_c;
     A.ops = ops;
     A.big = big;
-    A.count = count;
     A.mu = mu;
     A.status = status;
     int dev = 0;
     cudaGetDevice(&dev);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int shape = br_group(count, sms > 0 ? sms : 1, keys.br_group, keys.tune_br);
     const long nsm = sms > 0 ? sms : 1;
-    if (shape == kBrPair || shape == kBrPairStaged)
-        return launch_pair(A, nsm >= 2 ? nsm / 2 : 1, dev, stream);
     (void)grid;
-    if (shape == kBrSplit || shape == kBrSplitStaged)
-        return launch_wide(A, (unsigned)(count < nsm ? count : nsm), dev, stream);
-    // the throughput shape (the other codes are accepted for saved tuning
-    // files and options)
-    return launch_tc(A, (unsigned)(count < nsm ? count : nsm), dev, stream);
+    const int shape = br_group(count, (int)nsm, keys.br_group, keys.tune_br);
+    const long tail = br_tail(count, nsm, keys.br_group, shape);
+    A.first = 0;
+    A.count = count - tail;
+    cudaError_t e = launch_shape(A, shape, nsm, dev, stream);
+    if (tail && e == cudaSuccess) {
+        A.first = count - tail;
+        A.count = count;
+        e = launch_shape(A, 2 * tail <= nsm ? kBrPair : kBrSplit, nsm, dev, stream);
+    }
+    return e;
+}
+
+int blind_rotate_kernels(long count, int num_sms, const DevKeys &keys)
+{
+    if (count <= 0)
+        return 0;
+    const long nsm = num_sms > 0 ? num_sms : 1;
+    const int shape = br_group(count, (int)nsm, keys.br_group, keys.tune_br);
+    return br_tail(count, nsm, keys.br_group, shape) ? 2 : 1;
 }
 
 }  // namespace tgb

@@ -12,7 +12,6 @@
 namespace tgb {
 
 cudaError_t upload_ntt_constants(uint2 *twb_dev, uint4 *tb_op_dev, cudaStream_t stream);
-cudaError_t launch_ksk_limbs(const uint4 *ksk, uint4 *limb, cudaStream_t stream);
 cudaError_t launch_bk_to_ntt(const int32_t *bk_dev, uint32_t *bk_ntt, int n, const uint2 *twb,
                              cudaStream_t stream);
 cudaError_t launch_keygen(int n, const int32_t *s, const int32_t *S, const uint32_t *bk_mask,
@@ -103,7 +102,8 @@ int run_bootstrap(tfhe_ctx *ctx, const uint8_t *ops, const int32_t *a, const int
                          ctx->num_sms, ctx->status, stream, &ctx->keys);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "key switch launch");
-    ctx->launches += 1 + keyswitch_kernels(count, ctx->num_sms, &ctx->keys);
+    ctx->launches += blind_rotate_kernels(count, ctx->num_sms, ctx->keys) +
+                     keyswitch_kernels(count, ctx->num_sms, &ctx->keys);
     return TFHE_OK;
 }
 
@@ -169,8 +169,6 @@ int tfhe_ctx_set_keys(tfhe_ctx *ctx, const int32_t *bk, const int32_t *ksk, void
         e = cudaMalloc(&ctx->bk_ntt, (size_t)n * 2 * 2 * kN * kRows * sizeof(uint32_t));
     if (e == cudaSuccess && !ctx->ksk)
         e = cudaMalloc(&ctx->ksk, ksk_rows * kLweStride * sizeof(int32_t));
-    if (e == cudaSuccess && !ctx->ksk_limb)
-        e = cudaMalloc(&ctx->ksk_limb, kKlBytes);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "cudaMalloc(keys)");
     const int32_t *bk_dev = bk;
@@ -192,7 +190,7 @@ int tfhe_ctx_set_keys(tfhe_ctx *ctx, const int32_t *bk, const int32_t *ksk, void
                               (size_t)(n + 1) * sizeof(int32_t), (size_t)(n + 1) * sizeof(int32_t),
                               ksk_rows, cudaMemcpyDefault, st);
     if (e == cudaSuccess)
-        e = launch_ksk_limbs(ctx->ksk, ctx->ksk_limb, st);
+        e = make_ksk_limbs(ctx, st);
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(st);
     cudaFree(bk_tmp);
@@ -303,7 +301,7 @@ int tfhe_blind_rotate_extract(tfhe_ctx *ctx, const uint8_t *ops, const int32_t *
                                         ctx->br_grid, (cudaStream_t)stream);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "blind rotation launch");
-    ctx->launches += 1;
+    ctx->launches += blind_rotate_kernels((long)count, ctx->num_sms, ctx->keys);
     return TFHE_OK;
 }
 

@@ -986,7 +986,8 @@ static cudaError_t enqueue_levels(tfhe_ctx *ctx, Plan &P, cudaStream_t st, bool 
             e = mark(3 * (l - 1) + 2);
         if (e != cudaSuccess)
             return e;
-        kernels += 1 + keyswitch_kernels(cnt, ctx->num_sms, &ctx->keys);
+        kernels += blind_rotate_kernels(cnt, ctx->num_sms, ctx->keys) +
+                   keyswitch_kernels(cnt, ctx->num_sms, &ctx->keys);
     }
     P.kernels_per_run = kernels;
     return cudaSuccess;

@@ -55,7 +55,6 @@ static void bk_residues(uint8_t *payload, size_t bytes, bool centred)
     }
 }
 
-cudaError_t launch_ksk_limbs(const uint4 *ksk, uint4 *limb, cudaStream_t stream);
 
 static size_t ksk_bytes()
 {
@@ -156,14 +155,12 @@ extern "C" int tfhe_ctx_load_keys(tfhe_ctx *ctx, const char *path)
         e = cudaMalloc(&ctx->bk_ntt, h.bk_bytes);
     if (e == cudaSuccess && !ctx->ksk)
         e = cudaMalloc(&ctx->ksk, h.ksk_bytes);
-    if (e == cudaSuccess && !ctx->ksk_limb)
-        e = cudaMalloc(&ctx->ksk_limb, kKlBytes);
     if (e == cudaSuccess)
         e = cudaMemcpy(ctx->bk_ntt, payload.data(), h.bk_bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(ctx->ksk, payload.data() + h.bk_bytes, h.ksk_bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = launch_ksk_limbs(ctx->ksk, ctx->ksk_limb, 0);
+        e = make_ksk_limbs(ctx, 0);
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(0);
     if (e != cudaSuccess)

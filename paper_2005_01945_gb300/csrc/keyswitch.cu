@@ -27,7 +27,7 @@
 //    j-range split up to 32 ways (the autotuner's other candidate).
 #include <cuda_fp16.h>
 
-#include "common.cuh"
+#include "runtime.h"
 
 namespace tgb {
 
@@ -805,10 +805,17 @@ __global__ void __launch_bounds__(288, 1) k_keyswitch_tensor(const KsArgs A)
     }
 }
 
-cudaError_t launch_ksk_limbs(const uint4 *ksk, uint4 *limb, cudaStream_t stream)
+// The limbs of the context's key.  Without room for them the key switch runs on
+// the key's rows (the tiled kernel).
+cudaError_t make_ksk_limbs(tfhe_ctx *ctx, cudaStream_t stream)
 {
+    if (!ctx->ksk_limb && cudaMalloc(&ctx->ksk_limb, kKlBytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        ctx->ksk_limb = nullptr;
+        return cudaSuccess;
+    }
     k_ksk_limbs<<<dim3(kN, kKsDigits), kLweStride, 0, stream>>>(
-        reinterpret_cast<const uint32_t *>(ksk), limb);
+        reinterpret_cast<const uint32_t *>(ctx->ksk), ctx->ksk_limb);
     return cudaGetLastError();
 }
 

@@ -131,6 +131,7 @@ extern "C" int tfhe_bootstrap_gates_noalloc(tfhe_ctx *ctx, const uint8_t *ops, c
                          ctx->status, st, &ctx->keys);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "key switch launch");
-    ctx->launches += 1 + keyswitch_kernels(n, ctx->num_sms, &ctx->keys);
+    ctx->launches += blind_rotate_kernels(n, ctx->num_sms, ctx->keys) +
+                     keyswitch_kernels(n, ctx->num_sms, &ctx->keys);
     return TFHE_OK;
 }

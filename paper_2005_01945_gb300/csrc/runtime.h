@@ -82,6 +82,9 @@ cudaError_t launch_keyswitch(const uint4 *ksk, const int32_t *big, int32_t *out,
                              int num_sms, uint32_t *status, cudaStream_t stream,
                              const DevKeys *choice = nullptr);
 
+// Kernels one launch_blind_rotate call issues.
+int blind_rotate_kernels(long count, int num_sms, const DevKeys &keys);
+cudaError_t make_ksk_limbs(tfhe_ctx *ctx, cudaStream_t stream);
 int keyswitch_kernels(long count, int num_sms, const DevKeys *choice = nullptr);
 void keyswitch_force_chunks(int chunks);
 

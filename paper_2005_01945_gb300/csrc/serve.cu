@@ -659,7 +659,8 @@ static void srv_loop(Server *Sp)
         I.gates = count;
         {
             std::lock_guard<std::mutex> lock(S.mu);
-            ctx->launches += 1 + keyswitch_kernels(count, ctx->num_sms, &ctx->keys) +
+            ctx->launches += blind_rotate_kernels(count, ctx->num_sms, ctx->keys) +
+                             keyswitch_kernels(count, ctx->num_sms, &ctx->keys) +
                              (long)finishing.size();
             S.stats.gates += count;
             S.stats.iterations++;

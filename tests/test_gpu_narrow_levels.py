@@ -39,6 +39,7 @@ def gpu(orc):
 
 
 @pytest.mark.parametrize("shape,count", [(0, 1), (0, 76), (0, 77), (0, 152), (0, 153), (16, 229),
+                                         (0, 609), (0, 684), (0, 685), (0, 760), (0, 761),
                                          (8, 459)])
 def test_widths(gpu, orc, shape, count):
     torch, api, p, P = gpu["torch"], gpu["api"], gpu["p"], gpu["P"]
