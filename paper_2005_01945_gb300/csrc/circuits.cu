@@ -1100,25 +1100,45 @@ static int run_plan(tfhe_ctx *ctx, Plan &P, const tfhe_job *jobs, cudaStream_t s
 // Both schedules are costed with the autotuner's measurements: a level of w
 // gates costs the measured time of its width bucket while w fits one wave,
 // ceil(w / wave) wave times above, and the narrow unit is used once it is at
-// least 1 % cheaper.  Decided
-// once per job mix; without autotuner measurements the unit is one wave of
-// 4 per SM.
+// least 1 % cheaper.  Decided once per job mix.  Without autotuner measurements
+// the times are the ones below, and only a mix of at most two bootstraps per SM
+// and level on average is costed (a wider one's narrow schedule costs more, and
+// building it takes as long as the schedule itself): one 32-bit Dadda product
+// ran 22 levels of up to 528 gates in 48.1 ms and runs them at 152 in 41.3.
+constexpr float kLevelMs[3] = {2.10f, 3.66f, 5.43f};   // levels of 1, 2 and 4 per SM
+constexpr float kPairShare = 0.79f;                    // of a level of one per two SMs
+
 static long choose_wave(tfhe_ctx *ctx, CircuitCache &C, const std::string &sig,
                         const tfhe_job *jobs, size_t njobs)
 {
     const long w1 = ctx->num_sms, w4 = 4L * ctx->num_sms;
     const DevKeys &K = ctx->keys;
-    const float t4 = K.wave_ms[0];
-    if (!(t4 > 0.f))
-        return w4;
-    auto it = C.wave_choice.find(sig);
+    const bool tuned = K.wave_ms[0] > 0.f;
+    const float t4 = tuned ? K.wave_ms[0] : kLevelMs[2];
+    if (!tuned) {
+        double gates = 0;
+        long depth = 0;
+        for (size_t j = 0; j < njobs; ++j) {
+            const auto net = get_netlist(jobs[j].kind, jobs[j].width, jobs[j].rows, jobs[j].cols);
+            if (!net || jobs[j].batch < 0)
+                return w4;   // refused when the schedule is built
+            gates += (double)net->op.size() * (double)jobs[j].batch;
+            depth = std::max(depth, (long)net->depth);
+        }
+        if (gates > 2.0 * w1 * depth)
+            return w4;
+    }
+    const std::string key = tuned ? sig : sig + "|untuned";
+    auto it = C.wave_choice.find(key);
     if (it != C.wave_choice.end())
         return it->second;
     auto level_cost = [&](long n) -> double {
         if (n > w4)
             return (double)((n + w4 - 1) / w4) * t4;
         const int b = tune_bucket(n);
-        return K.tune_ms[b] > 0.f ? K.tune_ms[b] : t4;
+        const float ms = tuned ? K.tune_ms[b] : b < 3 ? kLevelMs[b] : t4;
+        const bool pair = 2 * n <= w1 && (!tuned || K.tune_br[b] == kBrSplit);
+        return ms > 0.f ? (pair ? kPairShare * ms : ms) : t4;
     };
     auto cost = [&](long unit) -> double {
         Schedule S;
@@ -1131,12 +1151,12 @@ static long choose_wave(tfhe_ctx *ctx, CircuitCache &C, const std::string &sig,
     };
     const double c4 = cost(w4);
     long pick = w4;
-    if (c4 >= 0 && K.tune_ms[0] > 0.f && w1 <= kTuneEdge[0]) {
+    if (c4 >= 0 && (!tuned || K.tune_ms[0] > 0.f) && w1 <= kTuneEdge[0]) {
         const double c1 = cost(w1);
         if (c1 >= 0 && c1 < 0.99 * c4)
             pick = w1;
     }
-    C.wave_choice[sig] = pick;
+    C.wave_choice[key] = pick;
     return pick;
 }
 
