@@ -91,8 +91,8 @@ def parse():
     ap.add_argument("--no-latency", action="store_true")
     ap.add_argument("--cpu-gates", type=int, default=128)
     ap.add_argument("--br-only", type=int, default=0, help="profile mode: blind rotation alone")
-    ap.add_argument("--br-group", type=int, default=0, help="blind-rotation CTA shape: 1, 2, 4 bootstraps per CTA, 8 = one "
-                         "bootstrap on 8 warps, 16 = one bootstrap on two CTAs (0: automatic)")
+    ap.add_argument("--br-group", type=int, default=0, help="blind-rotation shape: 1 = four bootstraps per CTA, 8 = one "
+                         "bootstrap on 16 warps, 16 = one bootstrap on two CTAs (0: automatic)")
     ap.add_argument("--ks-only", type=int, default=0,
                     help="profile mode: key switch alone on this many uniform LWE_N samples")
     ap.add_argument("--tc-products", type=int, default=0,
@@ -762,7 +762,7 @@ def br_roofline(p, br_ms, br_launch, br_boot, step_ms_total, ks_ms, sm_count, sm
     peak_ops = sm_count * INT32_LANES_PER_SM * sm_max * 1e6
     ops = OPS_PER_CMUX * p.n * br_boot
     achieved = ops / (br_ms / 1e3) if br_ms > 0 else 0.0
-    return {"kernel": "k_blind_rotate", "bound": "alu", "achieved": achieved / 1e12,
+    return {"kernel": "k_blind_rotate_tc", "bound": "alu", "achieved": achieved / 1e12,
             "peak": peak_ops / 1e12, "unit": "Tops/s (int32)", "frac": achieved / peak_ops,
             "peak_basis": f"{sm_count} SMs x {INT32_LANES_PER_SM} INT32 "
                           f"lanes x {sm_max:.0f} MHz (max SM clock)",
@@ -937,12 +937,12 @@ def main():
     ks_calls = max(br_launch, 1)
     ks_bytes = KSK_BYTES + br_boot / ks_calls * (p.N + 1 + p.n + 1) * 4
     ks_gbs = ks_bytes / (ks_ms / ks_calls / 1e3) / 1e9 if ks_ms > 0 else 0.0
-    keyswitch = {"kernel": "k_keyswitch_tiled", "bound": "smem", "achieved_hbm": ks_gbs,
+    keyswitch = {"kernel": "k_keyswitch_tensor", "bound": "L2 (key limbs)", "achieved_hbm": ks_gbs,
                  "peak_hbm": hbm, "unit": "GB/s", "frac_hbm": ks_gbs / hbm,
                  "algorithmic_bytes_per_call": ks_bytes, "calls": ks_calls,
                  "avg_call_ms": ks_ms / ks_calls,
-                 "note": "reads the key once per call from DRAM; bound by shared-memory "
-                         "bandwidth (selected key rows delivered per gate), not HBM"}
+                 "note": "one-hot digits times fp16 key limbs on the tensor pipe; bound by "
+                         "the limbs' way from L2 (75 MB per 256 gates), not HBM"}
 
     # ---- configs 2 and 3 (device-resident inputs, L2 flushed before each
     # timed run, same keys and tuned shapes), each verified by decryption

@@ -316,7 +316,7 @@ typedef enum {
                              /*    autotuned, else by batch size                    */
     TFHE_OPT_SCHEDULE = 4,   /* tfhe_schedule policy of circuit schedules           */
     TFHE_OPT_LEVEL_WIDTH = 5,/* target gates per level for BALANCED (0: one wave    */
-                             /*    of 4 bootstraps per SM, or of 5 per SM (shape 5) */
+                             /*    of 4 bootstraps per SM, or one bootstrap per SM  */
                              /*    where the autotuner's wave times make that       */
                              /*    schedule cheaper)                                */
     TFHE_OPT_KS_KERNEL = 6,  /* key-switch kernel: 64 = tiled (64 gates per CTA, key */

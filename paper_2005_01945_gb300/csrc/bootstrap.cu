@@ -978,9 +978,9 @@ __device__ __forceinline__ void tb_release(uint32_t tmem, int warp)
 //              while V_1 runs once every warp has read V_0; then modulo q_1
 //   pointwise, inverse, CRT as warp (p, h)
 // Bound: the integer multiplies (IMAD 2, IMAD.HI and IMAD.WIDE 4 cycles of the
-// one pipe that has them): 4.2K cycles of that pipe per warp and step, busy 3/4
-// of the time.  608 gates with the key switch: 5.56 ms (109K bootstraps/s)
-// against 7.85 ms with both passes as unsigned butterflies.  The same first
+// one pipe that has them): 4.1K cycles of that pipe per warp and step, busy 80 %
+// of the time.  608 bootstraps: 5.36 ms (113K/s); with the key switch 5.56 ms when
+// that took 0.22, against 7.85 ms with both passes as unsigned butterflies.  The same first
 // pass in CTAs whose bootstraps run in lockstep took 7.4-8.1 ms: every wait and
 // table load stood alone.  The inverse's last pass on the tensor pipe too
 // (three limbs of each residue, CRT from the sums): 6.4 ms; the products take
