@@ -452,7 +452,8 @@ __device__ __forceinline__ bool bk_wait(unsigned long long *bar, uint32_t parity
     return false;
 }
 
-// Phase 4: CRT of (v0 mod q0, v1 mod q1), any representatives in [-8q, 8q), to
+// Phase 4: CRT of (v0 mod q0, v1 mod q1), any representatives within 8q of each
+// other (the signed inverse leaves [-q / 4, 5 q / 4], the others [0, 8q)), to
 // the centred integer, mod 2^32.  Garner: the exact coefficient S satisfies
 // |S| <= 4 N 2^9 2^31 = 2^52, so u = (S - v0) / q0 is an integer of magnitude
 // at most 2^25 + 8, about q1 / 4, and u = (v1 - v0) q0^-1 mod q1.  The
