@@ -325,9 +325,12 @@ typedef enum {
                              /*    or 0 (default): autotuned, else the tensor-pipe  */
                              /*    kernel above 64 gates and the tiled kernel up to */
                              /*    there (recorded by the autotuner as 64)          */
-    TFHE_OPT_TEST_FREE_HBM = 8,/* test hook for serving admission, 0 (default) off: */
-                             /*    a serving loop started afterwards takes this     */
-                             /*    many bytes as the device's free memory           */
+    TFHE_OPT_TEST_FREE_HBM = 8,/* test hook for short memory, 0 (default) off: a     */
+                             /*    serving loop started and keys set or loaded      */
+                             /*    afterwards take this many bytes as the device's  */
+                             /*    free memory (serving admission; the key limbs of */
+                             /*    the tensor-pipe key switch, 75.5 MB, without     */
+                             /*    which the tiled kernel runs in its place)        */
     TFHE_OPT_TEST_KS_STALL = 7 /* test hook for the timeout path, 0 (default) off:  */
                              /*    1 makes every stage of the tiled key switch also */
                              /*    wait on an mbarrier that nothing completes, so   */

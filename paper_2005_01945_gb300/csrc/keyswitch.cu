@@ -809,7 +809,8 @@ __global__ void __launch_bounds__(288, 1) k_keyswitch_tensor(const KsArgs A)
 // the key's rows (the tiled kernel).
 cudaError_t make_ksk_limbs(tfhe_ctx *ctx, cudaStream_t stream)
 {
-    if (!ctx->ksk_limb && cudaMalloc(&ctx->ksk_limb, kKlBytes) != cudaSuccess) {
+    const bool room = !ctx->test_free_hbm || ctx->test_free_hbm >= kKlBytes;
+    if (!ctx->ksk_limb && (!room || cudaMalloc(&ctx->ksk_limb, kKlBytes) != cudaSuccess)) {
         (void)cudaGetLastError();
         ctx->ksk_limb = nullptr;
         return cudaSuccess;
@@ -831,11 +832,14 @@ static thread_local int ks_forced_chunks = 0;
 // k_keyswitch.  A forced choice (autotuner, TFHE_OPT_KS_KERNEL) wins, then
 // the tuned value for the width bucket; untuned, or where the tuner kept the
 // default (recorded as kKsTiled), the tensor-pipe kernel above one tile of the
-// tiled one.  Up to there the two take 41 and 45 us alone, but behind a blind
+// tiled one.  A context without the key's limbs has the tiled kernel in the
+// tensor-pipe kernel's place, whoever asks for it.  Up to there the two take 41 and 45 us alone, but behind a blind
 // rotation the 75 MB of limbs come from further away than the 50 MB of rows: one
 // gate 1.645 ms with the limbs, 1.625 with the rows.
 static int ks_chunks(long count, int num_sms, const DevKeys *choice)
 {
+    if (ks_forced_chunks == kKsTensor)
+        return choice && choice->ksk_limb ? kKsTensor : kKsTiled;
     if (ks_forced_chunks)
         return ks_forced_chunks;
     if (choice && choice->ks_kernel > 0)

@@ -30,7 +30,7 @@ struct tfhe_ctx {
     std::string err;                 // last failure message (guarded by err_mu: the
     mutable std::mutex err_mu;       // serving calls fail from several threads)
     uint64_t launches = 0;           // kernels issued (graph nodes count per replay)
-    size_t test_free_hbm = 0;        // test hook: serving takes this as the free HBM
+    size_t test_free_hbm = 0;        // test hook: taken as the free HBM (serving, key limbs)
     tgb::CircuitCache *circuits = nullptr;
     tgb::Server *server = nullptr;
 };

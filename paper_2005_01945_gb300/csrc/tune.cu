@@ -2,8 +2,8 @@
 // kernels: the blind-rotation shape (4 independent bootstraps per CTA, one
 // bootstrap on a CTA's 16 warps, or one bootstrap on a cluster of two CTAs)
 // and the
-// key-switch kernel (the default, on the tensor pipe, recorded as 64, or
-// the direct kernel with its j-split of 1 .. 32 chunks), chosen per
+// key-switch kernel (the default, on the tensor pipe or, in a context without
+// the key's limbs, tiled; recorded as 64; or the direct kernel with its j-split of 1 .. 32 chunks), chosen per
 // level-width bucket by timing the candidates on synthetic ciphertexts
 // with the context's keys.  It also records the time of a level at each
 // bucket's widest width, from which the circuit schedules choose their

@@ -78,3 +78,33 @@ def test_extreme_limbs_and_sums(gpu, word, count):
         assert (got[3:] == got[0]).all()
     finally:
         ctx.close()
+
+
+def test_context_without_limbs(gpu, orc):
+    """Keys set while memory is too short for the key's limbs: the key switch
+    and the autotuner run on the key's rows, before and after tuning."""
+    torch, api, p = gpu["torch"], gpu["api"], gpu["p"]
+    g = synth._gen(32, "nolimb")
+    ksk = g.integers(0, 1 << 32, size=(N, T, D, p.n + 1), dtype=np.uint64).astype(np.uint32)
+    big = g.integers(0, 1 << 32, size=(608, api.BIG_STRIDE), dtype=np.uint64).astype(np.uint32)
+    want = orc.keyswitch(oparams(p), ksk, big[:, :N + 1])
+    bk_dev = api.to_device(np.zeros((p.n, 4, 2, N), dtype=np.uint32))
+    ksk_dev = api.to_device(ksk)
+    limbs = N * T * D * 512 * 3 * 2
+    ctx = api.Context(p)
+    try:
+        ctx.set_option(api.OPT_TEST_FREE_HBM, limbs - 1)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ctx.set_keys(bk_dev, ksk_dev)
+        ctx.set_option(api.OPT_TEST_FREE_HBM, 0)
+        # the transformed key and the padded rows alone
+        assert before - torch.cuda.mem_get_info()[0] < p.n * 4 * 2 * 2 * N * 4 + limbs // 3 * 2 + limbs // 2
+        assert np.array_equal(_run(gpu, ctx, big)[:, :p.n + 1], want)
+        ctx.autotune()
+        assert np.array_equal(_run(gpu, ctx, big)[:, :p.n + 1], want)
+        # with room again, the limbs come with the next keys
+        ctx.set_keys(bk_dev, ksk_dev)
+        assert np.array_equal(_run(gpu, ctx, big)[:, :p.n + 1], want)
+    finally:
+        ctx.close()
