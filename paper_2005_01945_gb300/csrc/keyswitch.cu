@@ -46,8 +46,8 @@ struct KsArgs {
     int j_chunk;              // j values per CTA (blockIdx.y selects the chunk)
     int atomic;               // 1: add into pre-initialised rows
     uint32_t *status;
-    long spin;                // tiled kernel: tries of one bounded mbarrier wait
-    int stall;                // tiled kernel, test hook: every stage's wait also waits
+    long spin;                // tiled, tensor: tries of one bounded mbarrier wait
+    int stall;                // tiled, tensor, test hook: every stage's wait also waits
                               // on a barrier that nothing completes, so it runs out
 };
 
@@ -514,6 +514,7 @@ struct KlSmem {
     uint8_t a[kKlStages][2][kKlABytes];
     uint8_t b[kKlStages][kKlBBytes];
     unsigned long long full_a[kKlStages], full_b[kKlStages], empty[kKlStages], done;
+    unsigned long long never;                             // test hook: never completes
     uint32_t tmem;
     volatile int abort;                                   // a wait ran out
 };
@@ -639,6 +640,7 @@ __global__ void __launch_bounds__(288, 1) k_keyswitch_tensor(const KsArgs A)
             mbar_init(&S.empty[s], 1);
         }
         mbar_init(&S.done, 1);
+        mbar_init(&S.never, 1);   // no thread ever arrives on it
         S.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -664,7 +666,9 @@ __global__ void __launch_bounds__(288, 1) k_keyswitch_tensor(const KsArgs A)
             for (int it = 0; it < np; ++it) {
                 const int s = it % kKlStages;
                 const uint32_t ph = (uint32_t)(it / kKlStages) & 1u;
-                left = !kl_wait(S, &S.full_b[s], ph, A.spin) || !kl_wait(S, &S.full_a[s], ph, A.spin);
+                left = !kl_wait(S, &S.full_b[s], ph, A.spin) ||
+                       !kl_wait(S, &S.full_a[s], ph, A.spin) ||
+                       (A.stall && !kl_wait(S, &S.never, 0u, A.spin));
                 if (left)
                     break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -721,8 +725,11 @@ __global__ void __launch_bounds__(288, 1) k_keyswitch_tensor(const KsArgs A)
 #pragma unroll
             for (int u = 0; u < 3; ++u, ++it) {
                 const int s = it % kKlStages;
-                ok = ok && (it < kKlStages ||
-                            kl_wait(S, &S.empty[s], (uint32_t)(it / kKlStages - 1) & 1u, A.spin));
+                // a wait may run out in one lane and not in another: the warp goes
+                // on, or leaves for the CTA's barrier, as one
+                ok = __all_sync(~0u, it < kKlStages ||
+                                         kl_wait(S, &S.empty[s], (uint32_t)(it / kKlStages - 1) & 1u,
+                                                 A.spin));
                 if (!ok)
                     break;
                 if (two || tid < 128) {
@@ -848,7 +855,7 @@ static int ks_chunks(long count, int num_sms, const DevKeys *choice)
     if (tuned > 0 && tuned != kKsTiled)
         return tuned;
     (void)num_sms;
-    return choice && choice->ksk_limb && !choice->ks_stall && count > kKtTile ? kKsTensor : kKsTiled;
+    return choice && choice->ksk_limb && count > kKtTile ? kKsTensor : kKsTiled;
 }
 
 // j-chunks of the tensor-pipe kernel: the split with the least CTA waves times
@@ -915,7 +922,7 @@ cudaError_t launch_keyswitch(const uint4 *ksk, const int32_t *big, int32_t *out,
     A.j_chunk = kN / chunks;
     A.atomic = chunks > 1;
     A.status = status;
-    const bool stall = tiled && choice && choice->ks_stall;
+    const bool stall = (tiled || tensor) && choice && choice->ks_stall;
     A.spin = stall ? kKtStallSpin : kKtSpin;
     A.stall = stall ? 1 : 0;
     if (A.atomic) {

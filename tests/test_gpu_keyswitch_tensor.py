@@ -108,3 +108,26 @@ def test_context_without_limbs(gpu, orc):
         assert np.array_equal(_run(gpu, ctx, big)[:, :p.n + 1], want)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("count", [65, 300])
+def test_wait_timeout_is_reported_and_recoverable(gpu, orc, count):
+    """Every stage's wait of the issuing thread runs out, and the waits of the
+    warps that write the one-hot rows run out or are called off: the kernel ends,
+    the status word says so (bit 2), and the next call is exact."""
+    api, p, torch = gpu["api"], gpu["p"], gpu["torch"]
+    g = synth._gen(33, "stall")
+    ksk = g.integers(0, 1 << 32, size=(N, T, D, p.n + 1), dtype=np.uint64).astype(np.uint32)
+    big = g.integers(0, 1 << 32, size=(count, api.BIG_STRIDE), dtype=np.uint64).astype(np.uint32)
+    want = orc.keyswitch(oparams(p), ksk, big[:, :N + 1])
+    ctx = _ctx(gpu, ksk)
+    try:
+        out = torch.zeros((count, 512), dtype=torch.int32, device="cuda")
+        for _ in range(3):
+            ctx.set_option(api.OPT_TEST_KS_STALL, 1)
+            ctx.keyswitch(api.to_device(big), out)
+            ctx.set_option(api.OPT_TEST_KS_STALL, 0)
+            assert ctx.status() == 4
+            assert np.array_equal(_run(gpu, ctx, big)[:, :p.n + 1], want)
+    finally:
+        ctx.close()
