@@ -332,9 +332,9 @@ typedef enum {
                              /*    the tensor-pipe key switch, 75.5 MB, without     */
                              /*    which the tiled kernel runs in its place)        */
     TFHE_OPT_TEST_KS_STALL = 7 /* test hook for the timeout path, 0 (default) off:  */
-                             /*    1 makes every stage of the tiled and of the      */
-                             /*    tensor-pipe key switch also wait on an mbarrier  */
-                             /*    that nothing completes, so                       */
+                             /*    1 makes every stage of the tiled key switch, and */
+                             /*    the first of the tensor-pipe one, also wait on an */
+                             /*    mbarrier that nothing completes, so              */
                              /*    each bounded wait runs out after a short budget; */
                              /*    the kernel then lets the copies it issued land,  */
                              /*    the call sets status bit 2 (timeout), its outputs */

@@ -47,7 +47,8 @@ struct KsArgs {
     int atomic;               // 1: add into pre-initialised rows
     uint32_t *status;
     long spin;                // tiled, tensor: tries of one bounded mbarrier wait
-    int stall;                // tiled, tensor, test hook: every stage's wait also waits
+    int stall;                // test hook: every stage of the tiled kernel and the first
+                              // of the tensor kernel also waits
                               // on a barrier that nothing completes, so it runs out
 };
 
@@ -660,15 +661,16 @@ __global__ void __launch_bounds__(288, 1) k_keyswitch_tensor(const KsArgs A)
         if (lane == 0) {
             const uint4 *limb = A.limb;
             int issued = 0;
-            bool left = false;   // a wait ran out
+            // a wait ran out (the test hook's stands before the stages: in each of
+            // them the unused branch cost 2.5 %)
+            bool left = A.stall && !kl_wait(S, &S.never, 0u, A.spin);
             for (; issued < kKlStages && issued < np; ++issued)
                 kl_load_b(S, limb, tile, p0 + issued, issued);
-            for (int it = 0; it < np; ++it) {
+            for (int it = 0; it < np && !left; ++it) {
                 const int s = it % kKlStages;
                 const uint32_t ph = (uint32_t)(it / kKlStages) & 1u;
                 left = !kl_wait(S, &S.full_b[s], ph, A.spin) ||
-                       !kl_wait(S, &S.full_a[s], ph, A.spin) ||
-                       (A.stall && !kl_wait(S, &S.never, 0u, A.spin));
+                       !kl_wait(S, &S.full_a[s], ph, A.spin);
                 if (left)
                     break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -721,18 +723,19 @@ __global__ void __launch_bounds__(288, 1) k_keyswitch_tensor(const KsArgs A)
                 cur[k] = live ? (nx[k] + (1u << 15)) >> 16 : 0u;   // rounded to 16 bits
             if (win + 1 < nw)
                 kl_window(nx, src + (win + 1) * kKlWin, live);
-            bool ok = true;
 #pragma unroll
             for (int u = 0; u < 3; ++u, ++it) {
                 const int s = it % kKlStages;
-                // a wait may run out in one lane and not in another: the warp goes
-                // on, or leaves for the CTA's barrier, as one
-                ok = __all_sync(~0u, it < kKlStages ||
-                                         kl_wait(S, &S.empty[s], (uint32_t)(it / kKlStages - 1) & 1u,
-                                                 A.spin));
-                if (!ok)
-                    break;
-                if (two || tid < 128) {
+                const bool go = it < kKlStages ||
+                                kl_wait(S, &S.empty[s], (uint32_t)(it / kKlStages - 1) & 1u, A.spin);
+                // a wait may run out in one lane and not in another, so no lane
+                // leaves: once the flag is set no wait takes time and the warp runs
+                // its stages out
+                if (!go && !S.abort) {
+                    S.abort = 1;
+                    atomicOr(A.status, kErrTimeout);
+                }
+                if (go && (two || tid < 128)) {
                     uint8_t *o = dst + s * (2 * kKlABytes);
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
@@ -747,13 +750,6 @@ __global__ void __launch_bounds__(288, 1) k_keyswitch_tensor(const KsArgs A)
                 if (lane == 0)
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&S.full_a[s]))
                                  : "memory");
-            }
-            if (!ok) {
-                if (!S.abort) {
-                    S.abort = 1;
-                    atomicOr(A.status, kErrTimeout);
-                }
-                break;
             }
         }
     }

@@ -112,7 +112,7 @@ def test_context_without_limbs(gpu, orc):
 
 @pytest.mark.parametrize("count", [65, 300])
 def test_wait_timeout_is_reported_and_recoverable(gpu, orc, count):
-    """Every stage's wait of the issuing thread runs out, and the waits of the
+    """The issuing thread's first wait runs out, and the waits of the
     warps that write the one-hot rows run out or are called off: the kernel ends,
     the status word says so (bit 2), and the next call is exact."""
     api, p, torch = gpu["api"], gpu["p"], gpu["torch"]
