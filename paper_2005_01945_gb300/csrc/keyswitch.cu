@@ -48,8 +48,8 @@ struct KsArgs {
     uint32_t *status;
     long spin;                // tiled, tensor: tries of one bounded mbarrier wait
     int stall;                // test hook: every stage of the tiled kernel and the first
-                              // of the tensor kernel also waits
-                              // on a barrier that nothing completes, so it runs out
+                              // of the tensor kernel also waits on a barrier that nothing
+                              // completes, so the wait runs out
 };
 
 __device__ __forceinline__ long ks_dest(const KsArgs &A, long g)
@@ -509,6 +509,7 @@ constexpr int kKlStages = 4;
 constexpr uint32_t kKlBBytes = kKlCols * 128;             // 24 KB of limbs
 constexpr uint32_t kKlABytes = 128 * 128;                 // 16 KB of one-hot rows (128 gates)
 constexpr int kKlRow = kKlWords + 1;                      // words of a transposed result row
+constexpr long kKlMaxGates = 65535L * kKlGates;           // gates of a launch (grid z)
 static_assert(kKlBytes == (size_t)(kLweStride / kKlWords) * kKlUnits * kKlBBytes, "limb bytes");
 
 struct KlSmem {
@@ -890,7 +891,8 @@ int keyswitch_kernels(long count, int num_sms, const DevKeys *choice)
     if (c == kKsTiled)
         return kt_chunks(count, num_sms) > 1 ? 2 : 1;
     if (c == kKsTensor)
-        return kl_chunks(count, num_sms) > 1 ? 2 : 1;
+        return (kl_chunks(count, num_sms) > 1 ? 1 : 0) +
+               (int)((count + kKlMaxGates - 1) / kKlMaxGates);
     return c > 1 ? 2 : 1;
 }
 
@@ -939,10 +941,24 @@ cudaError_t launch_keyswitch(const uint4 *ksk, const int32_t *big, int32_t *out,
                 return e;
             prepared[dev] = 1;
         }
-        dim3 grid((unsigned)chunks, (unsigned)(kLweStride / kKlWords),
-                  (unsigned)((count + kKlGates - 1) / kKlGates));
-        k_keyswitch_tensor<<<grid, 288, sizeof(KlSmem), stream>>>(A);
-        return cudaGetLastError();
+        // a launch per 16.8M gates, on rows of its own
+        for (long first = 0; first < count; first += kKlMaxGates) {
+            A.count = count - first < kKlMaxGates ? count - first : kKlMaxGates;
+            A.big = big + first * kBigStride;
+            if (idx_out) {
+                A.idx_out = idx_out + first;
+            } else {
+                A.out = out + first * kLweStride;
+                A.rows_out = rows_out - first;
+            }
+            dim3 grid((unsigned)chunks, (unsigned)(kLweStride / kKlWords),
+                      (unsigned)((A.count + kKlGates - 1) / kKlGates));
+            k_keyswitch_tensor<<<grid, 288, sizeof(KlSmem), stream>>>(A);
+            cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess)
+                return e;
+        }
+        return cudaSuccess;
     }
     if (tiled) {
         static int prepared[64] = {0};

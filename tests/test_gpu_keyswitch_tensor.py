@@ -131,3 +131,36 @@ def test_wait_timeout_is_reported_and_recoverable(gpu, orc, count):
             assert np.array_equal(_run(gpu, ctx, big)[:, :p.n + 1], want)
     finally:
         ctx.close()
+
+
+def test_beyond_65535_gate_tiles(gpu, orc):
+    """More gate tiles than the smaller grid dimensions hold (65,535 x 256
+    samples), around that edge and in the last, ragged tile."""
+    torch, api, p = gpu["torch"], gpu["api"], gpu["p"]
+    edge = 65535 * 256
+    count = edge + 257
+    if torch.cuda.mem_get_info()[0] < count * (api.BIG_STRIDE + 512) * 4 + (4 << 30):
+        pytest.skip("needs 107 GB of free device memory")
+    g = synth._gen(34, "many")
+    ksk = g.integers(0, 1 << 32, size=(N, T, D, p.n + 1), dtype=np.uint64).astype(np.uint32)
+    sample = np.array([0, 255, 256, edge - 1, edge, edge + 255, edge + 256])
+    rows = g.integers(0, 1 << 32, size=(len(sample), api.BIG_STRIDE), dtype=np.uint64)
+    rows = rows.astype(np.uint32)
+    want = orc.keyswitch(oparams(p), ksk, np.ascontiguousarray(rows[:, :N + 1]))
+    ctx = _ctx(gpu, ksk)
+    try:
+        big = torch.zeros((count, api.BIG_STRIDE), dtype=torch.int32, device="cuda")
+        for s, r in zip(sample, rows):
+            big[int(s)].copy_(api.to_device(r))
+        out = torch.full((count, 512), 7, dtype=torch.int32, device="cuda")
+        ctx.keyswitch(big, out)
+        torch.cuda.synchronize()
+        assert ctx.status() == 0
+        got = np.stack([out[int(s)].cpu().numpy() for s in sample]).view(np.uint32)
+        assert np.array_equal(got[:, :p.n + 1], want)
+        assert not got[:, p.n + 1:].any()
+        assert not out[1:255].any() and not out[edge + 1:edge + 255].any()   # zero samples
+    finally:
+        big = out = None
+        torch.cuda.empty_cache()
+        ctx.close()
