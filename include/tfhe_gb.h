@@ -331,7 +331,7 @@ typedef enum {
                              /*    free memory (serving admission; the key limbs of */
                              /*    the tensor-pipe key switch, 75.5 MB, without     */
                              /*    which the tiled kernel runs in its place)        */
-    TFHE_OPT_TEST_KS_STALL = 7 /* test hook for the timeout path, 0 (default) off:  */
+    TFHE_OPT_TEST_KS_STALL = 7,/* test hook for the timeout path, 0 (default) off:  */
                              /*    1 makes every stage of the tiled key switch, and */
                              /*    the first of the tensor-pipe one, also wait on an */
                              /*    mbarrier that nothing completes, so              */
@@ -339,6 +339,14 @@ typedef enum {
                              /*    the kernel then lets the copies it issued land,  */
                              /*    the call sets status bit 2 (timeout), its outputs */
                              /*    are undefined, and the context stays usable     */
+    TFHE_OPT_TEST_BR_STALL = 9 /* test hook for the blind rotation's timeout path, */
+                             /*    0 (default) off: k > 0 makes the wait for the   */
+                             /*    k-th tensor-pipe product of a bootstrap's slot  */
+                             /*    run out after about a second (shape 1; shape 8: */
+                             /*    the k-th CMux step's second product); no        */
+                             /*    further work is issued, the product in flight   */
+                             /*    is waited for, and the rest is as for           */
+                             /*    TFHE_OPT_TEST_KS_STALL                          */
 } tfhe_option;
 
 int tfhe_ctx_set_option(tfhe_ctx *ctx, int option, int64_t value);

@@ -117,7 +117,7 @@ EXPORTS = {
 GATE, ADD, MUL, MATVEC, ADD_MAJ, ADD_NW, MUL_TREE, MUL_FULL, MUL_KARATSUBA, MUL_TREE_MAJ, \
     ADD_PREFIX, MUL_DADDA = range(12)
 OPT_GRAPHS, OPT_PER_GATE, OPT_PROFILE, OPT_BR_GROUP, OPT_SCHEDULE, OPT_LEVEL_WIDTH, \
-    OPT_KS_KERNEL, OPT_TEST_KS_STALL, OPT_TEST_FREE_HBM = range(9)
+    OPT_KS_KERNEL, OPT_TEST_KS_STALL, OPT_TEST_FREE_HBM, OPT_TEST_BR_STALL = range(10)
 KS_TILED = 64   # OPT_KS_KERNEL value of the tiled key-switch kernel
 SCHED_ASAP, SCHED_BALANCED = 0, 1
 

@@ -419,14 +419,16 @@ struct BrArgs {
     uint32_t *status;
 };
 
-constexpr long kBkSpin = 1L << 20;                           // x ~1 us per try
+// Tries of a bounded wait, about 4 us each: about a second (a constant: with the
+// limit as an argument the two-CTA shape took 1.7 % longer).
+constexpr long kBkSpin = 1L << 18;
 
 __device__ __forceinline__ uint32_t br_saddr(const void *p)
 {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// Bounded wait for phase `parity` of a stage barrier; false if it ran out.
+// Bounded wait for phase `parity` of a barrier; false if it ran out.
 __device__ __forceinline__ bool bk_wait(unsigned long long *bar, uint32_t parity)
 {
     uint32_t ok;
@@ -631,8 +633,10 @@ struct TbOps {                  // one CTA
     uint8_t b1[kTbCols * 16 * 2];   // the K step of the accumulators' start value
     uint8_t a1[128 * 16 * 2];
     unsigned long long bar[4];  // MMA completion of each bootstrap
+    unsigned long long spare[4];    // test hook: completion of the product whose wait runs out
     uint32_t tmem;
     volatile int abort[4];      // a wait of the bootstrap ran out
+    int skipped[4];             // ... and the step's second product was not issued
 };
 
 // Barrier of the 128 threads of bootstrap slot `bi`.
@@ -915,7 +919,10 @@ __device__ __forceinline__ void tb_setup(const BrArgs &A, TbOps &O, int tid, int
     if (tid < 4) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(br_saddr(&O.bar[tid]))
                      : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(br_saddr(&O.spare[tid]))
+                     : "memory");
         O.abort[tid] = 0;
+        O.skipped[tid] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -1026,7 +1033,8 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
             boot_sync(bi);
             if (tb == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                tb_mma(acc_cols, dig_op, O, 0, &O.bar[bi]);
+                tb_mma(acc_cols, dig_op, O, 0,
+                       phase + 1 == (uint32_t)A.keys.br_stall ? &O.spare[bi] : &O.bar[bi]);
             }
             int32_t x[32];
             const uint4 *bki = A.keys.bk_ntt + (((long)i * 2 + p) * 2 + h) * 1024;
@@ -1036,8 +1044,11 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
             for (int ph = 0; ph < 2; ++ph) {
                 const Prime pq((uint32_t)ph);
                 uint32_t *sl = S.fwd[ph][wr];
-                if (!bk_wait(&O.bar[bi], phase & 1)) {
+                const bool done = bk_wait(&O.bar[bi], phase & 1);
+                if (!done) {
                     O.abort[bi] = 1;
+                    if (ph == 0 && tb == 0)
+                        O.skipped[bi] = 1;
                     atomicOr(A.status, kErrTimeout);
                 }
                 ++phase;
@@ -1046,12 +1057,14 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
                 tb_combine(tl + bi * kTbCols, tl + kTbTw + 64 * ph, sl + lane * kRowV, pq);
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 if (ph == 0) {
-                    // V_1 overwrites V_0 once the four warps have read it
+                    // V_1 overwrites V_0 once the four warps have read it (and not
+                    // where the issuing thread's wait for V_0 ran out)
                     if (wr == 0) {
                         asm volatile("bar.sync %0, 128;" ::"r"(5 + bi) : "memory");
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        if (lane == 0)
-                            tb_mma(acc_cols, dig_op, O, 1, &O.bar[bi]);
+                        if (lane == 0 && done)
+                            tb_mma(acc_cols, dig_op, O, 1,
+                                   phase + 1 == (uint32_t)A.keys.br_stall ? &O.spare[bi] : &O.bar[bi]);
                     } else {
                         asm volatile("bar.arrive %0, 128;" ::"r"(5 + bi) : "memory");
                     }
@@ -1081,10 +1094,15 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
             br_extract<T>(A, g, S.acc, tb);
         boot_sync(bi);
     }
-    // after a wait that ran out: a product still in flight gets a bounded
-    // time to finish before TMEM is freed
-    if (O.abort[bi] && tb == 0)
-        (void)bk_wait(&O.bar[bi], (phase + 1) & 1);
+    // after a wait that ran out: the last product issued, the only one that may
+    // still be in flight, gets a bounded time to finish before TMEM is freed
+    if (O.abort[bi] && tb == 0) {
+        const uint32_t last = phase - 1 - (uint32_t)O.skipped[bi];
+        if (last + 1 == (uint32_t)A.keys.br_stall)
+            (void)bk_wait(&O.spare[bi], 0);
+        else
+            (void)bk_wait(&O.bar[bi], last & 1);
+    }
     tb_release(tmem, warp);
 }
 
@@ -1308,7 +1326,8 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_wide(const BrArgs A)
 #pragma unroll
     for (int e = 0; e < 8; ++e)
         tw[e] = __ldg(A.keys.twb + ((h * 2 + 1) * 32 + 2 * z + (e & 1) + 8 * (e >> 1)) * 32 + lane);
-    uint32_t phase = 0;
+    uint32_t phase = 0;   // executed CMux steps
+    const uint32_t stall = (uint32_t)A.keys.br_stall;   // test hook: V_1 of this step (from 1)
 
     for (long g = A.first + blockIdx.x; g < A.count && !O.abort[0]; g += gridDim.x) {
         const bool active = br_prologue<512>(A, g, tid, S.abar, true);
@@ -1331,7 +1350,8 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_wide(const BrArgs A)
             if (tid == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 tb_mma(tmem, br_saddr(S.dig), O, 0, &O.bar[0]);
-                tb_mma(tmem + kTbCols, br_saddr(S.dig), O, 1, &O.bar[1]);
+                tb_mma(tmem + kTbCols, br_saddr(S.dig), O, 1,
+                       phase + 1 == stall ? &O.spare[1] : &O.bar[1]);
             }
             uint4 kv[8];
             const uint4 *bki = A.keys.bk_ntt + (((long)i * 2 + p) * 2 + h) * 1024 + 8 * z * 32 + lane;
@@ -1393,9 +1413,13 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_wide(const BrArgs A)
     }
     // after a wait that ran out: products still in flight get a bounded time
     // to finish before TMEM is freed
-    if (O.abort[0] && tid == 0)
-        for (int b = 0; b < 2; ++b)
-            (void)bk_wait(&O.bar[b], (phase + 1) & 1);
+    if (O.abort[0] && tid == 0) {
+        (void)bk_wait(&O.bar[0], (phase - 1) & 1);
+        if (phase == stall)
+            (void)bk_wait(&O.spare[1], 0);
+        else
+            (void)bk_wait(&O.bar[1], (phase - 1) & 1);
+    }
     tb_release(tmem, warp);
 }
 

@@ -1344,6 +1344,12 @@ int tfhe_ctx_set_option(tfhe_ctx *ctx, int option, int64_t value)
         ctx->keys.ks_stall = value != 0;
         invalidate_graphs(ctx);
         return TFHE_OK;
+    case TFHE_OPT_TEST_BR_STALL:
+        if (value < 0 || value > INT32_MAX)
+            return fail(ctx, TFHE_EINVAL, "TFHE_OPT_TEST_BR_STALL must be >= 0");
+        ctx->keys.br_stall = (int)value;
+        invalidate_graphs(ctx);
+        return TFHE_OK;
     case TFHE_OPT_KS_KERNEL:
         if (value != 0 && value != kKsTiled &&
             !(value >= 1 && value <= 32 && (value & (value - 1)) == 0))
