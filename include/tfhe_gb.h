@@ -343,9 +343,11 @@ typedef enum {
                              /*    0 (default) off: k > 0 makes the wait for the   */
                              /*    k-th tensor-pipe product of a bootstrap's slot  */
                              /*    run out after about a second (shape 1; shape 8: */
-                             /*    the k-th CMux step's second product); no        */
-                             /*    further work is issued, the product in flight   */
-                             /*    is waited for, and the rest is as for           */
+                             /*    the k-th CMux step's second product; shape 16:  */
+                             /*    the first product of the call's k-th gate, in   */
+                             /*    its second CTA, where an even number of steps   */
+                             /*    went before).  The kernel ends early and waits  */
+                             /*    for what is in flight; the rest is as for       */
                              /*    TFHE_OPT_TEST_KS_STALL                          */
 } tfhe_option;
 

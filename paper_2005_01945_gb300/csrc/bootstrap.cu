@@ -634,8 +634,10 @@ struct TbOps {                  // one CTA
     uint8_t a1[128 * 16 * 2];
     unsigned long long bar[4];  // MMA completion of each bootstrap
     unsigned long long spare[4];    // test hook: completion of the product whose wait runs out
+                                    // (two-CTA shape: of all, after a wait that ran out)
     uint32_t tmem;
-    volatile int abort[4];      // a wait of the bootstrap ran out
+    volatile int abort[4];      // a wait of the bootstrap ran out (two-CTA shape: in this
+                                // step, from 1)
     int skipped[4];             // ... and the step's second product was not issued
 };
 
@@ -1441,8 +1443,12 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_wide(const BrArgs A)
 // step.  Their buffers alternate by executed CMux: one is rewritten two steps
 // after it was read, and the sender of the later step has waited for what the
 // reader sent in the step between.  Control flow is the same in both CTAs (same
-// gate, same abar, no branch on a wait that ran out), so each step's stores are
-// sent by both.
+// gate, same abar), so each step's stores are sent by both.
+// A CTA whose wait runs out executes one more step, without waiting, and ends; its
+// partner's next wait for residues then runs out, and it ends the same way.  Both
+// meet before they end, and each gives what is still on its way into it a bounded
+// time (pair_drain).  (The flag tested at other places of the step: one gate 1.64 to
+// 1.67 ms, so 1.61.)
 // Bound: the chain of a step (6.3K cycles, the multiply pipe busy half of them,
 // seven barriers and two waits).  One gate 1.65 ms against 2.05 ms on one CTA;
 // the shape it replaces (8 warps per CTA, butterflies in the first pass, key
@@ -1523,6 +1529,28 @@ __device__ __forceinline__ void ct32_cyc_block(uint32_t (&y)[8], const uint32_t 
         y[e] = csub(y[e], pr.kq(8));
 }
 
+// After a wait that ran out, one thread, behind the cluster's last barrier (both
+// CTAs have issued all they will): products and residues still on their way get a
+// bounded time before TMEM and shared memory are freed.  `steps` were executed
+// here; the partner's wait for the residues of the next one runs out, and it sends
+// its own of that one and of one more.
+__device__ __forceinline__ void pair_drain(PairSmem &S, TbOps &O, uint32_t steps)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                     br_saddr(&O.spare[0]))
+                 : "memory");
+    (void)bk_wait(&O.spare[0], 0);
+    for (uint32_t s = steps < 2 ? 0 : steps - 2; s < steps + 2; ++s) {
+        unsigned long long *bar = &S.got[s & 1];
+        if (s >= steps)   // the step has not posted its bytes: the partner's half
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(br_saddr(bar)),
+                         "r"(kPairBytes / 2)
+                         : "memory");
+        if (!bk_wait(bar, (s >> 1) & 1))
+            return;   // the partner has sent nothing further
+    }
+}
+
 __global__ void __launch_bounds__(512, 1) k_blind_rotate_pair(const BrArgs A)
 {
     extern __shared__ uint4 smem_raw[];
@@ -1554,8 +1582,15 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_pair(const BrArgs A)
     }
     cl.sync();   // the partner's shared memory and barriers are there
 
-    for (long g = A.first + cid; g < A.count; g += nclusters) {
+    for (long g = A.first + cid; g < A.count && !O.abort[0]; g += nclusters) {
         const bool active = br_prologue<512>(A, g, tid, S.abar, rank == 0);
+        if (tid == 0 && rank == 1 && g + 1 == A.keys.br_stall && !(phase & 1)) {
+            // test hook: two products complete a phase from here on (phases restart
+            // at 0), so the wait for the next one runs out
+            asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(br_saddr(&O.bar[0])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"(br_saddr(&O.bar[0])) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
         __syncthreads();
         br_acc_init<512>(A, S.acc, S.abar[n], tid);
         __syncthreads();
@@ -1566,8 +1601,13 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_pair(const BrArgs A)
 
         for (int i = 0; i < n; ++i) {
             const int a = S.abar[i];
+            const uint32_t left = (uint32_t)O.abort[0] - 1u;
             if (a == 0)
                 continue;   // X^0 acc - acc = 0: nothing changes
+            // a wait ran out in the step before the last one: every thread finds
+            // that here, where one of the last step may not be seen by all
+            if (left < phase - 1u)
+                break;
             const uint32_t use = phase++;
             const int par = use & 1;
             wide_digits(S.acc[p], own, S.dig + z * 2048 + (64 * p + lane) * 16 + 8 * (q & 1), c_lo,
@@ -1591,7 +1631,7 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_pair(const BrArgs A)
                     kv[e] = __ldg(bki + e * 32);
             }
             if (!O.abort[0] && !bk_wait(&O.bar[0], use & 1)) {
-                O.abort[0] = 1;   // wait no more; the status word has it
+                O.abort[0] = (int)phase;   // wait no more; the status word has it
                 atomicOr(A.status, kErrTimeout);
             }
             __syncwarp();
@@ -1623,7 +1663,7 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_pair(const BrArgs A)
                 }
             }
             if (!O.abort[0] && !bk_wait(&S.got[par], (use >> 1) & 1)) {
-                O.abort[0] = 1;
+                O.abort[0] = (int)phase;
                 atomicOr(A.status, kErrTimeout);
             }
             {
@@ -1642,17 +1682,13 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_pair(const BrArgs A)
             warps_sync<256>(13 + p);
         }
         __syncthreads();
-        if (active && rank == 0)
+        if (active && rank == 0 && !O.abort[0])
             br_extract<512>(A, g, S.acc, tid);
         __syncthreads();
     }
-    // after a wait that ran out: a product and stores still in flight get a
-    // bounded time to finish before TMEM and shared memory are freed
-    if (O.abort[0] && tid == 0 && phase) {
-        (void)bk_wait(&O.bar[0], (phase - 1) & 1);
-        (void)bk_wait(&S.got[(phase - 1) & 1], ((phase - 1) >> 1) & 1);
-    }
     cl.sync();   // neither CTA ends while the other may write to it
+    if (O.abort[0] && tid == 0)
+        pair_drain(S, O, phase);
     tb_release(tmem, warp);
 }
 

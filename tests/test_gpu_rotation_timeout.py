@@ -31,14 +31,19 @@ def gpu(orc):
 
 
 # shape 1: the first and the second product of a step, of the first step and of a
-# later one; 700 gates: two gates per slot
+# later one; 700 gates: two gates per slot.  Shape 16: a product of a gate's second
+# CTA, so that the first one's wait for residues runs out two steps later; of a gate
+# with one step, behind which the first CTA ends by itself; of a cluster's second gate
 @pytest.mark.parametrize("shape,count,products", [(1, 3, (1, 2, 5, 6)), (1, 700, (1, 2, 47, 60)),
-                                                  (8, 3, (1, 2, 20)), (8, 200, (1, 30))])
+                                                  (8, 3, (1, 2, 20)), (8, 200, (1, 30)),
+                                                  (16, 3, (1, 2, 3)), (16, 100, (1, 3, 77, 100))])
 def test_timeout_is_reported_and_recoverable(gpu, orc, shape, count, products):
     torch, api, p, P, ctx = gpu["torch"], gpu["api"], gpu["p"], gpu["P"], gpu["ctx"]
     g = synth._gen(37, f"stall{shape}{count}")
     cts = g.integers(0, 1 << 32, size=(count, 512), dtype=np.uint64).astype(np.uint32)
-    cts[:, :p.n] |= 1 << 22                # every step rotates
+    cts[:, :p.n] = cts[:, :p.n] & 0x7FFFFFFF | 1 << 22     # every step rotates
+    cts[2, :p.n] = 0
+    cts[2, 5] = 1 << 30                    # one step
     cts[:, p.n + 1:] = 0
     want = orc.bootstrap(P, gpu["bk"], gpu["ksk"], cts[:, :p.n + 1], mu=1 << 29)
     dev = api.to_device(cts)
