@@ -137,6 +137,32 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
         const int saved_group = K.br_group;
         int8_t br[8] = {0}, ks[8] = {0};
         float level_ms[8] = {0.f};
+        // Blind rotation of W gates in the shape K.br_group: best of three timed
+        // runs after a warm-up, as one slow run (a first launch of a kernel, a
+        // clock step) must not decide the 2 % rule below.  Each run follows a key
+        // switch (not timed), as every level of a circuit does: its key stream
+        // leaves the bootstrapping key partly out of L2, which is the state the
+        // shapes have to cope with.
+        auto br_time = [&](long W) -> float {
+            float best_ms = 1e30f;
+            for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {
+                e = launch_keyswitch(K.ksk, big, out, nullptr, W, W, ctx->prm.n, ctx->num_sms,
+                                     ctx->status, st, &K);
+                if (e == cudaSuccess)
+                    e = cudaEventRecord(e0, st);
+                if (e == cudaSuccess)
+                    e = launch_blind_rotate(K, nullptr, cts, nullptr, W, nullptr, nullptr, 0, big,
+                                            W, kMu, ctx->status, ctx->br_grid, st);
+                if (e == cudaSuccess)
+                    e = cudaEventRecord(e1, st);
+                if (e == cudaSuccess)
+                    e = cudaEventSynchronize(e1);
+                float ms = 0;
+                if (e == cudaSuccess && rep > 0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
+                    best_ms = ms < best_ms ? ms : best_ms;   // first run is a warm-up
+            }
+            return best_ms;
+        };
         for (int b = 0; b < 8 && e == cudaSuccess; ++b) {
             const long W = widths[b];
             // the latency shapes first: a later candidate is kept only if it
@@ -148,29 +174,7 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
                 if (B != 1 && W > 2L * ctx->num_sms)
                     continue;
                 K.br_group = B;
-                // best of three timed runs after a warm-up: one slow run
-                // (a first launch of a kernel, a clock step) must not
-                // decide the 2 % rule.  Each run follows a key switch (not
-                // timed), as every level of a circuit does: its 50 MB key
-                // stream leaves the bootstrapping key partly out of L2,
-                // which is the state the shapes have to cope with.
-                float tot = 1e30f;
-                for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {
-                    e = launch_keyswitch(K.ksk, big, out, nullptr, W, W, ctx->prm.n, ctx->num_sms,
-                                         ctx->status, st, &K);
-                    if (e == cudaSuccess)
-                        e = cudaEventRecord(e0, st);
-                    if (e == cudaSuccess)
-                        e = launch_blind_rotate(K, nullptr, cts, nullptr, W, nullptr, nullptr, 0,
-                                                big, W, kMu, ctx->status, ctx->br_grid, st);
-                    if (e == cudaSuccess)
-                        e = cudaEventRecord(e1, st);
-                    if (e == cudaSuccess)
-                        e = cudaEventSynchronize(e1);
-                    float ms = 0;
-                    if (e == cudaSuccess && rep > 0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
-                        tot = ms < tot ? ms : tot;   // first run is a warm-up
-                }
+                const float tot = br_time(W);
                 if (e == cudaSuccess && (br[b] == 0 || tot < 0.98f * best)) {
                     best = tot;
                     br[b] = (int8_t)B;
@@ -203,9 +207,15 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
                 }
             }
         }
-        // one full wave (4 bootstraps per SM) is bucket 2's widest level: the
-        // level schedules cost wider levels in waves
-        K.wave_ms[0] = level_ms[tune_bucket(4L * ctx->num_sms)];
+        // one full wave, 4 bootstraps per SM: the level schedules cost wider levels
+        // in waves.  On 152 SMs it is the widest level of its bucket
+        const long w4 = 4L * ctx->num_sms;
+        const int wb = tune_bucket(w4);
+        K.wave_ms[0] = level_ms[wb];
+        if (w4 != widths[wb] && w4 <= maxw && e == cudaSuccess) {
+            K.br_group = br[wb];
+            K.wave_ms[0] = br_time(w4);
+        }
         K.wave_ms[1] = 0.f;
         std::memcpy(K.tune_ms, level_ms, sizeof(level_ms));
         K.br_group = saved_group;
