@@ -1984,7 +1984,7 @@ static long br_tail(long count, long nsm, int forced, int shape)
 cudaError_t launch_blind_rotate(const DevKeys &keys, const uint8_t *ops, const int32_t *in_a,
                                 const int32_t *idx_a, long rows_a, const int32_t *in_b,
                                 const int32_t *idx_b, long rows_b, int32_t *big, long count,
-                                uint32_t mu, uint32_t *status, int grid, cudaStream_t stream,
+                                uint32_t mu, uint32_t *status, cudaStream_t stream,
                                 const int32_t *in_c, const int32_t *idx_c, long rows_c)
 {
     if (count <= 0)
@@ -2009,7 +2009,6 @@ cudaError_t launch_blind_rotate(const DevKeys &keys, const uint8_t *ops, const i
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long nsm = sms > 0 ? sms : 1;
-    (void)grid;
     const int shape = br_group(count, (int)nsm, keys.br_group, keys.tune_br);
     const long tail = br_tail(count, nsm, keys.br_group, shape);
     A.first = 0;

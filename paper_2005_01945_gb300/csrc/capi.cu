@@ -93,7 +93,7 @@ int run_bootstrap(tfhe_ctx *ctx, const uint8_t *ops, const int32_t *a, const int
     {
         NvtxRange r("tfhe: gate combine + mod switch + blind rotation + extraction");
         e = launch_blind_rotate(ctx->keys, ops, a, idx_a, rows_a, b, idx_b, rows_b, ctx->big,
-                                count, mu, ctx->status, ctx->br_grid, stream);
+                                count, mu, ctx->status, stream);
     }
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "blind rotation launch");
@@ -146,7 +146,6 @@ int tfhe_ctx_create(const tfhe_params *params, int device, tfhe_ctx **out)
         tfhe_ctx_destroy(ctx);
         return e == cudaErrorMemoryAllocation ? TFHE_ENOMEM : TFHE_ECUDA;
     }
-    ctx->br_grid = 4 * ctx->num_sms;
     ctx->keys.twb = ctx->twb;
     ctx->keys.tb_op = ctx->tb_op;
     ctx->keys.n = params->n;
@@ -298,7 +297,7 @@ int tfhe_blind_rotate_extract(tfhe_ctx *ctx, const uint8_t *ops, const int32_t *
     DeviceGuard dg(ctx->device);
     cudaError_t e = launch_blind_rotate(ctx->keys, ops, a, nullptr, (long)count, b, nullptr,
                                         (long)count, big, (long)count, kMu, ctx->status,
-                                        ctx->br_grid, (cudaStream_t)stream);
+                                        (cudaStream_t)stream);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "blind rotation launch");
     ctx->launches += blind_rotate_kernels((long)count, ctx->num_sms, ctx->keys);

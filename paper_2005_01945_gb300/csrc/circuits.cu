@@ -975,7 +975,7 @@ static cudaError_t enqueue_levels(tfhe_ctx *ctx, Plan &P, cudaStream_t st, bool 
         if (e == cudaSuccess)
             e = launch_blind_rotate(ctx->keys, P.d_ops + off, P.pool, P.d_ia + off, P.pool_rows,
                                     P.pool, P.d_ib + off, P.pool_rows, P.big, cnt, kMu,
-                                    ctx->status, ctx->br_grid, st, P.d_ic ? P.pool : nullptr,
+                                    ctx->status, st, P.d_ic ? P.pool : nullptr,
                                     P.d_ic ? P.d_ic + off : nullptr, P.pool_rows);
         if (e == cudaSuccess)
             e = mark(3 * (l - 1) + 1);
@@ -999,7 +999,7 @@ static cudaError_t enqueue_per_gate(tfhe_ctx *ctx, Plan &P, cudaStream_t st)
     for (long k = 0; k < P.gates; ++k) {
         cudaError_t e = launch_blind_rotate(ctx->keys, P.d_ops + k, P.pool, P.d_ia + k, P.pool_rows,
                                             P.pool, P.d_ib + k, P.pool_rows, P.big, 1, kMu,
-                                            ctx->status, ctx->br_grid, st,
+                                            ctx->status, st,
                                             P.d_ic ? P.pool : nullptr,
                                             P.d_ic ? P.d_ic + k : nullptr, P.pool_rows);
         if (e != cudaSuccess)

@@ -840,7 +840,7 @@ static thread_local int ks_forced_chunks = 0;
 // tensor-pipe kernel's place, whoever asks for it.  Up to there the two take 41 and 45 us alone, but behind a blind
 // rotation the 75 MB of limbs come from further away than the 50 MB of rows: one
 // gate 1.645 ms with the limbs, 1.625 with the rows.
-static int ks_chunks(long count, int num_sms, const DevKeys *choice)
+static int ks_chunks(long count, const DevKeys *choice)
 {
     if (ks_forced_chunks == kKsTensor)
         return choice && choice->ksk_limb ? kKsTensor : kKsTiled;
@@ -851,7 +851,6 @@ static int ks_chunks(long count, int num_sms, const DevKeys *choice)
     const int tuned = choice ? choice->tune_ks[tune_bucket(count)] : 0;
     if (tuned > 0 && tuned != kKsTiled)
         return tuned;
-    (void)num_sms;
     return choice && choice->ksk_limb && count > kKtTile ? kKsTensor : kKsTiled;
 }
 
@@ -887,7 +886,7 @@ int keyswitch_kernels(long count, int num_sms, const DevKeys *choice)
 {
     if (count <= 0)
         return 0;
-    const int c = ks_chunks(count, num_sms, choice);
+    const int c = ks_chunks(count, choice);
     if (c == kKsTiled)
         return kt_chunks(count, num_sms) > 1 ? 2 : 1;
     if (c == kKsTensor)
@@ -903,7 +902,7 @@ cudaError_t launch_keyswitch(const uint4 *ksk, const int32_t *big, int32_t *out,
 {
     if (count <= 0)
         return cudaSuccess;
-    const int pick = ks_chunks(count, num_sms, choice);
+    const int pick = ks_chunks(count, choice);
     const bool tiled = pick == kKsTiled;
     const bool tensor = pick == kKsTensor;
     const int chunks = tiled ? kt_chunks(count, num_sms)

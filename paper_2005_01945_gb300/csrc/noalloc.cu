@@ -124,7 +124,7 @@ extern "C" int tfhe_bootstrap_gates_noalloc(tfhe_ctx *ctx, const uint8_t *ops, c
     cudaStream_t st = (cudaStream_t)stream;
     NvtxRange range("tfhe: gate bootstrapping (fixed scratch)");
     cudaError_t e = launch_blind_rotate(ctx->keys, ops, a, nullptr, n, b, nullptr, n, big, n, kMu,
-                                        ctx->status, ctx->br_grid, st);
+                                        ctx->status, st);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "blind rotation launch");
     e = launch_keyswitch(ctx->keys.ksk, big, out, nullptr, n, n, ctx->prm.n, ctx->num_sms,

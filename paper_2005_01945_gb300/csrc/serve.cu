@@ -634,8 +634,7 @@ static void srv_loop(Server *Sp)
         if (e == cudaSuccess)
             e = launch_blind_rotate(ctx->keys, I.d_ops, S.pool, I.d_idx, S.pool_rows, S.pool,
                                     I.d_idx + icap, S.pool_rows, S.big, count, kMu, ctx->status,
-                                    ctx->br_grid, S.st, S.pool, I.d_idx + 2 * icap,
-                                    S.pool_rows);
+                                    S.st, S.pool, I.d_idx + 2 * icap, S.pool_rows);
         if (e == cudaSuccess)
             e = launch_keyswitch(ctx->keys.ksk, S.big, S.pool, I.d_idx + 3 * icap, S.pool_rows,
                                  count, ctx->prm.n, ctx->num_sms, ctx->status, S.st,
@@ -739,7 +738,7 @@ int tfhe_serve_start(tfhe_ctx *ctx, size_t hbm_budget_bytes, size_t max_batch_ga
     Server *S = new Server();
     S->ctx = ctx;
     S->test_free_hbm = ctx->test_free_hbm;
-    S->max_batch = max_batch_gates ? (long)max_batch_gates : 8L * ctx->br_grid;
+    S->max_batch = max_batch_gates ? (long)max_batch_gates : 32L * ctx->num_sms;
     S->big_rows = S->max_batch;
     size_t fr = 0, total = 0;
     cudaError_t e = cudaMemGetInfo(&fr, &total);

@@ -152,7 +152,7 @@ extern "C" int tfhe_ctx_autotune(tfhe_ctx *ctx, const char *cache_path, int32_t 
                     e = cudaEventRecord(e0, st);
                 if (e == cudaSuccess)
                     e = launch_blind_rotate(K, nullptr, cts, nullptr, W, nullptr, nullptr, 0, big,
-                                            W, kMu, ctx->status, ctx->br_grid, st);
+                                            W, kMu, ctx->status, st);
                 if (e == cudaSuccess)
                     e = cudaEventRecord(e1, st);
                 if (e == cudaSuccess)
