@@ -766,6 +766,11 @@ def br_roofline(p, br_ms, br_launch, br_boot, step_ms_total, ks_ms, sm_count, sm
             "peak": peak_ops / 1e12, "unit": "Tops/s (int32)", "frac": achieved / peak_ops,
             "peak_basis": f"{sm_count} SMs x {INT32_LANES_PER_SM} INT32 "
                           f"lanes x {sm_max:.0f} MHz (max SM clock)",
+            # the operations are those of the algorithm, not of the kernel
+            "ops_basis": f"{OPS_PER_CMUX} algorithmic operations per CMux, unsigned butterflies "
+                         "at 7; the kernel runs a forward transform's first pass on the tensor "
+                         "pipe and its other butterflies in 4 instructions, so frac is a rate "
+                         "of algorithmic work and not the share of the pipe in use",
             "launches": br_launch, "bootstraps": br_boot,
             "avg_launch_ms": br_ms / max(br_launch, 1),
             "share_of_step": br_ms / max(step_ms_total, 1e-9),

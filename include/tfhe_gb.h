@@ -317,8 +317,8 @@ typedef enum {
     TFHE_OPT_SCHEDULE = 4,   /* tfhe_schedule policy of circuit schedules           */
     TFHE_OPT_LEVEL_WIDTH = 5,/* target gates per level for BALANCED (0: one wave    */
                              /*    of 4 bootstraps per SM, or one bootstrap per SM  */
-                             /*    where the autotuner's wave times make that       */
-                             /*    schedule cheaper)                                */
+                             /*    where that schedule costs less by the            */
+                             /*    autotuner's times, or, untuned, by fixed ones)   */
     TFHE_OPT_KS_KERNEL = 6,  /* key-switch kernel: 64 = tiled (64 gates per CTA, key */
                              /*    rows staged in shared memory by bulk copies),    */
                              /*    1, 2, 4, .. 32 = direct kernel with that j-split, */

@@ -385,8 +385,8 @@ class Context:
         self._c(lib().tfhe_ctx_set_option(self._h, option, int(value)))
 
     def autotune(self, cache_path=None) -> dict:
-        """Pick blind-rotation group sizes and key-switch j-splits per level
-        width by timing them on this device (results are unchanged)."""
+        """Pick blind-rotation shapes and key-switch kernels per level width by
+        timing them on this device (results are unchanged)."""
         ch = np.zeros(16, dtype=np.int32)
         self._c(lib().tfhe_ctx_autotune(self._h, cache_path.encode() if cache_path else None,
                                         ctypes.c_void_p(ch.ctypes.data)))

@@ -601,7 +601,7 @@ __device__ __forceinline__ void br_extract(const BrArgs &A, long g, const uint32
 // the twiddle as a Shoup product: 17 issue cycles per point (2 ffma, 3 imad
 // or shift-adds at 2, 1 add, Shoup 8) against 35 of an 80-butterfly pass and
 // its twiddle product.  The twiddles of both primes stay in TMEM beside the
-// accumulators (64 words per lane and sub-partition, read like them), so the
+// accumulators (128 words per lane, columns 384 on, read like them), so the
 // pass takes nothing from the load/store pipe but its result's transpose.
 constexpr int kTbCols = 96;                        // 32 outputs x 3 limbs of one prime
 constexpr uint32_t kTbOpBytes = kTbCols * 32 * 2;  // constant operand of one prime, 6 KB
@@ -747,7 +747,7 @@ __device__ __forceinline__ void pointwise_v(int32_t (&x)[32], const uint32_t (*f
     }
 }
 
-// Phase 4 (see crt_rows) of registers r0 .. r0 + NR - 1 on vector-ordered
+// Phase 4 (crt_lift) of registers r0 .. r0 + NR - 1 on vector-ordered
 // residue rows.
 template <int NR>
 __device__ __forceinline__ void crt_rows_v(uint32_t *acc, const uint32_t *x0, const uint32_t *x1,
@@ -1450,7 +1450,7 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_wide(const BrArgs A)
 // time (pair_drain).  (The flag tested at other places of the step: one gate 1.64 to
 // 1.67 ms, so 1.61.)
 // Bound: the chain of a step (6.3K cycles, the multiply pipe busy half of them,
-// seven barriers and two waits).  One gate 1.65 ms against 2.05 ms on one CTA;
+// seven barriers and two waits).  One gate 1.61 ms against 2.06 ms on one CTA;
 // the shape it replaces (8 warps per CTA, butterflies in the first pass, key
 // staged by bulk copies) took 2.53 ms.
 struct PairSmem {
@@ -1890,11 +1890,11 @@ static int br_group(long count, int num_sms, int forced, const int8_t *tuned)
 {
     if (br_shape_ok(forced))
         return forced;
-    // at most one bootstrap per SM: 2.09 ms on 16 warps (152 gates) against
-    // 3.27 ms for the throughput shape; 301 gates: 4.15 against 4.09 ms
+    // at most one bootstrap per SM: 2.03 ms on 16 warps (152 gates) against
+    // 2.75 ms for the throughput shape; 301 gates: 4.06 against 3.50 ms
     const int t = tuned[tune_bucket(count)];
     const int shape = br_shape_ok(t) ? t : count > num_sms ? 1 : kBrSplit;
-    // at most one per two SMs: 1.69 ms on two CTAs (76 gates) against 2.07 ms on
+    // at most one per two SMs: 1.60 ms on two CTAs (76 gates) against 2.03 ms on
     // one (a tuned choice stands for its bucket's widest level)
     return shape == kBrSplit && 2 * count <= num_sms ? kBrPair : shape;
 }
@@ -1973,8 +1973,8 @@ static cudaError_t launch_shape(const BrArgs &A, int shape, long nsm, int dev, c
 
 // Gates at the end of a level that leave at most one bootstrap per SM for its
 // last wave of the throughput shape: they run on the shapes of narrow levels
-// instead, behind it (a wave of one per SM takes 3.0 - 3.3 ms there, 1.7 - 2.1
-// ms on those; two per SM, 3.6 ms, would take two rounds).
+// instead, behind it (a wave of one per SM takes 2.6 - 2.75 ms there, 1.6 - 2.0
+// ms on those; two per SM, 3.5 ms, would take two rounds).
 static long br_tail(long count, long nsm, int forced, int shape)
 {
     const long tail = count % (4 * nsm);

@@ -635,7 +635,7 @@ struct CircuitCache {
     bool per_gate = false;
     bool profile = false;
     int policy = TFHE_SCHED_BALANCED;
-    long level_width = 0;            // 0: one wave, of 4 or 5 bootstraps per SM
+    long level_width = 0;            // 0: one wave, or one bootstrap per SM
     std::map<std::string, long> wave_choice;   // job signature -> chosen wave
     std::vector<Plan *> profiled;    // plans whose events hold the last run
     cudaStream_t capture_stream = nullptr;

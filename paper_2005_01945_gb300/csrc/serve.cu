@@ -343,8 +343,9 @@ struct Server {
 // Estimated device time (ms) of one serving iteration of n gates: the
 // autotuner's measured level time of n's width bucket while n fits one wave
 // of 4 bootstraps per SM, whole waves above.  Untuned (wave_ms 0) in units
-// of one wave, with the ratios measured on GB300: a level of at most one
-// bootstrap per SM takes 0.35 of a full wave, of at most two per SM 0.55.
+// of one wave, with fixed ratios: a level of at most one bootstrap per SM takes
+// 0.35 of a full wave, of at most two per SM 0.55 (the present kernels' are 0.38,
+// 0.30 up to one per two SMs, and 0.65).
 static double iter_cost(long n, int num_sms, const float *level_ms, float wave_ms)
 {
     const long w4 = 4L * num_sms;
