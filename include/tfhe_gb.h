@@ -340,14 +340,15 @@ typedef enum {
                              /*    the call sets status bit 2 (timeout), its outputs */
                              /*    are undefined, and the context stays usable     */
     TFHE_OPT_TEST_BR_STALL = 9 /* test hook for the blind rotation's timeout path, */
-                             /*    0 (default) off: k > 0 makes the wait for the   */
-                             /*    k-th tensor-pipe product of a bootstrap's slot  */
-                             /*    run out after about a second (shape 1; shape 8: */
-                             /*    the k-th CMux step's second product; shape 16:  */
-                             /*    the first product of the call's k-th gate, in   */
-                             /*    its second CTA, where an even number of steps   */
-                             /*    went before).  The kernel ends early and waits  */
-                             /*    for what is in flight; the rest is as for       */
+                             /*    0 (default) off: k > 0 makes the wait for a     */
+                             /*    tensor-pipe product run out after about a       */
+                             /*    second: in the k-th CMux step of each           */
+                             /*    bootstrap's slot (shape 1 its first product,    */
+                             /*    shape 8 its second), or (shape 16) the first of */
+                             /*    the call's k-th gate, in its second CTA, where  */
+                             /*    an even number of steps went before.  The       */
+                             /*    kernel ends early and waits for what is in      */
+                             /*    flight; the rest is as for                      */
                              /*    TFHE_OPT_TEST_KS_STALL                          */
 } tfhe_option;
 

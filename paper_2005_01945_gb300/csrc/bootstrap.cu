@@ -638,7 +638,6 @@ struct TbOps {                  // one CTA
     uint32_t tmem;
     volatile int abort[4];      // a wait of the bootstrap ran out (two-CTA shape: in this
                                 // step, from 1)
-    int skipped[4];             // ... and the step's second product was not issued
 };
 
 // Barrier of the 128 threads of bootstrap slot `bi`.
@@ -924,7 +923,6 @@ __device__ __forceinline__ void tb_setup(const BrArgs &A, TbOps &O, int tid, int
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(br_saddr(&O.spare[tid]))
                      : "memory");
         O.abort[tid] = 0;
-        O.skipped[tid] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -1046,11 +1044,8 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
             for (int ph = 0; ph < 2; ++ph) {
                 const Prime pq((uint32_t)ph);
                 uint32_t *sl = S.fwd[ph][wr];
-                const bool done = bk_wait(&O.bar[bi], phase & 1);
-                if (!done) {
+                if (!bk_wait(&O.bar[bi], phase & 1)) {
                     O.abort[bi] = 1;
-                    if (ph == 0 && tb == 0)
-                        O.skipped[bi] = 1;
                     atomicOr(A.status, kErrTimeout);
                 }
                 ++phase;
@@ -1059,14 +1054,13 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
                 tb_combine(tl + bi * kTbCols, tl + kTbTw + 64 * ph, sl + lane * kRowV, pq);
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 if (ph == 0) {
-                    // V_1 overwrites V_0 once the four warps have read it (and not
-                    // where the issuing thread's wait for V_0 ran out)
+                    // V_1 overwrites V_0 once the four warps have read it (where a
+                    // wait for V_0 ran out, too: both are waited for at the end)
                     if (wr == 0) {
                         asm volatile("bar.sync %0, 128;" ::"r"(5 + bi) : "memory");
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        if (lane == 0 && done)
-                            tb_mma(acc_cols, dig_op, O, 1,
-                                   phase + 1 == (uint32_t)A.keys.br_stall ? &O.spare[bi] : &O.bar[bi]);
+                        if (lane == 0)
+                            tb_mma(acc_cols, dig_op, O, 1, &O.bar[bi]);
                     } else {
                         asm volatile("bar.arrive %0, 128;" ::"r"(5 + bi) : "memory");
                     }
@@ -1096,14 +1090,12 @@ __global__ void __launch_bounds__(512, 1) k_blind_rotate_tc(const BrArgs A)
             br_extract<T>(A, g, S.acc, tb);
         boot_sync(bi);
     }
-    // after a wait that ran out: the last product issued, the only one that may
-    // still be in flight, gets a bounded time to finish before TMEM is freed
+    // after a wait that ran out: the step's two products get a bounded time to
+    // finish, in their order, before TMEM is freed (an even phase and an odd one; a
+    // wait for a phase that is not the barrier's current one would end at once)
     if (O.abort[bi] && tb == 0) {
-        const uint32_t last = phase - 1 - (uint32_t)O.skipped[bi];
-        if (last + 1 == (uint32_t)A.keys.br_stall)
-            (void)bk_wait(&O.spare[bi], 0);
-        else
-            (void)bk_wait(&O.bar[bi], last & 1);
+        (void)bk_wait(&O.bar[bi], phase & 1);
+        (void)bk_wait(&O.bar[bi], (phase + 1) & 1);
     }
     tb_release(tmem, warp);
 }
@@ -1910,7 +1902,10 @@ static cudaError_t launch_tc(const BrArgs &A, unsigned blocks, int dev, cudaStre
             return e;
         prepared[dev] = 1;
     }
-    k_blind_rotate_tc<<<blocks, 512, smem, stream>>>(A);
+    BrArgs B = A;
+    if (B.keys.br_stall)   // test hook: of the step's two products the first
+        B.keys.br_stall = 2 * B.keys.br_stall - 1;
+    k_blind_rotate_tc<<<blocks, 512, smem, stream>>>(B);
     return cudaGetLastError();
 }
 

@@ -1345,8 +1345,8 @@ int tfhe_ctx_set_option(tfhe_ctx *ctx, int option, int64_t value)
         invalidate_graphs(ctx);
         return TFHE_OK;
     case TFHE_OPT_TEST_BR_STALL:
-        if (value < 0 || value > INT32_MAX)
-            return fail(ctx, TFHE_EINVAL, "TFHE_OPT_TEST_BR_STALL must be >= 0");
+        if (value < 0 || value > 1 << 20)
+            return fail(ctx, TFHE_EINVAL, "TFHE_OPT_TEST_BR_STALL must be 0 .. 1048576");
         ctx->keys.br_stall = (int)value;
         invalidate_graphs(ctx);
         return TFHE_OK;

@@ -117,7 +117,7 @@ struct DevKeys {
     int ks_stall;          // test hook (TFHE_OPT_TEST_KS_STALL): the stage waits
                            // of the tiled and tensor key switch run out
     int br_stall;          // test hook (TFHE_OPT_TEST_BR_STALL): the wait for this
-                           // product of a bootstrap's slot (from 1) runs out
+                           // product, step or gate (by shape; from 1) runs out
     // Autotuned launch shapes per level-width bucket (0 = not tuned): bucket b
     // covers widths up to kTuneEdge[b] (the last bucket is unbounded).
     int8_t tune_br[8];     // blind-rotation shape

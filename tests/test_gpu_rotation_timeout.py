@@ -30,14 +30,14 @@ def gpu(orc):
     ctx.close()
 
 
-# shape 1: the first and the second product of a step, of the first step and of a
-# later one; 700 gates: two gates per slot.  Shape 16: a product of a gate's second
-# CTA, so that the first one's wait for residues runs out two steps later; of a gate
-# with one step, behind which the first CTA ends by itself; of a cluster's second gate
-@pytest.mark.parametrize("shape,count,products", [(1, 3, (1, 2, 5, 6)), (1, 700, (1, 2, 47, 60)),
-                                                  (8, 3, (1, 2, 20)), (8, 200, (1, 30)),
-                                                  (16, 3, (1, 2, 3)), (16, 100, (1, 3, 77, 100))])
-def test_timeout_is_reported_and_recoverable(gpu, orc, shape, count, products):
+# Shapes 1 and 8: the first step and later ones; 700 and 200 gates: two gates per slot.
+# Shape 16: a product of a gate's second CTA, so that the first one's wait for residues
+# runs out two steps later; of a gate with one step, behind which the first CTA ends by
+# itself; of a cluster's second gate
+@pytest.mark.parametrize("shape,count,where", [(1, 3, (1, 2, 24)), (1, 700, (1, 24, 25, 30)),
+                                               (8, 3, (1, 2, 20)), (8, 200, (1, 30)),
+                                               (16, 3, (1, 2, 3)), (16, 100, (1, 3, 77, 100))])
+def test_timeout_is_reported_and_recoverable(gpu, orc, shape, count, where):
     torch, api, p, P, ctx = gpu["torch"], gpu["api"], gpu["p"], gpu["P"], gpu["ctx"]
     g = synth._gen(37, f"stall{shape}{count}")
     cts = g.integers(0, 1 << 32, size=(count, 512), dtype=np.uint64).astype(np.uint32)
@@ -49,7 +49,7 @@ def test_timeout_is_reported_and_recoverable(gpu, orc, shape, count, products):
     dev = api.to_device(cts)
     ctx.set_option(api.OPT_BR_GROUP, shape)
     try:
-        for k in products:
+        for k in where:
             out = torch.zeros((count, 512), dtype=torch.int32, device="cuda")
             ctx.set_option(api.OPT_TEST_BR_STALL, k)
             ctx.bootstrap(dev, out, mu=1 << 29)
