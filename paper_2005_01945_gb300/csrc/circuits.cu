@@ -1102,9 +1102,11 @@ static int run_plan(tfhe_ctx *ctx, Plan &P, const tfhe_job *jobs, cudaStream_t s
 // ceil(w / wave) wave times above, and the narrow unit is used once it is at
 // least 1 % cheaper.  Decided once per job mix.  Without autotuner measurements
 // the times are the ones below, and only a mix of at most two bootstraps per SM
-// and level on average is costed (a wider one's narrow schedule costs more, and
-// building it takes as long as the schedule itself): one 32-bit Dadda product
-// ran 22 levels of up to 528 gates in 48.1 ms and runs them at 152 in 41.3.
+// and level on average is costed: a wider one's narrow schedule rarely costs less
+// (5 of 127 mixes by these times, 1 to 5 %), and building it takes as long as the
+// schedule itself.  A forced shape's times order the two schedules the same way
+// (no mix of several hundred costs more at 152 by them).  One 32-bit Dadda product
+// ran 22 levels of up to 528 gates in 48.1 ms and runs them at 152 in 41.0.
 constexpr float kLevelMs[3] = {2.10f, 3.66f, 5.43f};   // levels of 1, 2 and 4 per SM
 constexpr float kPairShare = 0.79f;                    // of a level of one per two SMs
 
